@@ -181,7 +181,7 @@ struct Smem {
     int trBase;       // first trail slot of the CTA's block
 };
 
-enum { kCntLive = 0, kCntLiveIn, kCntWords, kCntTrail, kCntHits, kCntLocal, kCntMiss, kCntPruned, kCntWin, kCntTuples };
+enum { kCntLive = 0, kCntLiveIn, kCntWords, kCntTrail, kCntHits, kCntLocal, kCntMiss, kCntPruned, kCntWin, kCntTuples, kCntHard };
 
 // ---------------------------------------------------------------------------
 // plan: Algorithm 1 lines 1-3 and the row selection of Algorithm 2.
@@ -212,33 +212,97 @@ __device__ void plan(const TableDev& T, const VarLayout& V, const uint32_t* __re
     if (tid < 8) sm.flags[tid] = 0;
     __syncthreads();
     CT_STAMP(16);
-    for (int i = tid; i < T.arity; i += kThreads) {
-        const int nw = V.nw(i);
-        const uint32_t* d = dom + V.off(i);
-        const uint32_t* l = T.lastDom + V.ld(i);
-        int nd = 0, ndel = 0;
-        uint32_t grow = 0u;
-        for (int q = 0; q < nw; ++q) {
-            const uint32_t dv = d[q], lv = l[q];
-            grow |= dv & ~lv;
-            nd += __popc(dv);
-            ndel += __popc(lv & ~dv);
-            if (domCopy) domCopy[V.ld(i) + q] = dv;
-            for (int lv0 = snapFrom; lv0 < snapTo; ++lv0) T.levelDom[(size_t)lv0 * T.DW + V.ld(i) + q] = lv;
+    // 2^lg adjacent lanes share a variable, a lane per domain word (a wide
+    // domain's words in turns), and add their counts by shuffles; the words of
+    // kAhead rounds of variables are loaded before the first is used. Domains of
+    // one or two words (lg = 0): a thread per variable, less code to fetch
+    // (measured 0.2 us faster per call on six variables of one word; at 100
+    // variables of 16 words the lanes take the plan from 19.4 to 13.4 us).
+    const int lg = T.wordLanesLog, gl = 1 << lg, sub = tid & (gl - 1), grp = tid >> lg, ngrp = kThreads >> lg;
+    if (lg == 0) {
+        for (int i = tid; i < T.arity; i += kThreads) {
+            const int nw = V.nw(i);
+            const uint32_t* d = dom + V.off(i);
+            const uint32_t* l = T.lastDom + V.ld(i);
+            int nd = 0, ndel = 0;
+            uint32_t grow = 0u;
+            for (int q = 0; q < nw; ++q) {
+                const uint32_t dv = d[q], lv = l[q];
+                grow |= dv & ~lv;
+                nd += __popc(dv);
+                ndel += __popc(lv & ~dv);
+                if (domCopy) domCopy[V.ld(i) + q] = dv;
+                for (int lv0 = snapFrom; lv0 < snapTo; ++lv0) T.levelDom[(size_t)lv0 * T.DW + V.ld(i) + q] = lv;
+            }
+            sup[i] = nd > 1;
+            if (i < kLocalMaxArity) sm.nd[i] = nd;
+            if (grow) atomicExch(&sm.flags[0], 1);
+            if (nd == 0) atomicExch(&sm.flags[1], 1);
+            if (nd > 1) atomicAdd(&sm.flags[5], 1);
+            int k = 0;
+            if (ndel > 0) {
+                // Algorithm 2, line 3: the delta mask when |Delta| < |dom| (strict).
+                if (ndel < nd) { k = ndel | kCodeDelta; atomicAdd(&sm.flags[3], 1); }
+                else { k = nd; atomicAdd(&sm.flags[4], 1); }
+                atomicAdd(&sm.flags[2], 1);
+            }
+            K[i] = k;
         }
-        sup[i] = nd > 1;
-        if (i < kLocalMaxArity) sm.nd[i] = nd;
-        if (grow) atomicExch(&sm.flags[0], 1);
-        if (nd == 0) atomicExch(&sm.flags[1], 1);
-        if (nd > 1) atomicAdd(&sm.flags[5], 1);
-        int k = 0;
-        if (ndel > 0) {
-            // Algorithm 2, line 3: the delta mask when |Delta| < |dom| (strict).
-            if (ndel < nd) { k = ndel | kCodeDelta; atomicAdd(&sm.flags[3], 1); }
-            else { k = nd; atomicAdd(&sm.flags[4], 1); }
-            atomicAdd(&sm.flags[2], 1);
+    } else {
+        constexpr int kAhead = 4;
+        for (int b0 = 0; b0 < T.arity; b0 += kAhead * ngrp) {
+            uint32_t dv[kAhead], lv[kAhead];
+            int nwv[kAhead];
+    #pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int i = b0 + u * ngrp + grp;
+                nwv[u] = 0;
+                dv[u] = lv[u] = 0u;
+                if (i < T.arity) {
+                    nwv[u] = V.nw(i);
+                    if (sub < nwv[u]) {
+                        dv[u] = dom[V.off(i) + sub];
+                        lv[u] = T.lastDom[V.ld(i) + sub];
+                    }
+                }
+            }
+    #pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                if (b0 + u * ngrp >= T.arity) break;  // the same for every thread
+                const int i = b0 + u * ngrp + grp;
+                int nd = 0, ndel = 0;
+                uint32_t grow = 0u;
+                for (int q = sub; q < nwv[u]; q += gl) {
+                    if (q != sub) {
+                        dv[u] = dom[V.off(i) + q];
+                        lv[u] = T.lastDom[V.ld(i) + q];
+                    }
+                    grow |= dv[u] & ~lv[u];
+                    nd += __popc(dv[u]);
+                    ndel += __popc(lv[u] & ~dv[u]);
+                    if (domCopy) domCopy[V.ld(i) + q] = dv[u];
+                    for (int v = snapFrom; v < snapTo; ++v) T.levelDom[(size_t)v * T.DW + V.ld(i) + q] = lv[u];
+                }
+                for (int o = gl >> 1; o > 0; o >>= 1) {
+                    nd += __shfl_xor_sync(0xffffffffu, nd, o);
+                    ndel += __shfl_xor_sync(0xffffffffu, ndel, o);
+                }
+                if (grow) atomicExch(&sm.flags[0], 1);
+                if (i >= T.arity || sub != 0) continue;
+                sup[i] = nd > 1;
+                if (i < kLocalMaxArity) sm.nd[i] = nd;
+                if (nd == 0) atomicExch(&sm.flags[1], 1);
+                if (nd > 1) atomicAdd(&sm.flags[5], 1);
+                int k = 0;
+                if (ndel > 0) {
+                    // Algorithm 2, line 3: the delta mask when |Delta| < |dom| (strict).
+                    if (ndel < nd) { k = ndel | kCodeDelta; atomicAdd(&sm.flags[3], 1); }
+                    else { k = nd; atomicAdd(&sm.flags[4], 1); }
+                    atomicAdd(&sm.flags[2], 1);
+                }
+                K[i] = k;
+            }
         }
-        K[i] = k;
     }
     __syncthreads();
     CT_STAMP(17);
@@ -283,26 +347,65 @@ __device__ void plan(const TableDev& T, const VarLayout& V, const uint32_t* __re
         __syncthreads();
     }
     CT_STAMP(18);
-    // Codes: the removed values (delta) or the remaining ones (reset).
-    for (int i = tid; i < T.arity; i += kThreads) {
-        const int k = K[i] & kCodeRow;
-        if (k == 0) continue;
-        const bool delta = (K[i] & kCodeDelta) != 0;
-        const int nw = V.nw(i);
-        const uint32_t* d = dom + V.off(i);
-        const uint32_t* l = T.lastDom + V.ld(i);
-        const int row0 = V.row0(i);
-        int out = rowOff[i];
-        const int last = out + k - 1;
-        for (int q = 0; q < nw; ++q) {
-            uint32_t bits = delta ? (l[q] & ~d[q]) : d[q];
-            while (bits) {
-                const int b = __ffs(bits) - 1;
-                bits &= bits - 1u;
-                int code = row0 + q * 32 + b;
-                if (delta) code |= kCodeDelta;
-                if (out == last) code |= kCodeLast;
-                codes[out++] = code;
+    // Codes: the removed values (delta) or the remaining ones (reset), a
+    // variable's words over its lanes again.
+    if (lg == 0) {
+        for (int i = tid; i < T.arity; i += kThreads) {
+            const int k = K[i] & kCodeRow;
+            if (k == 0) continue;
+            const bool delta = (K[i] & kCodeDelta) != 0;
+            const int nw = V.nw(i);
+            const uint32_t* d = dom + V.off(i);
+            const uint32_t* l = T.lastDom + V.ld(i);
+            const int row0 = V.row0(i);
+            int out = rowOff[i];
+            const int last = out + k - 1;
+            for (int q = 0; q < nw; ++q) {
+                uint32_t bits = delta ? (l[q] & ~d[q]) : d[q];
+                while (bits) {
+                    const int b = __ffs(bits) - 1;
+                    bits &= bits - 1u;
+                    int code = row0 + q * 32 + b;
+                    if (delta) code |= kCodeDelta;
+                    if (out == last) code |= kCodeLast;
+                    codes[out++] = code;
+                }
+            }
+        }
+    } else {
+        for (int b0 = 0; b0 < T.arity; b0 += ngrp) {
+            const int i = b0 + grp;
+            const int ki = i < T.arity ? K[i] : 0;
+            const int k = ki & kCodeRow;
+            if (!__any_sync(0xffffffffu, k != 0)) continue;
+            const bool delta = (ki & kCodeDelta) != 0;
+            const int nw = k ? V.nw(i) : 0;
+            const int nwMax = lg < 5 ? gl : max(gl, __reduce_max_sync(0xffffffffu, nw));
+            int out = k ? rowOff[i] : 0;
+            const int last = out + k - 1;
+            for (int q0 = 0; q0 < nwMax; q0 += gl) {
+                const int q = q0 + sub;
+                uint32_t bits = 0u;
+                if (q < nw) {
+                    const uint32_t d = dom[V.off(i) + q];
+                    bits = delta ? (T.lastDom[V.ld(i) + q] & ~d) : d;
+                }
+                const int c = __popc(bits);
+                int inc = c;
+                for (int o = 1; o < gl; o <<= 1) {
+                    const int a = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (sub >= o) inc += a;
+                }
+                int at = out + inc - c;
+                while (bits) {
+                    const int b = __ffs(bits) - 1;
+                    bits &= bits - 1u;
+                    int code = V.row0(i) + q * 32 + b;
+                    if (delta) code |= kCodeDelta;
+                    if (at == last) code |= kCodeLast;
+                    codes[at++] = code;
+                }
+                out += __shfl_sync(0xffffffffu, inc, (tid & 31) | (gl - 1));
             }
         }
     }
@@ -660,13 +763,16 @@ __device__ __forceinline__ int probe_windows(const TableDev& T, int r, int res, 
     bool complete = false;
     if (!kLive && T.useResidues) {
         // the chunks that follow the residue, dead or alive: two windows per
-        // round of loads, tested in order
+        // round of loads, tested in order; a table of at most kProbes windows
+        // is covered by them, and a value they miss has no support
         const int W4 = T.W4;
+        complete = W4 <= 32 * kProbes;
         const uint4* row = T.sup + (size_t)r * W4;
         // (one window per round when the chunks are recomputed from more than
         // four rows: their row loads)
         constexpr int kStep = kE > 4 ? 1 : 2;
         for (int b = 0; b < kProbes; b += kStep) {
+            if (complete && b * 32 >= W4) break;
             const int c0 = (int)(((long long)res + 1 + b * 32 + lane) % W4);
             const int c1 = (int)(((long long)res + 1 + (b + 1) * 32 + lane) % W4);
             const bool two = kStep == 2 && b + 1 < kProbes;
@@ -763,26 +869,80 @@ __device__ __forceinline__ int probe_windows(const TableDev& T, int r, int res, 
     return complete ? kProbeGone : kProbeUndecided;
 }
 
-// A residue miss searched by probe_windows; a value not found goes to the
-// hard list, marked kNoSupport when it has no support (removed without a
-// scan; a scan keeps the mark, atomicMin), else for the full scan.
-__device__ __forceinline__ void note_probe(const TableDev& T, int r, int o, uint32_t* s_cnt) {
-    if (o != kProbeFound && (threadIdx.x & 31) == 0) {
-        const bool complete = o == kProbeGone;
-        const unsigned m = atomicAdd(&T.ctrl->nhard, 1u);
-        T.hardRow[m] = r;
-        T.foundChunk[m] = complete ? kNoSupport : kNoChunk;
-        if (!complete) {
-            atomicAdd(&T.ctrl->nscan, 1);
-            atomicAdd(&s_cnt[kCntMiss], 1u);
-        }
+// The outcome of a residue miss's search (one thread per value): an unsupported value (bit `bit` of packed domain word `word`) is
+// marked removed, an undecided one goes to the hard list for the full scan.
+__device__ __forceinline__ void note_probe(const TableDev& T, int r, int word, int bit, int o, uint32_t* s_cnt) {
+    if (o == kProbeFound) return;
+    atomicAdd(&s_cnt[kCntHard], 1u);
+    if (o == kProbeGone) {
+        atomicOr(&T.removed[word], 1u << bit);
+        return;
     }
+    const int m = atomicAdd(&T.ctrl->nscan, 1);
+    T.hardRow[m] = r;
+    T.foundChunk[m] = kNoChunk;
+    atomicAdd(&s_cnt[kCntMiss], 1u);
 }
 
 template <bool kLive, int kProbes = kLocalProbes, int kE = 0>
-__device__ __forceinline__ void probe_miss(const TableDev& T, int r, int res, uint32_t* s_cnt,
+__device__ __forceinline__ void probe_miss(const TableDev& T, int r, int word, int bit, int res, uint32_t* s_cnt,
                                            const int32_t* codes = nullptr, int nrows = 0) {
-    note_probe(T, r, probe_windows<kLive, kProbes, kE>(T, r, res, s_cnt, codes, nrows), s_cnt);
+    const int o = probe_windows<kLive, kProbes, kE>(T, r, res, s_cnt, codes, nrows);
+    if ((threadIdx.x & 31) == 0) note_probe(T, r, word, bit, o, s_cnt);
+}
+
+// Residue misses of a warp (lanes `miss`, each holding its value r and residue
+// res) searched over the chunks that follow the residues, dead or alive, K
+// values at a time so that K rows' loads are in flight (after the update's
+// barrier only). Returns the lane's own outcome.
+template <int K>
+__device__ __forceinline__ int probe_dense_lanes(const TableDev& T, unsigned miss, int r, int res, uint32_t* s_cnt) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int W4 = T.W4;
+    const int nwin = min(kLocalProbes, (W4 + 31) >> 5);
+    int mine = nwin * 32 >= W4 ? kProbeGone : kProbeUndecided;
+    while (miss) {
+        int ln[K], c[K];
+        const uint4* row[K];
+        unsigned open = 0u;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            ln[k] = miss ? __ffs(miss) - 1 : 0;
+            if (miss) open |= 1u << k;
+            miss &= miss - 1u;
+            row[k] = T.sup + (size_t)__shfl_sync(FULL, r, ln[k]) * W4;
+            c[k] = (int)(((long long)__shfl_sync(FULL, res, ln[k]) + 1 + lane) % W4);
+        }
+        for (int b = 0; b < nwin && open; ++b) {
+            if (lane == 0) atomicAdd(&s_cnt[kCntWin], (uint32_t)__popc(open));
+            uint4 s[K], t[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                if ((open >> k) & 1u) {
+                    s[k] = ld_sup(row[k] + c[k]);
+                    t[k] = __ldcg(T.curr + c[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                if (!((open >> k) & 1u)) continue;
+                const unsigned bal = __ballot_sync(FULL, nz(and4(s[k], t[k])));
+                if (bal) {
+                    const int cf = __shfl_sync(FULL, c[k], __ffs(bal) - 1);
+                    if (lane == ln[k]) {
+                        T.residue[r] = cf;
+                        mine = kProbeFound;
+                        atomicAdd(&s_cnt[kCntLocal], 1u);
+                    }
+                    open &= ~(1u << k);
+                }
+                c[k] += 32;
+                if (c[k] >= W4) c[k] %= W4;
+            }
+        }
+    }
+    return mine;
 }
 
 // Whole warp: wait (bounded) until every CTA of the launch has released its
@@ -807,27 +967,13 @@ __device__ __forceinline__ bool wait_update_done(Ctrl* C, unsigned limit) {
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-template <bool kLive>
-__device__ __forceinline__ void probe_row(const TableDev& T, int r, bool present, int res, uint4 supRes,
-                                          uint32_t* s_cnt) {
-    const int lane = threadIdx.x & 31;
-    if (!present) return;
-    if (T.useResidues) {
-        bool hit = false;
-        if (lane == 0) hit = nz(and4(supRes, __ldcg(T.curr + res)));
-        if (__shfl_sync(0xffffffffu, hit, 0)) {
-            if (lane == 0) atomicAdd(&s_cnt[kCntHits], 1u);
-            return;
-        }
-    }
-    probe_miss<kLive>(T, r, res, s_cnt);
-}
-
 // ---------------------------------------------------------------------------
 // scan: the hard values against the live chunks of one segment
 // ---------------------------------------------------------------------------
+// (entries [ma, mb) of the hard list; the list of one segment may be cut over
+// several warps)
 template <int U, bool kGlobal = false>
-__device__ __forceinline__ void scan_segment(const TableDev& T, int seg, int nh, const int32_t* s_rows) {
+__device__ __forceinline__ void scan_segment(const TableDev& T, int seg, int ma, int mb, const int32_t* s_rows) {
     const int lane = threadIdx.x & 31;
     const uint32_t mask = __ldcg(&T.segMask[seg]);
     if (mask == 0u) return;
@@ -835,20 +981,20 @@ __device__ __forceinline__ void scan_segment(const TableDev& T, int seg, int nh,
     const int w = seg * 32 + lane;
     const uint4 cur = act ? __ldcg(T.curr + w) : make_uint4(0u, 0u, 0u, 0u);
     const size_t W4 = (size_t)T.W4;
-    for (int m0 = 0; m0 < nh; m0 += U) {
+    for (int m0 = ma; m0 < mb; m0 += U) {
         bool hit[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int mm = m0 + u;
             hit[u] = false;
-            if (act && mm < nh) {
+            if (act && mm < mb) {
                 const int r = (!kGlobal && mm < kCodeCap) ? s_rows[mm] : __ldcg(&T.hardRow[mm]);
                 hit[u] = nz(and4(ld_sup(T.sup + (size_t)r * W4 + w), cur));
             }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (m0 + u < nh) {
+            if (m0 + u < mb) {
                 // any supporting chunk is a valid new residue: whichever
                 // segment's store lands last stays (a plain store: no
                 // round trip and no contended atomic per value)
@@ -859,9 +1005,18 @@ __device__ __forceinline__ void scan_segment(const TableDev& T, int seg, int nh,
     }
 }
 
-// Negative tables: the valid tuples carrying each hard value, summed over the
-// live chunks of one segment (foundChunk[m] holds the count).
-__device__ __forceinline__ void count_segment(const TableDev& T, int seg, int nh, const int32_t* s_rows) {
+// a * b, saturated at 2^62 (negative tables: products of domain sizes). The
+// high half decides the overflow: a 64-bit division per factor took 3 us of a
+// four-variable plan.
+__device__ __forceinline__ unsigned long long sat_mul(unsigned long long a, unsigned long long b) {
+    const unsigned long long cap = 1ull << 62, lo = a * b;
+    return (__umul64hi(a, b) != 0ull || lo > cap) ? cap : lo;
+}
+
+// Negative tables: the valid tuples carrying each hard value of [ma, mb),
+// summed over the live chunks of one segment (foundChunk[m] holds the count),
+// four rows' loads in flight.
+__device__ __forceinline__ void count_segment(const TableDev& T, int seg, int ma, int mb, const int32_t* s_rows) {
     const int lane = threadIdx.x & 31;
     const uint32_t mask = __ldcg(&T.segMask[seg]);
     if (mask == 0u) return;
@@ -869,16 +1024,24 @@ __device__ __forceinline__ void count_segment(const TableDev& T, int seg, int nh
     const int w = seg * 32 + lane;
     const uint4 cur = act ? __ldcg(T.curr + w) : make_uint4(0u, 0u, 0u, 0u);
     const size_t W4 = (size_t)T.W4;
-    for (int m = 0; m < nh; ++m) {
-        const int r = m < kCodeCap && s_rows ? s_rows[m] : __ldcg(&T.hardRow[m]);
-        uint32_t c = 0u;
-        if (act) {
-            const uint4 v = and4(ld_sup(T.sup + (size_t)r * W4 + w), cur);
-            c = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+    constexpr int U = 4;
+    for (int m0 = ma; m0 < mb; m0 += U) {
+        uint32_t c[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int m = m0 + u;
+            c[u] = 0u;
+            if (act && m < mb) {
+                const int r = m < kCodeCap && s_rows ? s_rows[m] : __ldcg(&T.hardRow[m]);
+                const uint4 v = and4(ld_sup(T.sup + (size_t)r * W4 + w), cur);
+                c[u] = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+            }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-        if (lane == 0 && c) atomicAdd(&T.foundChunk[m], (int)c);
+        for (int u = 0; u < U; ++u) {
+            const uint32_t sum = __reduce_add_sync(0xffffffffu, c[u]);
+            if (lane == 0 && sum) atomicAdd(&T.foundChunk[m0 + u], (int)sum);
+        }
     }
 }
 

@@ -32,7 +32,6 @@ constexpr int kLocalMaxArity = 512;    // every CTA plans for itself up to this 
 constexpr int kLocalMaxDW = 2048;      // this many domain words and kCodeCap rows
 constexpr int kStatusHdr = 24;         // int32 slots before the changed mask
 constexpr int32_t kNoChunk = 0x7fffffff;
-constexpr int32_t kNoSupport = -2;         // hard-list mark: no live chunk supports the value (no scan needed)
 // Row code of the update plan: supports row | flags.
 constexpr int32_t kCodeLast = 1 << 30;   // last row of its variable: apply the mask
 constexpr int32_t kCodeDelta = 1 << 29;  // variable on the delta path: mask = ~OR(rows)
@@ -83,13 +82,14 @@ struct Ctrl {
     uint32_t live;       // per call: chunks alive after updateTable
     uint32_t live_in;    // per call: chunks live at entry
     uint32_t words_in;   // per call: non-zero 32-bit words at entry
-    uint32_t nhard;      // per call: values left for the full index scan
+    uint32_t nhard;      // per call: values neither their residue nor the windows support
     uint32_t done;       // last-block-done ticket
     int32_t nrows;       // rows in the update plan
     int32_t nval, ndelta, nreset, nsup;
     int32_t hits, pruned, trail_added, local_found, misses, windows;
     int32_t live_state;  // live chunks after the last update (kept across calls)
-    int32_t nscan;       // per call: hard values that need the full scan (the others are known unsupported)
+    int32_t nscan;       // per call: hard values that need the full scan, listed in hardRow (the others
+                         // are known unsupported; the network kernel lists all hard values)
     uint32_t tuples;     // per call, negative tables: valid tuples after the update
     uint32_t upd_done;   // per call: CTAs done with the update (a filter beside it may wait on it)
     uint64_t t[4];       // %globaltimer stamps of CTA 0 (diagnostics)
@@ -120,6 +120,7 @@ struct TableDev {
                                 // other scope domains' sizes (saturated), written by the plan
     int32_t* hardRow;        // [R] values left for the full scan
     int32_t* foundChunk;     // [R]
+    uint32_t* removed;       // [DW] one-table kernel: values found unsupported by the call's probes (zero between calls)
     const int32_t* rowVar;   // [R] scope position of each row
     const int32_t* varRow0;  // [arity+1] first row of each variable (_supportJmp)
     const int32_t* varNW;    // [arity] words of each domain
@@ -131,6 +132,8 @@ struct TableDev {
     int32_t negative;        // 1: the tuples are forbidden (negative table)
     int32_t shard;           // 1: a word-range shard (one-table kernel only): no failure on an
                              // empty currTable, lastDom keeps the call's input domains
+    int32_t wordLanesLog;    // log2 of the lanes that share one variable's domain words (the widest domain's
+                             // words rounded up to a power of two, at most a warp; 0 up to two words)
     int32_t warpPlan;        // 1: the network kernel plans it with one warp (positive, arity
                              // <= 32, every domain <= kWarpPlanWords words)
     // Scopes of at most kParamArity variables: words, lastDom offset and first

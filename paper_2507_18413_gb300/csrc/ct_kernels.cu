@@ -18,18 +18,20 @@
 //            segment's live mask (the non-zero index) is rebuilt with one warp
 //            ballot.
 //   -- grid barrier --
-//   probe    Algorithm 1 line 5 (fail when currTable = 0), then one warp per
-//            value of s_sup (Algorithm 3 with residues): the residue chunk
-//            first (loaded beside the failure test); on a miss, up to four
-//            32-chunk windows after it; values still unresolved go to the
-//            hard list.
+//   probe    Algorithm 1 line 5 (fail when currTable = 0), then the values of
+//            s_sup (Algorithm 3 with residues), one per lane of a warp: the
+//            residue chunk first (loaded beside the failure test); on a miss,
+//            the warp searches up to four 32-chunk windows after it. A value
+//            its windows show to have no support is marked in a bitset of the
+//            domains' layout, one they leave undecided goes to the hard list.
 //   -- grid barrier --
-//   publish  with no hard value, the CTA that arrived last at the barrier
-//            writes lastDom's removals, the status block (mapped host memory)
-//            and resets the per-call counters; otherwise every warp holds a
-//            segment's live chunks and tests every hard value against them,
-//            and the last CTA to finish removes the values no chunk supports,
-//            stores new residues and publishes.
+//   publish  with no undecided value, the CTA that arrived last at the barrier
+//            takes the marked values off the domains, writes lastDom and the
+//            status block (mapped host memory) and resets the per-call
+//            counters; otherwise (segment, slice of the hard list) units are
+//            spread over the grid's warps, each holding a segment's live
+//            chunks and testing the slice's values against them, and the last
+//            CTA to finish decides them, stores new residues and publishes.
 // Calls of at most U supports rows (positive local-plan tables with
 // residues, at least half the chunks live at entry; ct_options.no_early_filter
 // switches this off) run the probes
@@ -83,34 +85,36 @@ static_assert(kSlotStatus == 0 && kSlotLiveOut == 1 && kSlotWordsIn == 2 && kSlo
 // to arrive at the final barrier, or the last to finish the full scan). Every
 // counter of the call is read in one round of loads (thread k reads header
 // slot k); t3 is the caller's stamp of the end of the probes (0: read it from
-// the control block).
-// nh < 0: the hard-value counts are read with the header, and with values
-// left undecided for the full scan the CTA returns false without publishing
-// (the hard values known unsupported are removed here).
-// Nothing but this CTA writes the domains during a call, so the first hard
-// entries (read whether or not they belong to this call, kept only below the
-// count) and the domain words are loaded in the same round as the header;
-// the removals go to a shared copy of the domains, which is what the host
-// receives. localDom: sm.dom already holds the call's domains (local plan).
-// lastDomHere: the filter ran beside the update, so no CTA wrote lastDom
-// after the plans (a CTA may still be reading it in its plan before the
-// barrier): this CTA writes it, the call's domains less the values it removes.
+// the control block). nh: the hard list's length after a full scan, which
+// decides its values here; 0 with none; < 0: not known yet, and with values
+// left for a full scan the CTA returns false without publishing.
+// The values the probes found unsupported are bits of T.removed, loaded in the
+// same round as the header (and, in the global plan, as the domain words); a
+// removal is a bit there too, so the work is per domain word, not per value,
+// with 2^wordLanesLog adjacent lanes on one variable's words. localDom: sm.dom
+// already holds the call's domains (local plan). early: the filter ran beside
+// the update (reported in the header; the failure is decided here).
+// Nobody else writes the domains or lastDom during a call: both are written
+// here, on CT_OK only.
 __device__ bool finalize(const TableDev& T, const VarLayout& V, uint32_t* __restrict__ dom, Smem& sm, int nh,
-                         uint64_t t3, bool localDom, bool lastDomHere = false) {
+                         uint64_t t3, bool localDom, bool early = false) {
     Ctrl* C = T.ctrl;
     const int tid = threadIdx.x;
     int32_t* H = T.statusBlk;
     __syncthreads();  // counters thread 0 of this CTA may have written just before
     const bool smemDom = localDom || T.DW <= kLocalMaxDW;
+    uint32_t* rm = smemDom ? reinterpret_cast<uint32_t*>(sm.codes) : T.removed;  // (sm.codes is free by now)
+    const int lg = T.wordLanesLog, gl = 1 << lg, sub = tid & (gl - 1), ngrp = kThreads >> lg;
     int preRow = 0, preFc = 0;
-    if (nh != 0) {
-        if (tid < T.R) {
-            preRow = __ldcg(&T.hardRow[tid]);
-            preFc = __ldcg(&T.foundChunk[tid]);
-        }
-        if (!localDom && smemDom)
-            for (int i = tid; i < T.arity; i += kThreads)
-                for (int k = 0; k < V.nw(i); ++k) sm.dom[V.ld(i) + k] = __ldcg(&dom[V.off(i) + k]);
+    if (tid < nh) {
+        preRow = __ldcg(&T.hardRow[tid]);
+        preFc = __ldcg(&T.foundChunk[tid]);
+    }
+    const uint32_t preRm = tid < T.DW ? __ldcg(&T.removed[tid]) : 0u;  // used only if the call has hard values
+    if (!localDom && smemDom) {
+#pragma unroll 4
+        for (int i = tid >> lg; i < T.arity; i += ngrp)
+            for (int q = sub; q < V.nw(i); q += gl) sm.dom[V.ld(i) + q] = __ldcg(&dom[V.off(i) + q]);
     }
     if (tid < kStatusHdr) {
         // one predicated load (two for a stamp difference) per slot, no
@@ -119,9 +123,8 @@ __device__ bool finalize(const TableDev& T, const VarLayout& V, uint32_t* __rest
         const int a = kHdrWord[tid], b = kHdrSub[tid];
         int32_t v = a >= 0 ? __ldcg(cw + a) : 0;
         const int32_t w = b >= 0 ? __ldcg(cw + b) : 0;
-        if (tid == kSlotHard && nh >= 0) v = nh;
         if (tid == kSlotT3 && t3) v = (int32_t)(uint32_t)t3;
-        if (tid == kSlotEarly) v = lastDomHere ? 1 : 0;
+        if (tid == kSlotEarly) v = early ? 1 : 0;
         sm.scan[tid] = v - w;
     }
     if (tid == 0) sm.cnt[kCntPruned] = 0u;
@@ -133,51 +136,71 @@ __device__ bool finalize(const TableDev& T, const VarLayout& V, uint32_t* __rest
     int st = sm.scan[kSlotStatus];
     // With the filter beside the update, the failure (Algorithm 1 line 5) is
     // decided here from the update's live count, read in the header round.
-    if (lastDomHere && st == CT_OK && sm.scan[kSlotLiveOut] == 0) st = CT_INFEASIBLE;
+    if (early && st == CT_OK && sm.scan[kSlotLiveOut] == 0) st = CT_INFEASIBLE;
     if (nh < 0 && st == CT_OK && sm.scan[kSlotScan] > 0) return false;
-    nh = sm.scan[kSlotHard];
-    if (st == CT_OK && nh > 0) {
-        uint32_t pruned = 0;
+    const bool any = sm.scan[kSlotHard] > 0;  // a value may be removed
+    if (any && smemDom) {
+        for (int q = tid; q < T.DW; q += kThreads) rm[q] = q == tid ? preRm : __ldcg(&T.removed[q]);
+        __syncthreads();
+    }
+    if (st == CT_OK && !any && smemDom) {
+        for (int q = tid; q < T.DW; q += kThreads) T.lastDom[q] = sm.dom[q];
+    } else if (st == CT_OK) {
         for (int m = tid; m < nh; m += kThreads) {
             const int r = m == tid ? preRow : __ldcg(&T.hardRow[m]);
             const int fc = m == tid ? preFc : __ldcg(&T.foundChunk[m]);
-            // positive tables: a chunk holding a support, or kNoChunk / kNoSupport;
+            // positive tables: a chunk holding a support, or kNoChunk;
             // negative tables: fc counts the valid forbidden tuples with the value
-            const bool keep = T.negative ? (unsigned long long)fc < sm.other[T.rowVar[r]] : (fc >= 0 && fc != kNoChunk);
+            const bool keep = T.negative ? (unsigned long long)fc < sm.other[T.rowVar[r]] : fc != kNoChunk;
             if (keep) {
                 if (!T.negative) T.residue[r] = fc;
             } else {
                 // Algorithm 3 line 4: no live tuple carries the value.
                 const int i = T.rowVar[r];
                 const int a = r - V.row0(i);
-                if (dom) atomicAnd(&dom[V.off(i) + (a >> 5)], ~(1u << (a & 31)));
-                if (smemDom) atomicAnd(&sm.dom[V.ld(i) + (a >> 5)], ~(1u << (a & 31)));
-                // a positive table's removed value carries no valid tuple, so
-                // lastDom may drop it now; a negative table's value still has
-                // valid forbidden tuples, which the next call removes as Delta;
-                // a shard's value may be supported by another shard
-                if (!T.negative && !T.shard && !lastDomHere)
-                    atomicAnd(&T.lastDom[V.ld(i) + (a >> 5)], ~(1u << (a & 31)));
-                atomicOr(reinterpret_cast<unsigned*>(&sm.scan[kChgBase + (i >> 5)]), 1u << (i & 31));
-                ++pruned;
+                atomicOr(&rm[V.ld(i) + (a >> 5)], 1u << (a & 31));
+            }
+        }
+        __syncthreads();
+        // a positive table's removed value carries no valid tuple, so lastDom
+        // drops it now; a negative table's value still has valid forbidden
+        // tuples, which the next call removes as Delta; a shard's value may be
+        // supported by another shard
+        const bool keepLast = T.negative || T.shard;
+        uint32_t pruned = 0;
+        for (int i = tid >> lg; i < T.arity; i += ngrp) {
+            for (int q = sub; q < V.nw(i); q += gl) {
+                const int w = V.ld(i) + q;
+                const uint32_t r = smemDom ? rm[w] : __ldcg(&rm[w]);
+                const uint32_t d = smemDom ? sm.dom[w] : __ldcg(&dom[V.off(i) + q]);
+                T.lastDom[w] = keepLast ? d : d & ~r;
+                if (r) {
+                    if (dom) dom[V.off(i) + q] = d & ~r;
+                    if (smemDom) sm.dom[w] = d & ~r;
+                    T.removed[w] = 0u;
+                    atomicOr(reinterpret_cast<unsigned*>(&sm.scan[kChgBase + (i >> 5)]), 1u << (i & 31));
+                    pruned += __popc(r);
+                }
             }
         }
         if (pruned) atomicAdd(&sm.cnt[kCntPruned], pruned);
         __syncthreads();
         if (sm.cnt[kCntPruned]) {
             // The changed mask and the domains of the variables that lost values
-            // go to the host (one thread per variable, all read at once).
+            // go to the host.
             uint32_t* outDom = reinterpret_cast<uint32_t*>(H + kStatusHdr + T.nChangedWords);
             for (int q = tid; q < T.nChangedWords; q += kThreads) H[kStatusHdr + q] = sm.scan[kChgBase + q];
-            for (int i = tid; i < T.arity; i += kThreads) {
+            for (int i = tid >> lg; i < T.arity; i += ngrp) {
                 if (!((sm.scan[kChgBase + (i >> 5)] >> (i & 31)) & 1)) continue;
-                for (int k = 0; k < V.nw(i); ++k)
-                    outDom[V.ld(i) + k] = smemDom ? sm.dom[V.ld(i) + k] : __ldcg(&dom[V.off(i) + k]);
+                for (int q = sub; q < V.nw(i); q += gl)
+                    outDom[V.ld(i) + q] = smemDom ? sm.dom[V.ld(i) + q] : __ldcg(&dom[V.off(i) + q]);
             }
         }
+    } else if (any) {
+        // what the probes beside a failed update marked is void
+        for (int q = tid; q < T.DW; q += kThreads)
+            if (smemDom ? rm[q] : __ldcg(&rm[q])) T.removed[q] = 0u;
     }
-    if (lastDomHere && st == CT_OK)
-        for (int q = tid; q < T.DW; q += kThreads) T.lastDom[q] = sm.dom[q];
     // Header: one slot per thread.
     if (tid < kStatusHdr && tid != kSlotStatus) {
         int32_t v = sm.scan[tid];
@@ -204,8 +227,8 @@ __device__ bool finalize(const TableDev& T, const VarLayout& V, uint32_t* __rest
 // residue while most chunks are live, over the LIVE chunks that follow it
 // (found through the non-zero index) when fewer than half are, where a value
 // whose windows covered every live chunk is known unsupported without a scan.
-__device__ __forceinline__ void probe_loaded(const TableDev& T, int r, bool present, int res, const uint4& supRes,
-                                             const uint4& curRes, bool sparse, uint32_t* s_cnt) {
+__device__ __forceinline__ void probe_loaded(const TableDev& T, int r, int word, int bit, bool present, int res,
+                                             const uint4& supRes, const uint4& curRes, bool sparse, uint32_t* s_cnt) {
     const int lane = threadIdx.x & 31;
     if (!present) return;
     if (T.useResidues) {
@@ -215,8 +238,8 @@ __device__ __forceinline__ void probe_loaded(const TableDev& T, int r, bool pres
             return;
         }
     }
-    if (sparse) probe_miss<true, kModelProbes>(T, r, res, s_cnt);
-    else probe_miss<false, kLocalProbes>(T, r, res, s_cnt);
+    if (sparse) probe_miss<true, kModelProbes>(T, r, word, bit, res, s_cnt);
+    else probe_miss<false, kLocalProbes>(T, r, word, bit, res, s_cnt);
 }
 
 // A value of s_sup probed beside the update (r and res uniform over the
@@ -227,8 +250,9 @@ __device__ __forceinline__ void probe_loaded(const TableDev& T, int r, bool pres
 // final once every CTA has released its update), the value is searched again
 // over the live chunks of the index the update left, after waiting for it.
 template <int E>
-__device__ __forceinline__ void probe_early(const TableDev& T, int r, bool present, int res, const int32_t* codes,
-                                            int nrows, bool sparse, unsigned limit, uint32_t* s_cnt) {
+__device__ __forceinline__ void probe_early(const TableDev& T, int r, int word, int bit, bool present, int res,
+                                            const int32_t* codes, int nrows, bool sparse, unsigned limit,
+                                            uint32_t* s_cnt) {
     const int lane = threadIdx.x & 31;
     if (!present) return;
     bool hit = false;
@@ -241,7 +265,7 @@ __device__ __forceinline__ void probe_early(const TableDev& T, int r, bool prese
                    : probe_windows<false, kLocalProbes, E>(T, r, res, s_cnt, codes, nrows);
     if (o == kProbeUndecided && wait_update_done(T.ctrl, limit) && 2u * __ldcg(&T.ctrl->live) < (uint32_t)T.W4)
         o = probe_windows<true, kModelProbes>(T, r, res, s_cnt);
-    note_probe(T, r, o, s_cnt);
+    if (lane == 0) note_probe(T, r, word, bit, o, s_cnt);
 }
 
 // Per-CTA counters of a phase into the control block (zero counts skipped).
@@ -287,9 +311,14 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     if (gwarp < T.nseg) seg0 = load_segment(T, gwarp, P.mark);
     // (the supports chunk at the residue is loaded after the plan, so that the
     // warp does not wait for the residue before the plan's loads)
+    // Local plans probe a value per warp; global ones (more than kCodeCap
+    // values) rpw values at a time, one per lane.
+    const int rpw = kLocal ? 1 : min(32, (T.R + nwarps - 1) / nwarps);
+    const int r0 = gwarp * rpw + lane;  // the lane's first value
+    const bool mine0 = T.useResidues && lane < rpw && r0 < T.R;
     int res0 = 0;
     uint4 supRes0 = make_uint4(0u, 0u, 0u, 0u);
-    if (T.useResidues && gwarp < T.R && lane == 0) res0 = T.residue[gwarp];
+    if (mine0) res0 = T.residue[r0];
     // With the filter beside the update (a call of at most U rows: one warp
     // per segment, one round), the warps after the round's segments take the
     // values first: warp g starts at value (g - nseg) mod nwarps.
@@ -310,19 +339,15 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             // every value of x_i is excluded when all prod_{j != i} |D_j| combinations
             // with it are forbidden: the products, saturated at 2^62
             if (tid == 0) {
-                const unsigned long long cap = 1ull << 62;
-                auto mul = [&](unsigned long long a, unsigned long long b) {
-                    return (b != 0 && a > cap / b) ? cap : a * b;
-                };
                 unsigned long long pre = 1ull;
                 for (int i = 0; i < T.arity; ++i) {
                     sm.other[i] = pre;
-                    pre = mul(pre, (unsigned long long)sm.nd[i]);
+                    pre = sat_mul(pre, (unsigned long long)sm.nd[i]);
                 }
                 unsigned long long suf = 1ull;
                 for (int i = T.arity - 1; i >= 0; --i) {
-                    sm.other[i] = mul(sm.other[i], suf);
-                    suf = mul(suf, (unsigned long long)sm.nd[i]);
+                    sm.other[i] = sat_mul(sm.other[i], suf);
+                    suf = sat_mul(suf, (unsigned long long)sm.nd[i]);
                 }
             }
             __syncthreads();
@@ -360,8 +385,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     // takes the same decision (each computed the same plan).
     const bool early = kLocal && ok && nrows > 0 && nrows <= U && nrows <= P.early && !T.negative && !T.shard &&
                        T.useResidues && 2 * P.prevLive >= T.W4;
-    if (T.useResidues && gwarp < T.R && lane == 0 && !early)
-        supRes0 = ld_sup(T.sup + (size_t)gwarp * T.W4 + res0);
+    if (mine0 && !early) supRes0 = ld_sup(T.sup + (size_t)r0 * T.W4 + res0);
 
     uint4 curRes0 = make_uint4(0u, 0u, 0u, 0u);
     bool sparse = 2 * P.prevLive < T.W4;  // fewer than half the chunks live (after the update: recomputed)
@@ -382,7 +406,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             C->live_in = (uint32_t)P.prevLive;
             C->t[2] = C->t[1];
         }
-        if (T.useResidues && gwarp < T.R && lane == 0) curRes0 = __ldcg(T.curr + res0);
+        if (mine0) curRes0 = __ldcg(T.curr + res0);
     } else {
         // update (Algorithm 2): the row list of a segment is cut into G slices,
         // G a power of two and at most P.maxSplit, as large as keeps every
@@ -483,7 +507,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
         // table with no valid forbidden tuple forbids nothing; an empty shard
         // supports no value, which the filter finds). The residue chunk of the
         // warp's first probe is loaded beside the failure test.
-        if (T.useResidues && gwarp < T.R && lane == 0) curRes0 = __ldcg(T.curr + res0);
+        if (mine0) curRes0 = __ldcg(T.curr + res0);
         const int st1 = __ldcg(&C->status);
         const uint32_t live1 = __ldcg(&C->live);
         sparse = 2u * live1 < (uint32_t)T.W4;
@@ -500,62 +524,110 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     // residue probes (Algorithm 3)
     if (tid < 12) sm.cnt[tid] = 0u;
     __syncthreads();
-    // lastDom := the domains of this call (values pruned below are cleared
-    // again by the finalizing CTA).
-    if (blockIdx.x == 0 && !early) {
-        if (kLocal) {
-            for (int q = tid; q < T.DW; q += kThreads) T.lastDom[q] = sm.dom[q];
-        } else {
-            for (int i = tid; i < T.arity; i += kThreads)
-                for (int q = 0; q < V.nw(i); ++q) T.lastDom[V.ld(i) + q] = dom[V.off(i) + q];
-        }
-    }
+    // Tables of at most kLocalProbes windows: the windows after the residue
+    // cover every chunk, so the live chunks need no index walk and no value is
+    // left for the full scan (a 2-chunk table's calls with an unsupported value
+    // 17.1 -> 10.4 us of device time).
+    if (T.W4 <= 32 * kLocalProbes) sparse = false;
     if (kLocal && T.negative) {
         // Negative tables: a value loses its support only when the valid
         // forbidden tuples carrying it are all prod_{j != i} |D_j| combinations;
         // values whose product exceeds the valid tuples keep it without a count.
         const unsigned long long liveT = __ldcg(&C->tuples);
-        for (int r = blockIdx.x * kThreads + tid; r < T.R; r += gridDim.x * kThreads) {
-            const int i = __ldg(&T.rowVar[r]);
-            const int a = r - V.row0(i);
-            const bool present = (sm.dom[V.ld(i) + (a >> 5)] >> (a & 31)) & 1u;
-            if (present && sm.other[i] <= liveT) {
-                const unsigned m = atomicAdd(&C->nhard, 1u);
+        for (int b0 = (blockIdx.x * kWarps + warp) * 32; b0 < T.R; b0 += gridDim.x * kThreads) {
+            const int r = b0 + lane;
+            bool need = false;
+            if (r < T.R) {
+                const int i = __ldg(&T.rowVar[r]);
+                const int a = r - V.row0(i);
+                need = ((sm.dom[V.ld(i) + (a >> 5)] >> (a & 31)) & 1u) && sm.other[i] <= liveT;
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, need);
+            if (!bal) continue;
+            int m = 0;
+            if (lane == 0) {
+                m = atomicAdd(&C->nscan, __popc(bal));
+                atomicAdd(&sm.cnt[kCntHard], (uint32_t)__popc(bal));
+            }
+            m = __shfl_sync(0xffffffffu, m, 0) + __popc(bal & lanemask_lt());
+            if (need) {
                 T.hardRow[m] = r;
                 T.foundChunk[m] = 0;
-                atomicAdd(&C->nscan, 1);
             }
         }
     } else if (early) {
         for (int r = pfirstE; r < T.R; r += nwarps) {
             const int i = __ldg(&T.rowVar[r]);
             const int a = r - V.row0(i);
-            const bool present = sm.sup[i] && ((sm.dom[V.ld(i) + (a >> 5)] >> (a & 31)) & 1u);
+            const int word = V.ld(i) + (a >> 5);
+            const bool present = sm.sup[i] && ((sm.dom[word] >> (a & 31)) & 1u);
             int res = resE;
             if (r != pfirstE && present && lane == 0) res = T.residue[r];
             res = __shfl_sync(0xffffffffu, res, 0);
-            if (nrows <= 4) probe_early<4>(T, r, present, res, sm.codes, nrows, sparse, bar.limit, sm.cnt);
-            else probe_early<U>(T, r, present, res, sm.codes, nrows, sparse, bar.limit, sm.cnt);
+            if (nrows <= 4)
+                probe_early<4>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.cnt);
+            else
+                probe_early<U>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.cnt);
         }
-    } else
-    for (int r = gwarp; r < T.R; r += nwarps) {
-        const int i = __ldg(&T.rowVar[r]);
-        const int a = r - V.row0(i);
-        bool present;
-        if (kLocal) {
-            present = sm.sup[i] && ((sm.dom[V.ld(i) + (a >> 5)] >> (a & 31)) & 1u);
-        } else {
-            present = __ldcg(&T.varSup[i]) && ((dom[V.off(i) + (a >> 5)] >> (a & 31)) & 1u);
+    } else if (kLocal) {
+        for (int r = gwarp; r < T.R; r += nwarps) {
+            const int i = __ldg(&T.rowVar[r]);
+            const int a = r - V.row0(i);
+            const int word = V.ld(i) + (a >> 5);
+            const bool present = sm.sup[i] && ((sm.dom[word] >> (a & 31)) & 1u);
+            int res = res0;
+            uint4 sr = supRes0, cr = curRes0;
+            if (r != gwarp && T.useResidues && present && lane == 0) {
+                res = T.residue[r];
+                sr = ld_sup(T.sup + (size_t)r * T.W4 + res);
+                cr = __ldcg(T.curr + res);
+            }
+            res = __shfl_sync(0xffffffffu, res, 0);
+            probe_loaded(T, r, word, a & 31, present, res, sr, cr, sparse, sm.cnt);
         }
-        int res = res0;
-        uint4 sr = supRes0, cr = curRes0;
-        if (r != gwarp && T.useResidues && present && lane == 0) {
-            res = T.residue[r];
-            sr = ld_sup(T.sup + (size_t)r * T.W4 + res);
-            cr = __ldcg(T.curr + res);
+    } else {
+        // one value per lane: its residue chunk; the warp then searches the
+        // values that missed it (a warp per value spent 80 us on 50,000 values
+        // of a 79-chunk table, mostly on round trips one after the other)
+        for (int b0 = gwarp * rpw; b0 < T.R; b0 += nwarps * rpw) {
+            const int r = b0 + lane;
+            bool need = false, hit = false;
+            int word = 0, bit = 0, res = res0;
+            if (lane < rpw && r < T.R) {
+                const int i = __ldg(&T.rowVar[r]);
+                const int a = r - V.row0(i);
+                word = V.ld(i) + (a >> 5);
+                bit = a & 31;
+                // (this call's removals are in T.removed: the domains stay as they came)
+                need = __ldcg(&T.varSup[i]) && ((dom[V.off(i) + (a >> 5)] >> bit) & 1u);
+                if (need && T.useResidues) {
+                    uint4 sr = supRes0, cr = curRes0;
+                    if (b0 != gwarp * rpw) {
+                        res = T.residue[r];
+                        sr = ld_sup(T.sup + (size_t)r * T.W4 + res);
+                        cr = __ldcg(T.curr + res);
+                    }
+                    hit = nz(and4(sr, cr));
+                    need = !hit;
+                }
+            }
+            const unsigned nhit = __popc(__ballot_sync(0xffffffffu, hit));
+            unsigned miss = __ballot_sync(0xffffffffu, need);
+            if (lane == 0 && nhit) atomicAdd(&sm.cnt[kCntHits], nhit);
+            int o = kProbeUndecided;  // the lane's outcome
+            if (T.useResidues && !sparse) {
+                o = probe_dense_lanes<4>(T, miss, r, res, sm.cnt);
+            } else if (T.useResidues) {
+                while (miss) {
+                    const int l = __ffs(miss) - 1;
+                    miss &= miss - 1u;
+                    const int ol = probe_windows<true, kModelProbes>(T, __shfl_sync(0xffffffffu, r, l),
+                                                                     __shfl_sync(0xffffffffu, res, l), sm.cnt);
+                    if (lane == l) o = ol;
+                }
+            }
+            if (need) note_probe(T, r, word, bit, o, sm.cnt);
         }
-        res = __shfl_sync(0xffffffffu, res, 0);
-        probe_loaded(T, r, present, res, sr, cr, sparse, sm.cnt);
     }
     __syncthreads();
     if (tid == 0) {
@@ -563,6 +635,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
         if (sm.cnt[kCntLocal]) atomicAdd(&C->local_found, (int)sm.cnt[kCntLocal]);
         if (sm.cnt[kCntMiss]) atomicAdd(&C->misses, (int)sm.cnt[kCntMiss]);
         if (sm.cnt[kCntWin]) atomicAdd(&C->windows, (int)sm.cnt[kCntWin]);
+        if (sm.cnt[kCntHard]) atomicAdd(&C->nhard, sm.cnt[kCntHard]);
     }
     CT_STAMP(4);
     const int r2 = bar_sync(bar, &sm.flag[0]);
@@ -585,20 +658,26 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
         CT_STAMP(6);
         return;
     }
-    if (__ldcg(&C->nscan) == 0) return;
-    const int nh = (int)__ldcg(&C->nhard);
+    const int nh = __ldcg(&C->nscan);
+    if (nh == 0) return;
     if (r2 == 2 && tid == 0) C->t[3] = t3;
-    // full scan of the hard values
+    // full scan of the undecided values: (segment, slice of the hard list)
+    // units, as many slices as the grid's warps have room for (a segment's
+    // whole list on one warp took 6.2 ms for 16,700 values of a 3-segment
+    // table, and 13.7 us of a negative table's 24 us call)
     CT_STAMP(11);
     {
         const int staged = min(nh, kCodeCap);
         for (int q = tid; q < staged; q += kThreads) sm.codes[q] = __ldcg(&T.hardRow[q]);
         __syncthreads();
         CT_STAMP(12);
-        if (T.negative) {
-            for (int seg = gwarp; seg < T.nseg; seg += nwarps) count_segment(T, seg, nh, sm.codes);
-        } else {
-            for (int seg = gwarp; seg < T.nseg; seg += nwarps) scan_segment<U>(T, seg, nh, sm.codes);
+        constexpr int kPer = 4;  // fewest values a slice is cut for
+        const int slices = max(1, min((nh + kPer - 1) / kPer, nwarps / T.nseg));
+        const int per = (nh + slices - 1) / slices;
+        for (int u = gwarp; u < T.nseg * slices; u += nwarps) {
+            const int seg = u % T.nseg, ma = (u / T.nseg) * per, mb = min(nh, ma + per);
+            if (T.negative) count_segment(T, seg, ma, mb, sm.codes);
+            else scan_segment<U>(T, seg, ma, mb, sm.codes);
         }
     }
     // last-block-done

@@ -686,19 +686,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
                     // a value of x_i loses its support when its valid forbidden
                     // tuples are all prod_{j != i} |D_j| combinations: the products,
                     // saturated at 2^62
-                    const unsigned long long cap = 1ull << 62;
-                    auto mul = [&](unsigned long long x, unsigned long long y) {
-                        return (y != 0 && x > cap / y) ? cap : x * y;
-                    };
                     unsigned long long pre = 1ull;
                     for (int i = 0; i < T.arity; ++i) {
                         T.other[i] = pre;
-                        pre = mul(pre, (unsigned long long)sm.nd[i]);
+                        pre = sat_mul(pre, (unsigned long long)sm.nd[i]);
                     }
                     unsigned long long suf = 1ull;
                     for (int i = T.arity - 1; i >= 0; --i) {
-                        T.other[i] = mul(T.other[i], suf);
-                        suf = mul(suf, (unsigned long long)sm.nd[i]);
+                        T.other[i] = sat_mul(T.other[i], suf);
+                        suf = sat_mul(suf, (unsigned long long)sm.nd[i]);
                     }
                 }
                 if (tid == 0) {
@@ -895,8 +891,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
                 const int k = find_prefix(pU, nwork, u, gpre);
                 const TableDev& T = M.tabs[__ldcg(&work[k])];
                 if (__ldcg(&T.ctrl->nscan) == 0) continue;
-                if (T.negative) count_segment(T, u - pre_at(pU, k, gpre), (int)__ldcg(&T.ctrl->nhard), nullptr);
-                else scan_segment<U, true>(T, u - pre_at(pU, k, gpre), (int)__ldcg(&T.ctrl->nhard), nullptr);
+                if (T.negative) count_segment(T, u - pre_at(pU, k, gpre), 0, (int)__ldcg(&T.ctrl->nhard), nullptr);
+                else scan_segment<U, true>(T, u - pre_at(pU, k, gpre), 0, (int)__ldcg(&T.ctrl->nhard), nullptr);
             }
             if (!sync()) return;
             phase(4);

@@ -17,6 +17,7 @@
 // kNaMaxRows supports rows (sum of the domain sizes) and kNaMaxChunks 128-bit
 // chunks of currTable (8,388,608 tuples). Backtracking is the caller's
 // business (it keeps copies of the buffers it wants to return to).
+#include <algorithm>
 #include <atomic>
 #include <cstddef>
 #include <cstring>
@@ -44,6 +45,7 @@ struct NaScratch {
     int32_t hardRow[kNaMaxRows];
     int32_t foundChunk[kNaMaxRows];
     int32_t residue[kNaMaxRows];
+    uint32_t removed[kNaMaxDW];
     int32_t rowVar[kNaMaxRows];
     int32_t varSup[kNaMaxArity];
     int32_t planK[kNaMaxArity];
@@ -90,6 +92,7 @@ __global__ void ct_noalloc_init_kernel(const __grid_constant__ NaInit p) {
         const uint32_t m = __ballot_sync(0xffffffffu, live);
         if (lane == 0) S->segMask[seg0 >> 5] = m;
     }
+    if (tid < kNaMaxDW) S->removed[tid] = 0u;
     if (tid == 0) {
         S->status[kSlotStatus] = kNaPending;
     }
@@ -193,6 +196,7 @@ extern "C" int ct_propagate_noalloc(int arity, const int32_t* dom_size, int64_t 
     T.other = nullptr;  // positive tables only
     T.hardRow = S->hardRow;
     T.foundChunk = S->foundChunk;
+    T.removed = S->removed;
     T.rowVar = S->rowVar;
     T.statusBlk = S->status;
     T.arity = arity;
@@ -203,6 +207,8 @@ extern "C" int ct_propagate_noalloc(int arity, const int32_t* dom_size, int64_t 
     T.DW = DW;
     T.nChangedWords = 1;
     T.useResidues = 1;
+    const int maxNW = *std::max_element(nw, nw + arity);
+    while (maxNW > 2 && T.wordLanesLog < 5 && (1 << T.wordLanesLog) < maxNW) ++T.wordLanesLog;
     for (int i = 0; i < arity; ++i) {
         T.pNW[i] = nw[i];
         T.pLD[i] = ld[i];

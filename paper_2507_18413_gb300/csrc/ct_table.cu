@@ -443,6 +443,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     if ((st = dalloc(ct, &d.other, (size_t)n)) != CT_OK) return st;
     if ((st = dalloc(ct, &d.hardRow, (size_t)R)) != CT_OK) return st;
     if ((st = dalloc(ct, &d.foundChunk, (size_t)R)) != CT_OK) return st;
+    if ((st = dalloc(ct, &d.removed, (size_t)DW)) != CT_OK) return st;
     if ((st = dalloc(ct, &rowVar, (size_t)R)) != CT_OK) return st;
     if ((st = dalloc(ct, &varRow0, (size_t)n + 1)) != CT_OK) return st;
     if ((st = dalloc(ct, &varNW, (size_t)n)) != CT_OK) return st;
@@ -465,6 +466,8 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     d.DW = DW;
     d.nChangedWords = ct->nChW;
     d.useResidues = (opt && opt->no_residues) ? 0 : 1;
+    const int maxNW = *std::max_element(ct->nw.begin(), ct->nw.end());
+    while (maxNW > 2 && d.wordLanesLog < 5 && (1 << d.wordLanesLog) < maxNW) ++d.wordLanesLog;
     d.warpPlan = (!ct->negative && n <= 32) ? 1 : 0;
     for (int i = 0; i < n; ++i)
         if (ct->nw[i] > kWarpPlanWords) d.warpPlan = 0;
@@ -524,6 +527,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     if ((st = upload(ct, varRow0, ct->row0)) != CT_OK) return st;
     if ((st = upload(ct, varNW, ct->nw)) != CT_OK) return st;
     if ((st = upload(ct, varLD, ct->ld)) != CT_OK) return st;
+    CT_CUDA(cudaMemsetAsync(d.removed, 0, (size_t)DW * sizeof(uint32_t), ct->stream));
     CT_CUDA(cudaMemsetAsync(d.other, 0, (size_t)n * sizeof(unsigned long long), ct->stream));
 
     Ctrl c{};
