@@ -19,13 +19,15 @@
 // Network: h1 = relu(W1 x + b1), h2 = relu(W2 h1 + b2), out = W3 . h2 + b3,
 // float32, weights flat as W1[64][8], b1, W2[64][64], b2, W3[64], b3.
 // Training: loss sum (out - y)^2 / (2B) per batch, Adam (Kingma and Ba, 2015;
-// beta1 0.9, beta2 0.999, eps 1e-8, bias-corrected), one CTA that keeps the
-// weights, both moments and the batch's activations in shared memory and
-// walks the given epoch orders in consecutive batches.
+// beta1 0.9, beta2 0.999, eps 1e-8, bias-corrected), one cluster of CTAs that
+// keeps the weights and the batch's activations in shared memory and the
+// moments in registers and walks the given epoch orders in consecutive batches.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "ct_learn.cuh"
 
@@ -346,154 +348,328 @@ struct TrainArgs {
     int32_t gradOnly;
 };
 
+// Training runs on one cluster of kTrainCtas CTAs. The passes over the layers
+// are split by samples (CTA r takes the r-th run of the batch, a half-warp per
+// sample, 16 lanes x 4 hidden units, so that the layers need no CTA barrier:
+// the activations a half-warp reads are the ones it wrote); the gradients and
+// Adam by units (CTA r owns units 8r .. 8r + 7 of both layers: their rows of W1
+// and W2, their biases and W3 entries, with the moments in registers). Each
+// half-warp stores what the owners need into their shared memory, and the
+// owners store the new weights into everybody's: two cluster barriers a batch.
+// Every sum runs in one thread over its inputs in order (units 0..63, samples
+// 0..b-1), whatever the split: Adam divides a gradient by its own size, so one
+// that cancels to rounding noise makes a full step, and another order of
+// summation would make another network.
+// What bounds a batch of 128 samples: the shared memory the products read
+// (about 1.2 us for the two 64 x 64 passes, 0.8 us for the gradients), the
+// chains of 64 and 128 dependent FMAs, the exchange and the barriers. W2 is
+// kept in both orders, so that the forward and the backward pass both read
+// consecutive 128-bit words (one order made every read of the other a 32-way
+// bank conflict: one CTA took 115 us per batch of 128).
 constexpr int kTrainThreads = 256;
+constexpr int kTrainCtas = 8;
+constexpr int kTrainSamples = kTrainBatch / kTrainCtas;  // per CTA and batch
+constexpr int kOwnU = kNH / kTrainCtas;                  // units a CTA owns
+constexpr int kRow = kNH + 4;                            // padded activation row (two samples of a warp: other banks)
+static_assert(kTrainSamples * 16 == kTrainThreads && kNH == 64 && kNF == 8 && kOwnU == 8,
+              "a half-warp per sample, 4 units per lane, 8 units per CTA");
 
-// Shared-memory layout of the training CTA (floats).
-constexpr int sW = 0, sM = sW + kNW, sV = sM + kNW, sX = sV + kNW, sY = sX + kTrainBatch * kNF,
-              sH1 = sY + kTrainBatch, sH2 = sH1 + kTrainBatch * kNH, sD1 = sH2 + kTrainBatch * kNH,
-              sOut = sD1 + kTrainBatch * kNH, sRed = sOut + kTrainBatch, sTotal = sRed + kTrainThreads;
-constexpr size_t kTrainSmem = (size_t)sTotal * sizeof(float);
+struct TrainSmem {
+    float w2[kNH * kNH];       // [j][i]: unit j of layer 2, input i
+    float w2t[kNH * kNH];      // [i][j]
+    float w1t[kNF * kNH];      // [i][j]
+    float b1[kNH], b2[kNH], w3[kNH];
+    // the whole batch, written by the CTAs that hold the samples
+    float h1[kTrainBatch * kRow];   // layer-1 activations
+    float x[kTrainBatch * kNF];
+    float d1o[kTrainBatch * kOwnU], d2o[kTrainBatch * kOwnU], h2o[kTrainBatch * kOwnU];  // of the owned units
+    float dout[kTrainBatch], sq[kTrainBatch];
+    // the CTA's own samples
+    float h2[kTrainSamples * kRow], d2[kTrainSamples * kRow];
+    float c[2][2];  // Adam's bias corrections of a batch, by batch parity
+    float b3;
+};
 
-__device__ __forceinline__ void adam(float* w, float* m, float* v, int i, float g, float lr, float c1, float c2) {
-    const float mi = 0.9f * m[i] + 0.1f * g;
-    const float vi = 0.999f * v[i] + 0.001f * g * g;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+
+__device__ __forceinline__ void fma4(float4& a, float s, const float4& v) {
+    a.x = fmaf(s, v.x, a.x);
+    a.y = fmaf(s, v.y, a.y);
+    a.z = fmaf(s, v.z, a.z);
+    a.w = fmaf(s, v.w, a.w);
 }
 
-__global__ void __launch_bounds__(kTrainThreads, 1) ct_mlp_train_kernel(const TrainArgs A) {
-    extern __shared__ float sm[];
-    float* W = sm + sW;
-    float* M = sm + sM;
-    float* V = sm + sV;
-    float* xb = sm + sX;
-    float* yb = sm + sY;
-    float* H1 = sm + sH1;  // activations of layer 1, then kept for the layer-1 mask
-    float* H2 = sm + sH2;  // activations of layer 2, then dL/dz2
-    float* D1 = sm + sD1;  // dL/dz1
-    float* dout = sm + sOut;
-    float* red = sm + sRed;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < kNW; i += kTrainThreads) {
-        W[i] = A.w[i];
-        M[i] = A.m[i];
-        V[i] = A.v[i];
+__device__ __forceinline__ float4 relu4(const float4& v) {
+    return make_float4(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f), fmaxf(v.z, 0.0f), fmaxf(v.w, 0.0f));
+}
+
+__device__ __forceinline__ float4 keep4(const float4& on, const float4& v) {
+    return make_float4(on.x > 0.0f ? v.x : 0.0f, on.y > 0.0f ? v.y : 0.0f, on.z > 0.0f ? v.z : 0.0f,
+                       on.w > 0.0f ? v.w : 0.0f);
+}
+
+// acc + sum_k row[k] * M[k][4q .. 4q+3], k ascending (the row broadcast to the
+// half-warp, M's rows read as consecutive float4 by its lanes).
+__device__ __forceinline__ float4 row_times(const float* row, const float* M, int q, float4 acc) {
+#pragma unroll 4
+    for (int k = 0; k < kNH; k += 4) {
+        const float4 r = ld4(row + k);
+        fma4(acc, r.x, ld4(M + (k + 0) * kNH + 4 * q));
+        fma4(acc, r.y, ld4(M + (k + 1) * kNH + 4 * q));
+        fma4(acc, r.z, ld4(M + (k + 2) * kNH + 4 * q));
+        fma4(acc, r.w, ld4(M + (k + 3) * kNH + 4 * q));
     }
-    __syncthreads();
-    int64_t t = A.t0;
+    return acc;
+}
+
+__device__ __forceinline__ void adam(float& w, float& m, float& v, float g, float lr, float c1, float c2) {
+    const float mi = 0.9f * m + 0.1f * g;
+    const float vi = 0.999f * v + 0.001f * g * g;
+    m = mi;
+    v = vi;
+    w -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+}
+
+__global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(kTrainThreads, 1)
+ct_mlp_train_kernel(const TrainArgs A) {
+    extern __shared__ __align__(16) unsigned char s_train[];
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(s_train);
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, half = lane >> 4, q = lane & 15;
+    const int sl = (tid >> 5) * 2 + half;  // the half-warp's sample in the CTA
+    TrainSmem* peer[kTrainCtas];
+#pragma unroll
+    for (int r = 0; r < kTrainCtas; ++r) peer[r] = cluster.map_shared_rank(&S, r);
+    for (int e = tid; e < kNH * kNH; e += kTrainThreads) {
+        const float u = A.w[oW2 + e];
+        S.w2[e] = u;
+        S.w2t[(e % kNH) * kNH + e / kNH] = u;
+    }
+    for (int e = tid; e < kNH * kNF; e += kTrainThreads) S.w1t[(e % kNF) * kNH + e / kNF] = A.w[oW1 + e];
+    if (tid < kNH) {
+        S.b1[tid] = A.w[oB1 + tid];
+        S.b2[tid] = A.w[oB2 + tid];
+        S.w3[tid] = A.w[oW3 + tid];
+    }
+    if (tid == 0) {
+        S.b3 = A.w[oB3];
+        S.c[0][0] = 1.0f - powf(0.9f, (float)(A.t0 + 1));
+        S.c[0][1] = 1.0f - powf(0.999f, (float)(A.t0 + 1));
+    }
+    for (int e = tid; e < kTrainBatch; e += kTrainThreads) S.sq[e] = 0.0f;
+    // The entries a thread owns: threads 0..127 four consecutive inputs of one
+    // W2 row, 128..191 a W1 entry, 192..215 a bias or W3 entry, 216 (CTA 0) b3.
+    const int uj = tid < 128 ? tid >> 4 : tid < 192 ? (tid - 128) / kNF : (tid - 192) & 7;  // owned unit
+    const int unit = rank * kOwnU + uj;
+    const int ui = tid < 128 ? 4 * (tid & 15) : (tid - 128) % kNF;  // its (first) input
+    const int nOwn = tid < 128 ? 4 : (tid < 216 || (tid == 216 && rank == 0)) ? 1 : 0;
+    const int e0 = tid < 128 ? oW2 + unit * kNH + ui
+                   : tid < 192 ? oW1 + unit * kNF + ui
+                   : tid < 200 ? oB1 + unit
+                   : tid < 208 ? oB2 + unit
+                   : tid < 216 ? oW3 + unit : oB3;
+    float w[4], m[4], v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        w[k] = k < nOwn ? A.w[e0 + k] : 0.0f;
+        m[k] = k < nOwn ? A.m[e0 + k] : 0.0f;
+        v[k] = k < nOwn ? A.v[e0 + k] : 0.0f;
+    }
     const int epochs = A.gradOnly ? 1 : A.epochs;
-    for (int e = 0; e < epochs; ++e) {
-        const int32_t* order = A.order + (size_t)e * A.n;
-        float lossSum = 0.0f;
-        int nb = 0;
-        const int nLast = A.gradOnly ? min(A.n, A.batch) : A.n;
-        for (int s0 = 0; s0 < nLast; s0 += A.batch) {
-            const int b = min(A.batch, nLast - s0);
-            for (int i = tid; i < b * kNF; i += kTrainThreads) xb[i] = A.X[(size_t)order[s0 + i / kNF] * kNF + i % kNF];
-            for (int i = tid; i < b; i += kTrainThreads) yb[i] = A.y[order[s0 + i]];
-            __syncthreads();
-            // forward
-            for (int q = tid; q < b * kNH; q += kTrainThreads) {
-                const int s = q / kNH, j = q % kNH;
-                float acc = W[oB1 + j];
-                for (int i = 0; i < kNF; ++i) acc += W[oW1 + j * kNF + i] * xb[s * kNF + i];
-                H1[q] = fmaxf(acc, 0.0f);
-            }
-            __syncthreads();
-            for (int q = tid; q < b * kNH; q += kTrainThreads) {
-                const int s = q / kNH, j = q % kNH;
-                float acc = W[oB2 + j];
-                for (int i = 0; i < kNH; ++i) acc += W[oW2 + j * kNH + i] * H1[s * kNH + i];
-                H2[q] = fmaxf(acc, 0.0f);
-            }
-            __syncthreads();
-            float part = 0.0f;
-            for (int s = tid; s < b; s += kTrainThreads) {
-                float o = W[oB3];
-                for (int j = 0; j < kNH; ++j) o += W[oW3 + j] * H2[s * kNH + j];
-                const float r = o - yb[s];
-                dout[s] = r / (float)b;
-                part += r * r;
-            }
-            red[tid] = part;
-            __syncthreads();
-            for (int o = kTrainThreads / 2; o > 0; o >>= 1) {
-                if (tid < o) red[tid] += red[tid + o];
-                __syncthreads();
-            }
-            const float loss = red[0] / (2.0f * (float)b);
-            ++t;
-            const float c1 = 1.0f - powf(0.9f, (float)t);
-            const float c2 = 1.0f - powf(0.999f, (float)t);
-            // layer 3 gradients (need the layer-2 activations), then dL/dz2 in place
-            float g3 = 0.0f;
-            if (tid < kNH) {
-                for (int s = 0; s < b; ++s) g3 += dout[s] * H2[s * kNH + tid];
-            } else if (tid == kNH) {
-                for (int s = 0; s < b; ++s) g3 += dout[s];
-            }
-            __syncthreads();
-            for (int q = tid; q < b * kNH; q += kTrainThreads) {
-                const int s = q / kNH, j = q % kNH;
-                H2[q] = H2[q] > 0.0f ? dout[s] * W[oW3 + j] : 0.0f;
-            }
-            __syncthreads();
-            if (tid <= kNH) {
-                const int i = tid < kNH ? oW3 + tid : oB3;
-                if (A.gradOnly) A.grad[i] = g3;
-                else adam(W, M, V, i, g3, A.lr, c1, c2);
-            }
-            // dL/dz1 with the old W2
-            for (int q = tid; q < b * kNH; q += kTrainThreads) {
-                const int s = q / kNH, i = q % kNH;
-                float acc = 0.0f;
-                if (H1[q] > 0.0f)
-                    for (int j = 0; j < kNH; ++j) acc += H2[s * kNH + j] * W[oW2 + j * kNH + i];
-                D1[q] = acc;
-            }
-            __syncthreads();
-            // layer 2 gradients and update
-            for (int q = tid; q < kNH * kNH + kNH; q += kTrainThreads) {
-                float g = 0.0f;
-                if (q < kNH * kNH) {
-                    const int j = q / kNH, i = q % kNH;
-                    for (int s = 0; s < b; ++s) g += H2[s * kNH + j] * H1[s * kNH + i];
-                    if (A.gradOnly) A.grad[oW2 + q] = g;
-                    else adam(W, M, V, oW2 + q, g, A.lr, c1, c2);
-                } else {
-                    const int j = q - kNH * kNH;
-                    for (int s = 0; s < b; ++s) g += H2[s * kNH + j];
-                    if (A.gradOnly) A.grad[oB2 + j] = g;
-                    else adam(W, M, V, oB2 + j, g, A.lr, c1, c2);
-                }
-            }
-            // layer 1 gradients and update
-            for (int q = tid; q < kNH * kNF + kNH; q += kTrainThreads) {
-                float g = 0.0f;
-                if (q < kNH * kNF) {
-                    const int j = q / kNF, i = q % kNF;
-                    for (int s = 0; s < b; ++s) g += D1[s * kNH + j] * xb[s * kNF + i];
-                    if (A.gradOnly) A.grad[oW1 + q] = g;
-                    else adam(W, M, V, oW1 + q, g, A.lr, c1, c2);
-                } else {
-                    const int j = q - kNH * kNF;
-                    for (int s = 0; s < b; ++s) g += D1[s * kNH + j];
-                    if (A.gradOnly) A.grad[oB1 + j] = g;
-                    else adam(W, M, V, oB1 + j, g, A.lr, c1, c2);
-                }
-            }
-            __syncthreads();
-            lossSum += loss;
-            ++nb;
+    const int nUse = A.gradOnly ? min(A.n, A.batch) : A.n;
+    const int nb = (nUse + A.batch - 1) / A.batch;
+    const long long total = (long long)nb * epochs;
+    // a batch's size, the samples per CTA, and the half-warp's sample (-1: none)
+    auto sample_of = [&](int ep, int pos, int& b, int& per) -> int {
+        const int s0 = pos * A.batch;
+        b = min(A.batch, nUse - s0);
+        per = (b + kTrainCtas - 1) / kTrainCtas;
+        const int i = rank * per + sl;
+        if (sl >= per || i >= b) return -1;
+        return __ldg(A.order + (size_t)ep * A.n + s0 + i);
+    };
+    // the samples are fetched one batch ahead, their indices two
+    int b = 0, per = 0, bN = 0, perN = 0, ep2 = 0, pos2 = 0;
+    auto advance = [&]() {
+        if (++pos2 == nb) {
+            pos2 = 0;
+            ++ep2;
         }
-        if (tid == 0) A.epochLoss[e] = nb ? lossSum / (float)nb : 0.0f;
+    };
+    float xv = 0.0f, yv = 0.0f;
+    bool valid = false;
+    int idxN = -1;
+    {
+        const int i0 = sample_of(0, 0, b, per);
+        valid = i0 >= 0;
+        if (valid) {
+            if (q < kNF) xv = __ldg(A.X + (size_t)i0 * kNF + q);
+            yv = __ldg(A.y + i0);
+        }
+        advance();
+        if (total > 1) idxN = sample_of(ep2, pos2, bN, perN);
+    }
+    cluster.sync();  // every CTA runs: its shared memory may be written
+    float lossSum = 0.0f;  // CTA 0, thread 224
+    int pos = 0, ep = 0;
+    for (long long kb = 0; kb < total; ++kb) {
+        // next batch's sample, and the one after's index
+        float xN = 0.0f, yN = 0.0f;
+        const bool validN = kb + 1 < total && idxN >= 0;
+        if (validN) {
+            if (q < kNF) xN = __ldg(A.X + (size_t)idxN * kNF + q);
+            yN = __ldg(A.y + idxN);
+        }
+        int b2n = 0, per2n = 0, idx2 = -1;
+        advance();
+        if (kb + 2 < total) idx2 = sample_of(ep2, pos2, b2n, per2n);
+        if ((tid >> 5) * 2 < per) {
+            const int sg = valid ? rank * per + sl : 0;  // the sample in the batch
+            // layer 1: units 4q .. 4q+3
+            float4 h = ld4(S.b1 + 4 * q);
+#pragma unroll
+            for (int i = 0; i < kNF; ++i) fma4(h, __shfl_sync(0xffffffffu, xv, (half << 4) + i), ld4(S.w1t + i * kNH + 4 * q));
+            h = relu4(h);
+            float* own2 = S.h2 + sl * kRow;
+            st4(own2 + 4 * q, h);  // (the row holds layer 1 until layer 2 is done)
+            __syncwarp();
+            float4 z = relu4(row_times(own2, S.w2t, q, ld4(S.b2 + 4 * q)));
+            __syncwarp();
+            st4(own2 + 4 * q, z);
+            __syncwarp();
+            // the output by one lane, units in order
+            float o = S.b3;
+            if (q == 0) {
+#pragma unroll 4
+                for (int j = 0; j < kNH; j += 4) {
+                    const float4 c = ld4(S.w3 + j), g = ld4(own2 + j);
+                    o = fmaf(c.x, g.x, o);
+                    o = fmaf(c.y, g.y, o);
+                    o = fmaf(c.z, g.z, o);
+                    o = fmaf(c.w, g.w, o);
+                }
+            }
+            o = __shfl_sync(0xffffffffu, o, half << 4);
+            const float r = o - yv, dz = r / (float)b;
+            const float4 c = ld4(S.w3 + 4 * q);
+            const float4 d2 = keep4(z, make_float4(dz * c.x, dz * c.y, dz * c.z, dz * c.w));
+            float* rowD = S.d2 + sl * kRow;
+            st4(rowD + 4 * q, d2);
+            __syncwarp();
+            const float4 d1 = keep4(h, row_times(rowD, S.w2, q, make_float4(0.0f, 0.0f, 0.0f, 0.0f)));
+            if (valid) {
+                // to every CTA: layer 1, the inputs, dL/dout; to a unit's owner: its activation and gradients
+#pragma unroll
+                for (int p = 0; p < kTrainCtas; ++p) {
+                    st4(peer[p]->h1 + sg * kRow + 4 * q, h);
+                    if (q < kNF) peer[p]->x[sg * kNF + q] = xv;
+                    if (q == 0) peer[p]->dout[sg] = dz;
+                }
+                TrainSmem* own = cluster.map_shared_rank(&S, q >> 1);
+                const int at = sg * kOwnU + 4 * (q & 1);
+                st4(own->d1o + at, d1);
+                st4(own->d2o + at, d2);
+                st4(own->h2o + at, z);
+                if (q == 0) peer[0]->sq[sg] = r * r;
+            }
+        }
+        cluster.sync();
+        // the owned entries: gradient over the batch (samples in order), Adam
+        const float c1 = S.c[kb & 1][0], c2 = S.c[kb & 1][1];
+        if (tid < 128) {
+            float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 8
+            for (int s = 0; s < b; ++s) fma4(g, S.d2o[s * kOwnU + uj], ld4(S.h1 + s * kRow + ui));
+            if (A.gradOnly) {
+                A.grad[e0] = g.x;
+                A.grad[e0 + 1] = g.y;
+                A.grad[e0 + 2] = g.z;
+                A.grad[e0 + 3] = g.w;
+            } else {
+                adam(w[0], m[0], v[0], g.x, A.lr, c1, c2);
+                adam(w[1], m[1], v[1], g.y, A.lr, c1, c2);
+                adam(w[2], m[2], v[2], g.z, A.lr, c1, c2);
+                adam(w[3], m[3], v[3], g.w, A.lr, c1, c2);
+#pragma unroll
+                for (int p = 0; p < kTrainCtas; ++p) {
+                    st4(peer[p]->w2 + unit * kNH + ui, make_float4(w[0], w[1], w[2], w[3]));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) peer[p]->w2t[(ui + k) * kNH + unit] = w[k];
+                }
+            }
+        } else if (nOwn) {
+            float g = 0.0f;
+            if (tid < 192) {
+#pragma unroll 8
+                for (int s = 0; s < b; ++s) g = fmaf(S.d1o[s * kOwnU + uj], S.x[s * kNF + ui], g);
+            } else if (tid < 208) {
+                const float* d = tid < 200 ? S.d1o : S.d2o;
+#pragma unroll 8
+                for (int s = 0; s < b; ++s) g += d[s * kOwnU + uj];
+            } else if (tid < 216) {
+#pragma unroll 8
+                for (int s = 0; s < b; ++s) g = fmaf(S.dout[s], S.h2o[s * kOwnU + uj], g);
+            } else {
+#pragma unroll 8
+                for (int s = 0; s < b; ++s) g += S.dout[s];
+            }
+            if (A.gradOnly) {
+                A.grad[e0] = g;
+            } else {
+                adam(w[0], m[0], v[0], g, A.lr, c1, c2);
+#pragma unroll
+                for (int p = 0; p < kTrainCtas; ++p) {
+                    TrainSmem* P = peer[p];
+                    float* at = tid < 192 ? &P->w1t[ui * kNH + unit]
+                                : tid < 200 ? &P->b1[unit]
+                                : tid < 208 ? &P->b2[unit]
+                                : tid < 216 ? &P->w3[unit] : &P->b3;
+                    *at = w[0];
+                }
+            }
+        } else if (tid >= 224) {
+            // the last warp: the batch's loss (CTA 0, a binary tree over the
+            // samples), the next batch's bias corrections
+            if (rank == 0) {
+                float l = lane < 32 ? (S.sq[lane] + S.sq[lane + 64]) + (S.sq[lane + 32] + S.sq[lane + 96]) : 0.0f;
+                __syncwarp();
+                for (int k = 0; k < kTrainBatch; k += 32) S.sq[lane + k] = 0.0f;
+#pragma unroll
+                for (int k = 16; k > 0; k >>= 1) l += __shfl_down_sync(0xffffffffu, l, k);
+                if (lane == 0) {
+                    lossSum += l / (2.0f * (float)b);
+                    if (pos + 1 == nb) {
+                        A.epochLoss[ep] = lossSum / (float)nb;
+                        lossSum = 0.0f;
+                    }
+                }
+            }
+            if (lane < 2) {
+                const float t = (float)(A.t0 + kb + 2);
+                S.c[(kb + 1) & 1][lane] = 1.0f - powf(lane == 0 ? 0.9f : 0.999f, t);
+            }
+        }
+        cluster.sync();
+        xv = xN;
+        yv = yN;
+        valid = validN;
+        idxN = idx2;
+        b = bN;
+        per = perN;
+        bN = b2n;
+        perN = per2n;
+        if (++pos == nb) {
+            pos = 0;
+            ++ep;
+        }
     }
     if (A.gradOnly) return;
-    for (int i = tid; i < kNW; i += kTrainThreads) {
-        A.w[i] = W[i];
-        A.m[i] = M[i];
-        A.v[i] = V[i];
+    for (int k = 0; k < nOwn; ++k) {
+        A.w[e0 + k] = w[k];
+        A.m[e0 + k] = m[k];
+        A.v[e0 + k] = v[k];
     }
 }
 
@@ -700,7 +876,7 @@ int run_train(ct_mlp* m, const float* x_host, const float* y_host, int64_t n, co
         e = cudaMalloc((void**)&dLoss, sizeof(float) * (size_t)std::max(epochs, 1));
         if (e == cudaSuccess) e = cudaMalloc((void**)&dGrad, sizeof(float) * kNW);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(ct_mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem);
+            e = cudaFuncSetAttribute(ct_mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem));
         if (e == cudaSuccess) {
             TrainArgs A;
             A.w = m->d_w;
@@ -717,7 +893,7 @@ int run_train(ct_mlp* m, const float* x_host, const float* y_host, int64_t n, co
             A.batch = batch;
             A.lr = lr;
             A.gradOnly = gradOnly ? 1 : 0;
-            ct_mlp_train_kernel<<<1, kTrainThreads, kTrainSmem, m->stream>>>(A);
+            ct_mlp_train_kernel<<<kTrainCtas, kTrainThreads, sizeof(TrainSmem), m->stream>>>(A);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess && loss_out)
