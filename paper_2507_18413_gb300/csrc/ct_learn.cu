@@ -349,78 +349,58 @@ struct TrainArgs {
 };
 
 // Training runs on one cluster of kTrainCtas CTAs. The passes over the layers
-// are split by samples (CTA r takes the r-th run of the batch, a half-warp per
-// sample, 16 lanes x 4 hidden units, so that the layers need no CTA barrier:
-// the activations a half-warp reads are the ones it wrote); the gradients and
-// Adam by units (CTA r owns units 8r .. 8r + 7 of both layers: their rows of W1
-// and W2, their biases and W3 entries, with the moments in registers). Each
-// half-warp stores what the owners need into their shared memory, and the
-// owners store the new weights into everybody's: two cluster barriers a batch.
+// are split by samples (CTA r takes the r-th run of the batch, a warp per two
+// samples, two units per lane, so that the layers need no CTA barrier: the
+// activations a warp reads are the ones it wrote, and a weight read serves both
+// samples); the gradients and Adam by units (CTA r owns units 8r .. 8r + 7 of
+// both layers: their rows of W1 and W2, their biases and W3 entries, with the
+// moments in registers). Each warp stores what the owners need into their
+// shared memory, and the owners store the new weights into everybody's: two
+// cluster barriers a batch.
 // Every sum runs in one thread over its inputs in order (units 0..63, samples
 // 0..b-1), whatever the split: Adam divides a gradient by its own size, so one
 // that cancels to rounding noise makes a full step, and another order of
 // summation would make another network.
-// What bounds a batch of 128 samples: the shared memory the products read
-// (about 1.2 us for the two 64 x 64 passes, 0.8 us for the gradients), the
-// chains of 64 and 128 dependent FMAs, the exchange and the barriers. W2 is
-// kept in both orders, so that the forward and the backward pass both read
-// consecutive 128-bit words (one order made every read of the other a 32-way
-// bank conflict: one CTA took 115 us per batch of 128).
+// What bounds a batch of 128 samples: the shared memory the products read, the
+// chains of 64 and 128 dependent FMAs, the exchange and the barriers. Rows of
+// W1 and W2 are padded so that the lanes' 128-bit reads of their units' rows
+// (forward) and the consecutive reads of one row (backward) are both free of
+// bank conflicts (unpadded, one of them is a 32-way conflict: one CTA took
+// 115 us per batch of 128; a half-warp per sample with W2 in both orders, the
+// second order's stores scattered over the cluster, 9.9 us).
 constexpr int kTrainThreads = 256;
 constexpr int kTrainCtas = 8;
 constexpr int kTrainSamples = kTrainBatch / kTrainCtas;  // per CTA and batch
 constexpr int kOwnU = kNH / kTrainCtas;                  // units a CTA owns
-constexpr int kRow = kNH + 4;                            // padded activation row (two samples of a warp: other banks)
+constexpr int kRow = kNH + 4;                            // padded rows of 64
+constexpr int kRow1 = kNF + 4;                           // padded W1 rows
 static_assert(kTrainSamples * 16 == kTrainThreads && kNH == 64 && kNF == 8 && kOwnU == 8,
-              "a half-warp per sample, 4 units per lane, 8 units per CTA");
+              "a warp per two samples, two units per lane, 8 units per CTA");
 
 struct TrainSmem {
-    float w2[kNH * kNH];       // [j][i]: unit j of layer 2, input i
-    float w2t[kNH * kNH];      // [i][j]
-    float w1t[kNF * kNH];      // [i][j]
+    float w2[kNH * kRow];      // [j][i]: unit j of layer 2, input i
+    float w1[kNH * kRow1];     // [j][i]
     float b1[kNH], b2[kNH], w3[kNH];
     // the whole batch, written by the CTAs that hold the samples
-    float h1[kTrainBatch * kRow];   // layer-1 activations
+    float h1[kTrainBatch * kNH];    // layer-1 activations
     float x[kTrainBatch * kNF];
     float d1o[kTrainBatch * kOwnU], d2o[kTrainBatch * kOwnU], h2o[kTrainBatch * kOwnU];  // of the owned units
     float dout[kTrainBatch], sq[kTrainBatch];
     // the CTA's own samples
-    float h2[kTrainSamples * kRow], d2[kTrainSamples * kRow];
+    float rx[kTrainSamples * kNF], r1[kTrainSamples * kNH], r2[kTrainSamples * kNH], rd[kTrainSamples * kNH];
+    float gw[kOwnU * kNH];  // gradient of the owned W2 rows
     float c[2][2];  // Adam's bias corrections of a batch, by batch parity
     float b3;
 };
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 __device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ void st2(float* p, const float2& v) { *reinterpret_cast<float2*>(p) = v; }
 
-__device__ __forceinline__ void fma4(float4& a, float s, const float4& v) {
-    a.x = fmaf(s, v.x, a.x);
-    a.y = fmaf(s, v.y, a.y);
-    a.z = fmaf(s, v.z, a.z);
-    a.w = fmaf(s, v.w, a.w);
-}
-
-__device__ __forceinline__ float4 relu4(const float4& v) {
-    return make_float4(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f), fmaxf(v.z, 0.0f), fmaxf(v.w, 0.0f));
-}
-
-__device__ __forceinline__ float4 keep4(const float4& on, const float4& v) {
-    return make_float4(on.x > 0.0f ? v.x : 0.0f, on.y > 0.0f ? v.y : 0.0f, on.z > 0.0f ? v.z : 0.0f,
-                       on.w > 0.0f ? v.w : 0.0f);
-}
-
-// acc + sum_k row[k] * M[k][4q .. 4q+3], k ascending (the row broadcast to the
-// half-warp, M's rows read as consecutive float4 by its lanes).
-__device__ __forceinline__ float4 row_times(const float* row, const float* M, int q, float4 acc) {
-#pragma unroll 4
-    for (int k = 0; k < kNH; k += 4) {
-        const float4 r = ld4(row + k);
-        fma4(acc, r.x, ld4(M + (k + 0) * kNH + 4 * q));
-        fma4(acc, r.y, ld4(M + (k + 1) * kNH + 4 * q));
-        fma4(acc, r.z, ld4(M + (k + 2) * kNH + 4 * q));
-        fma4(acc, r.w, ld4(M + (k + 3) * kNH + 4 * q));
-    }
-    return acc;
+// acc + a . b over the four components, in order
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
 }
 
 __device__ __forceinline__ void adam(float& w, float& m, float& v, float g, float lr, float c1, float c2) {
@@ -437,17 +417,13 @@ ct_mlp_train_kernel(const TrainArgs A) {
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(s_train);
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int rank = (int)cluster.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, half = lane >> 4, q = lane & 15;
-    const int sl = (tid >> 5) * 2 + half;  // the half-warp's sample in the CTA
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = lane >> 4, q = lane & 15;
+    const int sl = warp * 2 + half;  // the sample in the CTA a half-warp fetches and sends
     TrainSmem* peer[kTrainCtas];
 #pragma unroll
     for (int r = 0; r < kTrainCtas; ++r) peer[r] = cluster.map_shared_rank(&S, r);
-    for (int e = tid; e < kNH * kNH; e += kTrainThreads) {
-        const float u = A.w[oW2 + e];
-        S.w2[e] = u;
-        S.w2t[(e % kNH) * kNH + e / kNH] = u;
-    }
-    for (int e = tid; e < kNH * kNF; e += kTrainThreads) S.w1t[(e % kNF) * kNH + e / kNF] = A.w[oW1 + e];
+    for (int e = tid; e < kNH * kNH; e += kTrainThreads) S.w2[(e / kNH) * kRow + e % kNH] = A.w[oW2 + e];
+    for (int e = tid; e < kNH * kNF; e += kTrainThreads) S.w1[(e / kNF) * kRow1 + e % kNF] = A.w[oW1 + e];
     if (tid < kNH) {
         S.b1[tid] = A.w[oB1 + tid];
         S.b2[tid] = A.w[oB2 + tid];
@@ -459,23 +435,27 @@ ct_mlp_train_kernel(const TrainArgs A) {
         S.c[0][1] = 1.0f - powf(0.999f, (float)(A.t0 + 1));
     }
     for (int e = tid; e < kTrainBatch; e += kTrainThreads) S.sq[e] = 0.0f;
-    // The entries a thread owns: threads 0..127 four consecutive inputs of one
-    // W2 row, 128..191 a W1 entry, 192..215 a bias or W3 entry, 216 (CTA 0) b3.
-    const int uj = tid < 128 ? tid >> 4 : tid < 192 ? (tid - 128) / kNF : (tid - 192) & 7;  // owned unit
-    const int unit = rank * kOwnU + uj;
-    const int ui = tid < 128 ? 4 * (tid & 15) : (tid - 128) % kNF;  // its (first) input
-    const int nOwn = tid < 128 ? 4 : (tid < 216 || (tid == 216 && rank == 0)) ? 1 : 0;
-    const int e0 = tid < 128 ? oW2 + unit * kNH + ui
-                   : tid < 192 ? oW1 + unit * kNF + ui
-                   : tid < 200 ? oB1 + unit
-                   : tid < 208 ? oB2 + unit
-                   : tid < 216 ? oW3 + unit : oB3;
-    float w[4], m[4], v[4];
+    // The entries a thread owns: inputs 2 * lane, 2 * lane + 1 of the W2 row of
+    // owned unit `warp` (0, 1), and one more (2) in warps 2, 3 (a W1 entry per
+    // lane) and 4 (b1, b2, W3 of the owned units, 8 lanes each; b3 in CTA 0).
+    // (All of Adam on the two warps that sum the W2 gradients, 8 entries a
+    // thread, made 11,400 of a batch's 20,700 cycles: its divisions follow one
+    // another.)
+    const int uj = warp < 4 ? (tid & 63) / kNF : lane & 7;  // the extra entry's owned unit and input
+    const int unit = rank * kOwnU + uj, ui = lane % kNF;
+    const bool extra = warp == 2 || warp == 3 || (warp == 4 && (lane < 24 || (lane == 24 && rank == 0)));
+    const int ex = warp < 4 ? oW1 + unit * kNF + ui
+                   : lane < 8 ? oB1 + unit
+                   : lane < 16 ? oB2 + unit
+                   : lane < 24 ? oW3 + unit : oB3;
+    auto entry = [&](int k) { return k < 2 ? oW2 + (rank * kOwnU + warp) * kNH + 2 * lane + k : ex; };
+    float w[3], m[3], v[3];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        w[k] = k < nOwn ? A.w[e0 + k] : 0.0f;
-        m[k] = k < nOwn ? A.m[e0 + k] : 0.0f;
-        v[k] = k < nOwn ? A.v[e0 + k] : 0.0f;
+    for (int k = 0; k < 3; ++k) {
+        const bool own = k < 2 || extra;
+        w[k] = own ? A.w[entry(k)] : 0.0f;
+        m[k] = own ? A.m[entry(k)] : 0.0f;
+        v[k] = own ? A.v[entry(k)] : 0.0f;
     }
     const int epochs = A.gradOnly ? 1 : A.epochs;
     const int nUse = A.gradOnly ? min(A.n, A.batch) : A.n;
@@ -512,7 +492,7 @@ ct_mlp_train_kernel(const TrainArgs A) {
         if (total > 1) idxN = sample_of(ep2, pos2, bN, perN);
     }
     cluster.sync();  // every CTA runs: its shared memory may be written
-    float lossSum = 0.0f;  // CTA 0, thread 224
+    float lossSum = 0.0f;  // CTA 0, last warp
     int pos = 0, ep = 0;
     for (long long kb = 0; kb < total; ++kb) {
         // next batch's sample, and the one after's index
@@ -525,115 +505,140 @@ ct_mlp_train_kernel(const TrainArgs A) {
         int b2n = 0, per2n = 0, idx2 = -1;
         advance();
         if (kb + 2 < total) idx2 = sample_of(ep2, pos2, b2n, per2n);
-        if ((tid >> 5) * 2 < per) {
-            const int sg = valid ? rank * per + sl : 0;  // the sample in the batch
-            // layer 1: units 4q .. 4q+3
-            float4 h = ld4(S.b1 + 4 * q);
+        if (warp * 2 < per) {
+            const int sg = valid ? rank * per + sl : 0;  // the half-warp's sample in the batch
+            float* x0 = S.rx + warp * 2 * kNF;           // the warp's two samples: rows 0 and 1
+            float* h0 = S.r1 + warp * 2 * kNH;
+            float* z0 = S.r2 + warp * 2 * kNH;
+            float* d0 = S.rd + warp * 2 * kNH;
+            if (q < kNF) x0[half * kNF + q] = xv;
+            __syncwarp();
+            // layer 1: units lane and lane + 32 of both samples
+            float a[2][2];  // [unit][sample]
+            {
+                const float4 xa = ld4(x0), xb = ld4(x0 + 4), xc = ld4(x0 + 8), xd = ld4(x0 + 12);
 #pragma unroll
-            for (int i = 0; i < kNF; ++i) fma4(h, __shfl_sync(0xffffffffu, xv, (half << 4) + i), ld4(S.w1t + i * kNH + 4 * q));
-            h = relu4(h);
-            float* own2 = S.h2 + sl * kRow;
-            st4(own2 + 4 * q, h);  // (the row holds layer 1 until layer 2 is done)
+                for (int u = 0; u < 2; ++u) {
+                    const int j = lane + 32 * u;
+                    const float4 wa = ld4(S.w1 + j * kRow1), wb = ld4(S.w1 + j * kRow1 + 4);
+                    a[u][0] = fmaxf(dot4(wb, xb, dot4(wa, xa, S.b1[j])), 0.0f);
+                    a[u][1] = fmaxf(dot4(wb, xd, dot4(wa, xc, S.b1[j])), 0.0f);
+                    h0[j] = a[u][0];
+                    h0[kNH + j] = a[u][1];
+                }
+            }
             __syncwarp();
-            float4 z = relu4(row_times(own2, S.w2t, q, ld4(S.b2 + 4 * q)));
+            // layer 2
+            float z[2][2];
+            z[0][0] = z[0][1] = S.b2[lane];
+            z[1][0] = z[1][1] = S.b2[lane + 32];
+#pragma unroll 4
+            for (int i = 0; i < kNH; i += 4) {
+                const float4 ha = ld4(h0 + i), hb = ld4(h0 + kNH + i);
+                const float4 wa = ld4(S.w2 + lane * kRow + i), wb = ld4(S.w2 + (lane + 32) * kRow + i);
+                z[0][0] = dot4(wa, ha, z[0][0]);
+                z[0][1] = dot4(wa, hb, z[0][1]);
+                z[1][0] = dot4(wb, ha, z[1][0]);
+                z[1][1] = dot4(wb, hb, z[1][1]);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    z[u][t] = fmaxf(z[u][t], 0.0f);
+                    z0[t * kNH + lane + 32 * u] = z[u][t];
+                }
             __syncwarp();
-            st4(own2 + 4 * q, z);
-            __syncwarp();
-            // the output by one lane, units in order
+            // the outputs, units in order: lanes 0 and 16 a sample each
             float o = S.b3;
             if (q == 0) {
 #pragma unroll 4
-                for (int j = 0; j < kNH; j += 4) {
-                    const float4 c = ld4(S.w3 + j), g = ld4(own2 + j);
-                    o = fmaf(c.x, g.x, o);
-                    o = fmaf(c.y, g.y, o);
-                    o = fmaf(c.z, g.z, o);
-                    o = fmaf(c.w, g.w, o);
+                for (int j = 0; j < kNH; j += 4) o = dot4(ld4(S.w3 + j), ld4(z0 + half * kNH + j), o);
+            }
+            const float r = __shfl_sync(0xffffffffu, o, half << 4) - yv, dz = r / (float)b;
+            const float dz0 = __shfl_sync(0xffffffffu, dz, 0), dz1 = __shfl_sync(0xffffffffu, dz, 16);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int j = lane + 32 * u;
+                const float c = S.w3[j];
+                d0[j] = z[u][0] > 0.0f ? dz0 * c : 0.0f;
+                d0[kNH + j] = z[u][1] > 0.0f ? dz1 * c : 0.0f;
+            }
+            __syncwarp();
+            // dL/dz1 of inputs 2 * lane, 2 * lane + 1
+            float2 ga = make_float2(0.0f, 0.0f), gb = ga;
+#pragma unroll 4
+            for (int j = 0; j < kNH; j += 4) {
+                const float4 da = ld4(d0 + j), db = ld4(d0 + kNH + j);
+                const float fa[4] = {da.x, da.y, da.z, da.w}, fb[4] = {db.x, db.y, db.z, db.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float2 ww = ld2(S.w2 + (j + k) * kRow + 2 * lane);
+                    ga.x = fmaf(fa[k], ww.x, ga.x);
+                    ga.y = fmaf(fa[k], ww.y, ga.y);
+                    gb.x = fmaf(fb[k], ww.x, gb.x);
+                    gb.y = fmaf(fb[k], ww.y, gb.y);
                 }
             }
-            o = __shfl_sync(0xffffffffu, o, half << 4);
-            const float r = o - yv, dz = r / (float)b;
-            const float4 c = ld4(S.w3 + 4 * q);
-            const float4 d2 = keep4(z, make_float4(dz * c.x, dz * c.y, dz * c.z, dz * c.w));
-            float* rowD = S.d2 + sl * kRow;
-            st4(rowD + 4 * q, d2);
+            const float4 hs = ld4(h0 + half * kNH + 4 * q), zs = ld4(z0 + half * kNH + 4 * q),
+                         ds = ld4(d0 + half * kNH + 4 * q);
+            const float2 ha = ld2(h0 + 2 * lane), hb = ld2(h0 + kNH + 2 * lane);
+            __syncwarp();  // (dL/dz2 is read: its rows take dL/dz1)
+            st2(d0 + 2 * lane, make_float2(ha.x > 0.0f ? ga.x : 0.0f, ha.y > 0.0f ? ga.y : 0.0f));
+            st2(d0 + kNH + 2 * lane, make_float2(hb.x > 0.0f ? gb.x : 0.0f, hb.y > 0.0f ? gb.y : 0.0f));
             __syncwarp();
-            const float4 d1 = keep4(h, row_times(rowD, S.w2, q, make_float4(0.0f, 0.0f, 0.0f, 0.0f)));
             if (valid) {
                 // to every CTA: layer 1, the inputs, dL/dout; to a unit's owner: its activation and gradients
 #pragma unroll
                 for (int p = 0; p < kTrainCtas; ++p) {
-                    st4(peer[p]->h1 + sg * kRow + 4 * q, h);
+                    st4(peer[p]->h1 + sg * kNH + 4 * q, hs);
                     if (q < kNF) peer[p]->x[sg * kNF + q] = xv;
                     if (q == 0) peer[p]->dout[sg] = dz;
                 }
                 TrainSmem* own = cluster.map_shared_rank(&S, q >> 1);
                 const int at = sg * kOwnU + 4 * (q & 1);
-                st4(own->d1o + at, d1);
-                st4(own->d2o + at, d2);
-                st4(own->h2o + at, z);
+                st4(own->d1o + at, ld4(d0 + half * kNH + 4 * q));
+                st4(own->d2o + at, ds);
+                st4(own->h2o + at, zs);
                 if (q == 0) peer[0]->sq[sg] = r * r;
             }
         }
         cluster.sync();
         // the owned entries: gradient over the batch (samples in order), Adam
         const float c1 = S.c[kb & 1][0], c2 = S.c[kb & 1][1];
-        if (tid < 128) {
-            float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float ge = 0.0f;
+        if (warp < 2) {
+            // four owned W2 rows, two inputs per lane
+            float g[4][2] = {};
 #pragma unroll 8
-            for (int s = 0; s < b; ++s) fma4(g, S.d2o[s * kOwnU + uj], ld4(S.h1 + s * kRow + ui));
-            if (A.gradOnly) {
-                A.grad[e0] = g.x;
-                A.grad[e0 + 1] = g.y;
-                A.grad[e0 + 2] = g.z;
-                A.grad[e0 + 3] = g.w;
-            } else {
-                adam(w[0], m[0], v[0], g.x, A.lr, c1, c2);
-                adam(w[1], m[1], v[1], g.y, A.lr, c1, c2);
-                adam(w[2], m[2], v[2], g.z, A.lr, c1, c2);
-                adam(w[3], m[3], v[3], g.w, A.lr, c1, c2);
-#pragma unroll
-                for (int p = 0; p < kTrainCtas; ++p) {
-                    st4(peer[p]->w2 + unit * kNH + ui, make_float4(w[0], w[1], w[2], w[3]));
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) peer[p]->w2t[(ui + k) * kNH + unit] = w[k];
-                }
+            for (int s = 0; s < b; ++s) {
+                const float4 d = ld4(S.d2o + s * kOwnU + 4 * warp);
+                const float2 h = ld2(S.h1 + s * kNH + 2 * lane);
+                g[0][0] = fmaf(d.x, h.x, g[0][0]);
+                g[0][1] = fmaf(d.x, h.y, g[0][1]);
+                g[1][0] = fmaf(d.y, h.x, g[1][0]);
+                g[1][1] = fmaf(d.y, h.y, g[1][1]);
+                g[2][0] = fmaf(d.z, h.x, g[2][0]);
+                g[2][1] = fmaf(d.z, h.y, g[2][1]);
+                g[3][0] = fmaf(d.w, h.x, g[3][0]);
+                g[3][1] = fmaf(d.w, h.y, g[3][1]);
             }
-        } else if (nOwn) {
-            float g = 0.0f;
-            if (tid < 192) {
-#pragma unroll 8
-                for (int s = 0; s < b; ++s) g = fmaf(S.d1o[s * kOwnU + uj], S.x[s * kNF + ui], g);
-            } else if (tid < 208) {
-                const float* d = tid < 200 ? S.d1o : S.d2o;
-#pragma unroll 8
-                for (int s = 0; s < b; ++s) g += d[s * kOwnU + uj];
-            } else if (tid < 216) {
-#pragma unroll 8
-                for (int s = 0; s < b; ++s) g = fmaf(S.dout[s], S.h2o[s * kOwnU + uj], g);
-            } else {
-#pragma unroll 8
-                for (int s = 0; s < b; ++s) g += S.dout[s];
-            }
-            if (A.gradOnly) {
-                A.grad[e0] = g;
-            } else {
-                adam(w[0], m[0], v[0], g, A.lr, c1, c2);
 #pragma unroll
-                for (int p = 0; p < kTrainCtas; ++p) {
-                    TrainSmem* P = peer[p];
-                    float* at = tid < 192 ? &P->w1t[ui * kNH + unit]
-                                : tid < 200 ? &P->b1[unit]
-                                : tid < 208 ? &P->b2[unit]
-                                : tid < 216 ? &P->w3[unit] : &P->b3;
-                    *at = w[0];
-                }
-            }
-        } else if (tid >= 224) {
-            // the last warp: the batch's loss (CTA 0, a binary tree over the
-            // samples), the next batch's bias corrections
+            for (int k = 0; k < 4; ++k) st2(S.gw + (4 * warp + k) * kNH + 2 * lane, make_float2(g[k][0], g[k][1]));
+        } else if (warp < 4) {
+#pragma unroll 8
+            for (int s = 0; s < b; ++s) ge = fmaf(S.d1o[s * kOwnU + uj], S.x[s * kNF + ui], ge);
+        } else if (warp == 4) {
+            // b1, b2: sums of the units' gradients; W3: of dL/dout times the activation; b3: of dL/dout
+            const float* f = lane < 8 ? S.d1o + uj : lane < 16 ? S.d2o + uj : lane < 24 ? S.h2o + uj : S.dout;
+            const int step = lane < 24 ? kOwnU : 1;
+            const bool times = lane >= 16 && lane < 24;
+#pragma unroll 8
+            for (int s = 0; s < b; ++s) ge = fmaf(times ? S.dout[s] : 1.0f, f[s * step], ge);
+        } else if (warp == kTrainThreads / 32 - 1) {
+            // the batch's loss (CTA 0, a binary tree over the samples), the next batch's bias corrections
             if (rank == 0) {
-                float l = lane < 32 ? (S.sq[lane] + S.sq[lane + 64]) + (S.sq[lane + 32] + S.sq[lane + 96]) : 0.0f;
+                float l = (S.sq[lane] + S.sq[lane + 64]) + (S.sq[lane + 32] + S.sq[lane + 96]);
                 __syncwarp();
                 for (int k = 0; k < kTrainBatch; k += 32) S.sq[lane + k] = 0.0f;
 #pragma unroll
@@ -651,6 +656,31 @@ ct_mlp_train_kernel(const TrainArgs A) {
                 S.c[(kb + 1) & 1][lane] = 1.0f - powf(lane == 0 ? 0.9f : 0.999f, t);
             }
         }
+        __syncthreads();
+        const float2 gw = ld2(S.gw + warp * kNH + 2 * lane);
+        if (A.gradOnly) {
+            A.grad[entry(0)] = gw.x;
+            A.grad[entry(1)] = gw.y;
+            if (extra) A.grad[ex] = ge;
+        } else {
+            adam(w[0], m[0], v[0], gw.x, A.lr, c1, c2);
+            adam(w[1], m[1], v[1], gw.y, A.lr, c1, c2);
+#pragma unroll
+            for (int p = 0; p < kTrainCtas; ++p)
+                st2(peer[p]->w2 + (rank * kOwnU + warp) * kRow + 2 * lane, make_float2(w[0], w[1]));
+            if (extra) {
+                adam(w[2], m[2], v[2], ge, A.lr, c1, c2);
+#pragma unroll
+                for (int p = 0; p < kTrainCtas; ++p) {
+                    TrainSmem* P = peer[p];
+                    float* at = warp < 4 ? &P->w1[unit * kRow1 + ui]
+                                : lane < 8 ? &P->b1[unit]
+                                : lane < 16 ? &P->b2[unit]
+                                : lane < 24 ? &P->w3[unit] : &P->b3;
+                    *at = w[2];
+                }
+            }
+        }
         cluster.sync();
         xv = xN;
         yv = yN;
@@ -666,10 +696,13 @@ ct_mlp_train_kernel(const TrainArgs A) {
         }
     }
     if (A.gradOnly) return;
-    for (int k = 0; k < nOwn; ++k) {
-        A.w[e0 + k] = w[k];
-        A.m[e0 + k] = m[k];
-        A.v[e0 + k] = v[k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (k < 2 || extra) {
+            A.w[entry(k)] = w[k];
+            A.m[entry(k)] = m[k];
+            A.v[entry(k)] = v[k];
+        }
     }
 }
 
