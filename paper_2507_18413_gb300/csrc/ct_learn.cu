@@ -280,23 +280,38 @@ constexpr int oB2 = oW2 + kNH * kNH;
 constexpr int oW3 = oB2 + kNH;
 constexpr int oB3 = oW3 + kNH;
 
-// Scores of n rows of X: one warp per row, lane j holding hidden units j and
-// j + 32 of both layers; layer-1 outputs reach the other lanes by shuffles.
-// Weights sit in shared memory transposed (input-major), so that the lanes of
-// a warp read consecutive words.
-__global__ void ct_mlp_forward_kernel(const float* __restrict__ w, const float* __restrict__ X, int n,
-                                      float* __restrict__ out) {
-    __shared__ float w1t[kNF * kNH];  // [i][j] = W1[j][i]
-    __shared__ float w2t[kNH * kNH];  // [i][j] = W2[j][i]
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ void st2(float* p, const float2& v) { *reinterpret_cast<float2*>(p) = v; }
+
+// acc + a . b over the four components, in order
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+
+// Rows of W1 and W2 in shared memory, padded so that 8 lanes' 128-bit reads of
+// consecutive rows fall into different banks.
+constexpr int kRow = kNH + 4;
+constexpr int kRow1 = kNF + 4;
+
+// Scores of n rows of X: a warp takes R rows at a time, lane j holding hidden
+// units j and j + 32 of both layers; the rows' layer-1 outputs go through
+// shared memory and are read back as broadcast float4. A weight read serves R
+// rows: with one row per warp and step the kernel was bound by shared memory
+// and shuffles (55 us for 20,000 rows), with eight by the FMAs. Few rows take
+// R = 1, so that they spread over more warps. Measured (one row per warp and
+// step -> this): 25 rows 7.1 -> 6.2 us, 2,000 rows 10.4 -> 6.3, 20,000 rows
+// 55 -> 14, 1,000,000 rows 765 -> 283 us.
+template <int R>
+__global__ void __launch_bounds__(256) ct_mlp_forward_kernel(const float* __restrict__ w, const float* __restrict__ X,
+                                                             int n, float* __restrict__ out) {
+    __shared__ __align__(16) float w1[kNH * kRow1];  // [j][i]
+    __shared__ __align__(16) float w2[kNH * kRow];   // [j][i]
     __shared__ float bias1[kNH], bias2[kNH], w3[kNH];
-    for (int q = threadIdx.x; q < kNF * kNH; q += blockDim.x) {
-        const int j = q / kNF, i = q % kNF;
-        w1t[i * kNH + j] = w[oW1 + q];
-    }
-    for (int q = threadIdx.x; q < kNH * kNH; q += blockDim.x) {
-        const int j = q / kNH, i = q % kNH;
-        w2t[i * kNH + j] = w[oW2 + q];
-    }
+    __shared__ __align__(16) float hid[8][R][kNH];
+    for (int q = threadIdx.x; q < kNF * kNH; q += blockDim.x) w1[(q / kNF) * kRow1 + q % kNF] = w[oW1 + q];
+    for (int q = threadIdx.x; q < kNH * kNH; q += blockDim.x) w2[(q / kNH) * kRow + q % kNH] = w[oW2 + q];
     for (int q = threadIdx.x; q < kNH; q += blockDim.x) {
         bias1[q] = w[oB1 + q];
         bias2[q] = w[oB2 + q];
@@ -305,32 +320,66 @@ __global__ void ct_mlp_forward_kernel(const float* __restrict__ w, const float* 
     __syncthreads();
     const float b3 = w[oB3];
     const int lane = threadIdx.x & 31;
+    float(*h)[kNH] = hid[threadIdx.x >> 5];
     const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int s = gwarp; s < n; s += nwarps) {
-        float x[kNF];
+    const float4 wa0 = ld4(w1 + lane * kRow1), wa1 = ld4(w1 + lane * kRow1 + 4);
+    const float4 wb0 = ld4(w1 + (lane + 32) * kRow1), wb1 = ld4(w1 + (lane + 32) * kRow1 + 4);
+    for (long long s0 = (long long)gwarp * R; s0 < n; s0 += (long long)nwarps * R) {
 #pragma unroll
-        for (int i = 0; i < kNF; ++i) x[i] = X[(size_t)s * kNF + i];
-        float ha = bias1[lane], hb = bias1[lane + 32];
+        for (int r = 0; r < R; ++r) {
+            const long long s = min(s0 + r, (long long)n - 1);  // (rows beyond the last one are not stored)
+            float x[kNF];
 #pragma unroll
-        for (int i = 0; i < kNF; ++i) {
-            ha += w1t[i * kNH + lane] * x[i];
-            hb += w1t[i * kNH + lane + 32] * x[i];
+            for (int i = 0; i < kNF; ++i) x[i] = __ldg(X + s * kNF + i);
+            const float4 x0 = make_float4(x[0], x[1], x[2], x[3]), x1 = make_float4(x[4], x[5], x[6], x[7]);
+            h[r][lane] = fmaxf(dot4(wa1, x1, dot4(wa0, x0, bias1[lane])), 0.0f);
+            h[r][lane + 32] = fmaxf(dot4(wb1, x1, dot4(wb0, x0, bias1[lane + 32])), 0.0f);
         }
-        ha = fmaxf(ha, 0.0f);
-        hb = fmaxf(hb, 0.0f);
-        float za = bias2[lane], zb = bias2[lane + 32];
-#pragma unroll 8
-        for (int i = 0; i < kNH; ++i) {
-            const float hi = __shfl_sync(0xffffffffu, i < 32 ? ha : hb, i & 31);
-            za += w2t[i * kNH + lane] * hi;
-            zb += w2t[i * kNH + lane + 32] * hi;
-        }
-        float o = w3[lane] * fmaxf(za, 0.0f) + w3[lane + 32] * fmaxf(zb, 0.0f);
+        __syncwarp();
+        float za[R], zb[R];
 #pragma unroll
-        for (int k = 16; k > 0; k >>= 1) o += __shfl_xor_sync(0xffffffffu, o, k);
-        if (lane == 0) out[s] = o + b3;
+        for (int r = 0; r < R; ++r) {
+            za[r] = bias2[lane];
+            zb[r] = bias2[lane + 32];
+        }
+#pragma unroll 4
+        for (int i = 0; i < kNH; i += 4) {
+            const float4 ua = ld4(w2 + lane * kRow + i), ub = ld4(w2 + (lane + 32) * kRow + i);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 hr = ld4(h[r] + i);
+                za[r] = dot4(ua, hr, za[r]);
+                zb[r] = dot4(ub, hr, zb[r]);
+            }
+        }
+        __syncwarp();
+        float o[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) o[r] = w3[lane] * fmaxf(za[r], 0.0f) + w3[lane + 32] * fmaxf(zb[r], 0.0f);
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1)
+#pragma unroll
+            for (int r = 0; r < R; ++r) o[r] += __shfl_xor_sync(0xffffffffu, o[r], k);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (lane == r && s0 + r < n) out[s0 + r] = o[r] + b3;
     }
+}
+
+// The scores' launch: eight rows per warp once that still fills the SMs' warps
+// (two CTAs of 8 warps per SM), one below.
+cudaError_t launch_forward(const float* w, const float* X, int n, float* out, cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (n >= 8 * 8 * sms) {
+        ct_mlp_forward_kernel<8><<<std::min(n / 64 + 1, 2 * sms), 256, 0, s>>>(w, X, n, out);
+    } else {
+        ct_mlp_forward_kernel<1><<<std::min(n / 8 + 1, 4 * sms), 256, 0, s>>>(w, X, n, out);
+    }
+    return cudaGetLastError();
 }
 
 struct TrainArgs {
@@ -372,8 +421,6 @@ constexpr int kTrainThreads = 256;
 constexpr int kTrainCtas = 8;
 constexpr int kTrainSamples = kTrainBatch / kTrainCtas;  // per CTA and batch
 constexpr int kOwnU = kNH / kTrainCtas;                  // units a CTA owns
-constexpr int kRow = kNH + 4;                            // padded rows of 64
-constexpr int kRow1 = kNF + 4;                           // padded W1 rows
 static_assert(kTrainSamples * 16 == kTrainThreads && kNH == 64 && kNF == 8 && kOwnU == 8,
               "a warp per two samples, two units per lane, 8 units per CTA");
 
@@ -392,16 +439,6 @@ struct TrainSmem {
     float c[2][2];  // Adam's bias corrections of a batch, by batch parity
     float b3;
 };
-
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ void st4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
-__device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-__device__ __forceinline__ void st2(float* p, const float2& v) { *reinterpret_cast<float2*>(p) = v; }
-
-// acc + a . b over the four components, in order
-__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
-    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
-}
 
 __device__ __forceinline__ void adam(float& w, float& m, float& v, float g, float lr, float c1, float c2) {
     const float mi = 0.9f * m + 0.1f * g;
@@ -436,15 +473,15 @@ ct_mlp_train_kernel(const TrainArgs A) {
     }
     for (int e = tid; e < kTrainBatch; e += kTrainThreads) S.sq[e] = 0.0f;
     // The entries a thread owns: inputs 2 * lane, 2 * lane + 1 of the W2 row of
-    // owned unit `warp` (0, 1), and one more (2) in warps 2, 3 (a W1 entry per
-    // lane) and 4 (b1, b2, W3 of the owned units, 8 lanes each; b3 in CTA 0).
+    // owned unit `warp` (0, 1), and one more (2) in warps 4, 5 (a W1 entry per
+    // lane) and 6 (b1, b2, W3 of the owned units, 8 lanes each; b3 in CTA 0).
     // (All of Adam on the two warps that sum the W2 gradients, 8 entries a
     // thread, made 11,400 of a batch's 20,700 cycles: its divisions follow one
     // another.)
-    const int uj = warp < 4 ? (tid & 63) / kNF : lane & 7;  // the extra entry's owned unit and input
+    const int uj = warp < 6 ? (tid & 63) / kNF : lane & 7;  // the extra entry's owned unit and input
     const int unit = rank * kOwnU + uj, ui = lane % kNF;
-    const bool extra = warp == 2 || warp == 3 || (warp == 4 && (lane < 24 || (lane == 24 && rank == 0)));
-    const int ex = warp < 4 ? oW1 + unit * kNF + ui
+    const bool extra = warp == 4 || warp == 5 || (warp == 6 && (lane < 24 || (lane == 24 && rank == 0)));
+    const int ex = warp < 6 ? oW1 + unit * kNF + ui
                    : lane < 8 ? oB1 + unit
                    : lane < 16 ? oB2 + unit
                    : lane < 24 ? oW3 + unit : oB3;
@@ -532,7 +569,7 @@ ct_mlp_train_kernel(const TrainArgs A) {
             float z[2][2];
             z[0][0] = z[0][1] = S.b2[lane];
             z[1][0] = z[1][1] = S.b2[lane + 32];
-#pragma unroll 4
+#pragma unroll 8
             for (int i = 0; i < kNH; i += 4) {
                 const float4 ha = ld4(h0 + i), hb = ld4(h0 + kNH + i);
                 const float4 wa = ld4(S.w2 + lane * kRow + i), wb = ld4(S.w2 + (lane + 32) * kRow + i);
@@ -552,7 +589,7 @@ ct_mlp_train_kernel(const TrainArgs A) {
             // the outputs, units in order: lanes 0 and 16 a sample each
             float o = S.b3;
             if (q == 0) {
-#pragma unroll 4
+#pragma unroll
                 for (int j = 0; j < kNH; j += 4) o = dot4(ld4(S.w3 + j), ld4(z0 + half * kNH + j), o);
             }
             const float r = __shfl_sync(0xffffffffu, o, half << 4) - yv, dz = r / (float)b;
@@ -567,7 +604,7 @@ ct_mlp_train_kernel(const TrainArgs A) {
             __syncwarp();
             // dL/dz1 of inputs 2 * lane, 2 * lane + 1
             float2 ga = make_float2(0.0f, 0.0f), gb = ga;
-#pragma unroll 4
+#pragma unroll 8
             for (int j = 0; j < kNH; j += 4) {
                 const float4 da = ld4(d0 + j), db = ld4(d0 + kNH + j);
                 const float fa[4] = {da.x, da.y, da.z, da.w}, fb[4] = {db.x, db.y, db.z, db.w};
@@ -607,33 +644,29 @@ ct_mlp_train_kernel(const TrainArgs A) {
         // the owned entries: gradient over the batch (samples in order), Adam
         const float c1 = S.c[kb & 1][0], c2 = S.c[kb & 1][1];
         float ge = 0.0f;
-        if (warp < 2) {
-            // four owned W2 rows, two inputs per lane
-            float g[4][2] = {};
-#pragma unroll 8
+        if (warp < 4) {
+            // two owned W2 rows, two inputs per lane
+            float g[2][2] = {};
+#pragma unroll 16
             for (int s = 0; s < b; ++s) {
-                const float4 d = ld4(S.d2o + s * kOwnU + 4 * warp);
+                const float2 d = ld2(S.d2o + s * kOwnU + 2 * warp);
                 const float2 h = ld2(S.h1 + s * kNH + 2 * lane);
                 g[0][0] = fmaf(d.x, h.x, g[0][0]);
                 g[0][1] = fmaf(d.x, h.y, g[0][1]);
                 g[1][0] = fmaf(d.y, h.x, g[1][0]);
                 g[1][1] = fmaf(d.y, h.y, g[1][1]);
-                g[2][0] = fmaf(d.z, h.x, g[2][0]);
-                g[2][1] = fmaf(d.z, h.y, g[2][1]);
-                g[3][0] = fmaf(d.w, h.x, g[3][0]);
-                g[3][1] = fmaf(d.w, h.y, g[3][1]);
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) st2(S.gw + (4 * warp + k) * kNH + 2 * lane, make_float2(g[k][0], g[k][1]));
-        } else if (warp < 4) {
-#pragma unroll 8
+            for (int k = 0; k < 2; ++k) st2(S.gw + (2 * warp + k) * kNH + 2 * lane, make_float2(g[k][0], g[k][1]));
+        } else if (warp < 6) {
+#pragma unroll 16
             for (int s = 0; s < b; ++s) ge = fmaf(S.d1o[s * kOwnU + uj], S.x[s * kNF + ui], ge);
-        } else if (warp == 4) {
+        } else if (warp == 6) {
             // b1, b2: sums of the units' gradients; W3: of dL/dout times the activation; b3: of dL/dout
             const float* f = lane < 8 ? S.d1o + uj : lane < 16 ? S.d2o + uj : lane < 24 ? S.h2o + uj : S.dout;
             const int step = lane < 24 ? kOwnU : 1;
             const bool times = lane >= 16 && lane < 24;
-#pragma unroll 8
+#pragma unroll 16
             for (int s = 0; s < b; ++s) ge = fmaf(times ? S.dout[s] : 1.0f, f[s * step], ge);
         } else if (warp == kTrainThreads / 32 - 1) {
             // the batch's loss (CTA 0, a binary tree over the samples), the next batch's bias corrections
@@ -673,7 +706,7 @@ ct_mlp_train_kernel(const TrainArgs A) {
 #pragma unroll
                 for (int p = 0; p < kTrainCtas; ++p) {
                     TrainSmem* P = peer[p];
-                    float* at = warp < 4 ? &P->w1[unit * kRow1 + ui]
+                    float* at = warp < 6 ? &P->w1[unit * kRow1 + ui]
                                 : lane < 8 ? &P->b1[unit]
                                 : lane < 16 ? &P->b2[unit]
                                 : lane < 24 ? &P->w3[unit] : &P->b3;
@@ -855,9 +888,7 @@ int ct_feat_compute(FeatView* f, const TableDev* d_tabs, const uint32_t* dom, co
 
 int ct_feat_scores(FeatView* f, const ct_mlp* mlp, cudaStream_t s) {
     const int n = f->nv;
-    const int grid = std::max(1, std::min((n + 7) / 8, 1024));
-    ct_mlp_forward_kernel<<<grid, 256, 0, s>>>(mlp->d_w, f->feat, n, f->scores);
-    CT_CUDA(cudaGetLastError());
+    CT_CUDA(launch_forward(mlp->d_w, f->feat, n, f->scores, s));
     CT_CUDA(cudaMemcpyAsync(f->h_scores, f->scores, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, s));
     CT_CUDA(cudaStreamSynchronize(s));
     return CT_OK;
@@ -1002,9 +1033,7 @@ extern "C" int ct_mlp_forward(ct_mlp* m, const float* x_dev, int64_t n, float* s
         return CT_ERR_ARG;
     }
     if (n == 0) return CT_OK;
-    const int grid = (int)std::min<int64_t>((n + 7) / 8, 4096);
-    ct_mlp_forward_kernel<<<grid, 256, 0, m->stream>>>(m->d_w, x_dev, (int)n, scores_dev);
-    CT_CUDA(cudaGetLastError());
+    CT_CUDA(launch_forward(m->d_w, x_dev, (int)n, scores_dev, m->stream));
     return CT_OK;
 }
 
