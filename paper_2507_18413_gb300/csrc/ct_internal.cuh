@@ -326,6 +326,17 @@ cudaError_t launch_set_words(uint32_t* dst, const uint32_t* words, int n, cudaSt
 cudaError_t launch_copy_words(uint32_t* dst, const uint32_t* src, int n, cudaStream_t s);
 cudaError_t launch_read_ceiling(const uint4* p, size_t n16, cudaStream_t s);
 
+// Launchers of a table's construction (ct_build.cu). tup: device copies of the
+// tuples from tupleBase (a multiple of 1,024) on; lo, row0: first values and
+// row prefix of the scope. counts: tuples outside the domains, others with a
+// wildcard (added to). last: these are the table's last tuples.
+cudaError_t launch_check_tuples(const int32_t* tup, int64_t t, int n, const int32_t* lo, const int32_t* row0,
+                                unsigned long long* counts, cudaStream_t s);
+cudaError_t launch_build_rows(const int32_t* tup, int64_t tuples, int n, const int32_t* lo, const int32_t* row0,
+                              uint4* sup, uint4* del, int64_t W4, int64_t tupleBase, bool last, cudaStream_t s);
+// currTable, its index and trail links, and the residues (after the rows).
+cudaError_t launch_build_state(const TableDev& T, int64_t t, cudaStream_t s);
+
 }  // namespace ctk
 
 // Test hook of ct_propagate_noalloc (ct_noalloc.cu): the next call on the

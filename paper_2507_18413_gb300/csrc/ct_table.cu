@@ -277,6 +277,62 @@ void free_table(ct_table* ct) {
     delete ct;
 }
 
+// The tuple list on the device while a table is built, with the layout its
+// kernels need: a bounded scratch buffer (kStageInts components; lists beyond it
+// go through in chunks), freed when the construction ends. Not one of the
+// table's buffers.
+struct TupleStage {
+    static constexpr int64_t kStageInts = 1LL << 26;  // 256 MB
+    char* base = nullptr;
+    int32_t* lo = nullptr;
+    int32_t* row0 = nullptr;
+    unsigned long long* counts = nullptr;
+    int32_t* tup = nullptr;
+    int64_t cap = 0;              // tuples per chunk (a multiple of 1,024)
+    const int32_t* held = nullptr;  // host list whose chunk at heldAt is on the device
+    int64_t heldAt = 0;
+    std::vector<int32_t> meta;  // what lo and row0 are copied from (kept until the copy is done)
+    ~TupleStage() {
+        if (base) cudaFree(base);
+    }
+    // Room for t tuples of n components, or as many as memory allows.
+    int open(const ct_table* ct, int64_t t) {
+        const int n = ct->arity;
+        const int64_t whole = (t + 1023) / 1024 * 1024;
+        cap = std::max<int64_t>(1024, std::min(whole, kStageInts / n / 1024 * 1024));
+        const size_t head = ((size_t)(2 * n + 1) * sizeof(int32_t) + 2 * sizeof(unsigned long long) + 511) & ~size_t(255);
+        for (;; cap = std::max<int64_t>(1024, cap / 2 / 1024 * 1024)) {
+            const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), head + (size_t)cap * n * sizeof(int32_t));
+            if (e == cudaSuccess) break;
+            cudaGetLastError();
+            base = nullptr;
+            if (cap == 1024) {
+                ct_set_error("ct_create: device scratch for the tuples: %s", cudaGetErrorString(e));
+                return CT_ERR_OOM;
+            }
+        }
+        counts = reinterpret_cast<unsigned long long*>(base);
+        lo = reinterpret_cast<int32_t*>(base + 2 * sizeof(unsigned long long));
+        row0 = lo + n;
+        tup = reinterpret_cast<int32_t*>(base + head);
+        meta = ct->lo;
+        meta.insert(meta.end(), ct->row0.begin(), ct->row0.end());
+        CT_CUDA(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), ct->stream));
+        CT_CUDA(cudaMemcpyAsync(lo, meta.data(), meta.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ct->stream));
+        return CT_OK;
+    }
+    // The chunk of `tuples` that starts at tuple j0 (nothing to do if it is there).
+    int load(const ct_table* ct, const int32_t* tuples, int64_t t, int64_t j0) {
+        if (held == tuples && heldAt == j0) return CT_OK;
+        const int64_t m = std::min(cap, t - j0);
+        CT_CUDA(cudaMemcpyAsync(tup, tuples + j0 * ct->arity, (size_t)m * ct->arity * sizeof(int32_t),
+                                cudaMemcpyHostToDevice, ct->stream));
+        held = tuples;
+        heldAt = j0;
+        return CT_OK;
+    }
+};
+
 int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const int32_t* tuples, int64_t t,
           const ct_options* opt, bool negative) {
     const int n = ct->arity;
@@ -302,24 +358,48 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
         for (int a = 0; a < ct->size[i]; ++a) ct->rowVar[ct->row0[i] + a] = i;
 
     // Retained tuples: every value inside its initial domain or a wildcard
-    // (input order kept).
-    std::vector<int64_t> keep;
-    keep.reserve((size_t)t);
+    // (input order kept). A positive table's list is checked on the device, a
+    // short one (kHostCheck components: less time than the device's answer
+    // takes, about 20 us) here; a list that keeps all its tuples is used as it is.
+    constexpr int64_t kHostCheck = 8192;
+    ct->profile = opt && opt->profile;
+    ct->copyState = opt && opt->copy_state;
+    int st;
     int64_t nShort = 0;
-    for (int64_t j = 0; j < t; ++j) {
-        const int32_t* tu = tuples + j * n;
-        bool ok = true, star = false;
-        for (int i = 0; i < n && ok; ++i) {
-            if (tu[i] == CT_STAR) {
-                star = true;
-                continue;
-            }
-            const int64_t off = (int64_t)tu[i] - ct->lo[i];
-            ok = off >= 0 && off < ct->size[i];
+    TupleStage stage;
+    bool all = false;
+    if (!negative && t * n > kHostCheck) {
+        if ((st = stage.open(ct, t)) != CT_OK) return st;
+        for (int64_t j0 = 0; j0 < t; j0 += stage.cap) {
+            if ((st = stage.load(ct, tuples, t, j0)) != CT_OK) return st;
+            CT_CUDA(launch_check_tuples(stage.tup, std::min(stage.cap, t - j0), n, stage.lo, stage.row0, stage.counts,
+                                        ct->stream));
         }
-        if (ok) {
-            keep.push_back(j);
-            nShort += star;
+        unsigned long long c[2] = {0, 0};
+        CT_CUDA(cudaMemcpyAsync(c, stage.counts, sizeof(c), cudaMemcpyDeviceToHost, ct->stream));
+        CT_CUDA(cudaStreamSynchronize(ct->stream));
+        all = c[0] == 0;
+        nShort = (int64_t)c[1];
+    }
+    std::vector<int64_t> keep;
+    if (!all) {
+        keep.reserve((size_t)t);
+        nShort = 0;  // (counted again, over the retained tuples)
+        for (int64_t j = 0; j < t; ++j) {
+            const int32_t* tu = tuples + j * n;
+            bool ok = true, star = false;
+            for (int i = 0; i < n && ok; ++i) {
+                if (tu[i] == CT_STAR) {
+                    star = true;
+                    continue;
+                }
+                const int64_t off = (int64_t)tu[i] - ct->lo[i];
+                ok = off >= 0 && off < ct->size[i];
+            }
+            if (ok) {
+                keep.push_back(j);
+                nShort += star;
+            }
         }
     }
     ct->shortTuples = nShort;
@@ -356,11 +436,16 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
         }
         ct->negative = true;
     }
-    ct->t = (int64_t)keep.size();
+    std::vector<int32_t> packed;  // the retained tuples of a list that loses some
+    all = all || (int64_t)keep.size() == t;
+    if (!all) {
+        packed.reserve(keep.size() * (size_t)n);
+        for (int64_t j : keep) packed.insert(packed.end(), tuples + j * n, tuples + (j + 1) * n);
+        tuples = packed.data();
+    }
+    ct->t = all ? t : (int64_t)keep.size();
     ct->W = (ct->t + 31) / 32;
     ct->W4 = (ct->W + 3) / 4;
-    ct->profile = opt && opt->profile;
-    ct->copyState = opt && opt->copy_state;
     if (ct->t == 0) {
         ct->empty = true;
         return CT_INFEASIBLE;
@@ -374,55 +459,11 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     ct->nseg = (int)((W4 + 31) / 32);
     ct->localPlan = n <= kLocalMaxArity && DW <= kLocalMaxDW && R <= kCodeCap;
 
-    // supports rows (Sec. 2), value-major, 16-byte aligned rows of W4 chunks
-    // (a short tuple is in every row of its wildcard positions; the delta rows
-    // hold only the tuples whose component equals the row's value)
-    const size_t rowWords = (size_t)W4 * 4;
-    std::vector<uint32_t> hsup((size_t)R * rowWords, 0u);
-    std::vector<uint32_t> hdel;
-    if (nShort > 0) hdel.assign((size_t)R * rowWords, 0u);
-    for (int64_t jj = 0; jj < ct->t; ++jj) {
-        const int32_t* tu = tuples + keep[(size_t)jj] * n;
-        const uint32_t bit = 1u << (jj & 31);
-        const size_t word = (size_t)(jj >> 5);
-        for (int i = 0; i < n; ++i) {
-            if (tu[i] == CT_STAR) {
-                for (int a = 0; a < ct->size[i]; ++a) hsup[(size_t)(ct->row0[i] + a) * rowWords + word] |= bit;
-                continue;
-            }
-            const int row = ct->row0[i] + (tu[i] - ct->lo[i]);
-            hsup[(size_t)row * rowWords + word] |= bit;
-            if (nShort > 0) hdel[(size_t)row * rowWords + word] |= bit;
-        }
-    }
-    std::vector<int32_t> hres(R, 0);
-    for (int r = 0; r < R; ++r) {
-        const uint32_t* row = hsup.data() + (size_t)r * rowWords;
-        for (int64_t c = 0; c < W4; ++c) {
-            if (row[c * 4] | row[c * 4 + 1] | row[c * 4 + 2] | row[c * 4 + 3]) {
-                hres[r] = (int32_t)c;
-                break;
-            }
-        }
-    }
-    // currTable: every retained tuple is valid under the initial domains.
-    std::vector<uint32_t> hcurr(rowWords, 0u);
-    for (int64_t w = 0; w < ct->W; ++w) {
-        const int64_t rem = ct->t - w * 32;
-        hcurr[(size_t)w] = rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u);
-    }
-    // Non-zero index: every chunk below W4 holds a retained tuple at creation.
-    std::vector<uint32_t> hmask(ct->nseg, 0u);
-    for (int s = 0; s < ct->nseg; ++s) {
-        const int64_t left = W4 - (int64_t)s * 32;
-        hmask[s] = left >= 32 ? 0xffffffffu : ((1u << left) - 1u);
-    }
     std::vector<uint32_t> hdom(DW, 0u);
     for (int i = 0; i < n; ++i)
         for (int a = 0; a < ct->size[i]; ++a) hdom[ct->ld[i] + a / 32] |= 1u << (a % 32);
 
     TableDev& d = ct->dev;
-    int st;
     uint4* sup = nullptr;
     int32_t *rowVar = nullptr, *varRow0 = nullptr, *varNW = nullptr, *varLD = nullptr;
     if ((st = dalloc(ct, &sup, (size_t)R * W4)) != CT_OK) return st;
@@ -512,16 +553,17 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
         ct->grid = std::max(1, std::min(want, maxCo));
     }
 
-    CT_CUDA(cudaMemcpyAsync(sup, hsup.data(), hsup.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ct->stream));
-    if (nShort > 0)
-        CT_CUDA(cudaMemcpyAsync(supDel, hdel.data(), hdel.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                                ct->stream));
-    CT_CUDA(cudaMemsetAsync(d.curr, 0, padChunks * sizeof(uint4), ct->stream));
-    CT_CUDA(cudaMemcpyAsync(d.curr, hcurr.data(), hcurr.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                            ct->stream));
-    if ((st = upload(ct, d.segMask, hmask)) != CT_OK) return st;
-    CT_CUDA(cudaMemsetAsync(d.lastpos, 0xff, padChunks * sizeof(int32_t), ct->stream));
-    if ((st = upload(ct, d.residue, hres)) != CT_OK) return st;
+    // supports rows (Sec. 2), value-major, 16-byte aligned rows of W4 chunks (a
+    // short tuple is in every row of its wildcard positions; the delta rows hold
+    // only the tuples whose component equals the row's value)
+    if (!stage.base && (st = stage.open(ct, ct->t)) != CT_OK) return st;
+    for (int64_t j0 = 0; j0 < ct->t; j0 += stage.cap) {
+        const int64_t m = std::min(stage.cap, ct->t - j0);
+        if ((st = stage.load(ct, tuples, ct->t, j0)) != CT_OK) return st;
+        CT_CUDA(launch_build_rows(stage.tup, m, n, stage.lo, stage.row0, sup, nShort > 0 ? supDel : nullptr, W4, j0,
+                                  j0 + m == ct->t, ct->stream));
+    }
+    CT_CUDA(launch_build_state(d, ct->t, ct->stream));
     if ((st = upload(ct, d.lastDom, hdom)) != CT_OK) return st;
     if ((st = upload(ct, rowVar, ct->rowVar)) != CT_OK) return st;
     if ((st = upload(ct, varRow0, ct->row0)) != CT_OK) return st;
