@@ -212,7 +212,11 @@ struct ModelCtrl {
 // The batched search run on the device (ct_search_batch_device): B slots, each
 // a copy of the network (T tables, nv variables, DWs domain words), search the
 // subtrees of open nodes taken from a device queue, depth-first with
-// first-fail branching, between the rounds of the fixpoint kernel.
+// first-fail branching, between the rounds of the fixpoint kernel. A slot's
+// stack holds the frames whose right branch is untried (a right branch replaces
+// its frame, so the stack is at most one frame per left branch of the path);
+// when the queue is empty, idle slots take the right branch of other slots'
+// lowest frames.
 // ---------------------------------------------------------------------------
 struct SearchCtr {
     unsigned long long nodes, fails, solutions;
@@ -223,29 +227,39 @@ struct SearchCtr {
     int32_t started;     // the first decision phase ran
     int32_t cur, round;  // work-list parity to resume a launch with
     int32_t done;        // every slot idle and no open node left (or the node limit reached)
-    int32_t pad[2];
+    int32_t nIdle;       // slots that found the queue empty in this decision phase
+    int32_t nGive;       // slots with a frame to give in this decision phase
+    int32_t want;        // slots were idle in the last decision phase: offer frames
+    int32_t steals;      // right branches taken over
 };
 
 struct SearchDev {
     int32_t B, T, nv, DWs, maxLevels, segTotal;
     int32_t nopen;
     int32_t roundBudget;          // rounds per launch before it returns (the host launches again)
+    int32_t pathWords;            // words of a branch path (a bit per tree level: at most the values of all variables)
     long long nodeLimit;          // <= 0: none
     SearchCtr* ctr;
     // per slot
     int32_t* depth;               // [B] frames on the stack
+    int32_t* given;               // [B] of them, from the bottom, whose right branch another slot took
     int32_t* active;              // [B]
     int32_t* busy;                // [B] the slot has tables in the next round (set by the collection)
-    int32_t* openIdx;             // [B] open node of the current subtree
-    int32_t* depth0;              // [B] tree depth of that open node
-    int4* frames;                 // [B][maxLevels] (x, a, branch, -)
+    int32_t* openIdx;             // [B] open node the current subtree lies under
+    int32_t* rel;                 // [B] depth of the current node below that open node
+    int32_t* subSol;              // [B] a solution was found in the current subtree
+    uint32_t* path;               // [B][pathWords] branches from the open node to the current node, high bit first (1: right)
+    int4* frames;                 // [B][maxLevels] (x, a, depth of the branching node below the open node, -)
     uint32_t* levelDom;           // [B][maxLevels + 1][DWs] domains at each level (level 0: the root)
     int32_t* markAt;              // [B][maxLevels + 1][T] trail position of each table at each level
     int32_t* liveAt;              // [B][maxLevels + 1][T] live chunks of each table at each level
     uint32_t* snapSeg;            // [B][maxLevels + 1][segTotal] index masks of every table at each level
-    int32_t* firstOpen;           // [B] open node of the slot's first solution (INT_MAX: none)
+    int32_t* firstOpen;           // [B] open node of the slot's first solution in depth-first order (INT_MAX: none)
+    uint32_t* firstPath;          // [B][pathWords] its path below that open node
     uint32_t* firstSol;           // [B][DWs] the domains of that solution
     int4* restQ;                  // [B * T] queued restores: (slot table j, level, -, -)
+    int32_t* idleList;            // [B] idle slots of a decision phase
+    int32_t* giveList;            // [B] slots with a frame to give
     ModelTabCall* calls;          // [B * T] the fixpoint kernel's per-table calls (mark kept current)
     // per model variable and table
     const int32_t* varOff;        // [nv] first domain word of each variable in a slot

@@ -243,13 +243,21 @@ __device__ __forceinline__ void remove_value(const ModelDev& M, const TableDev& 
 // The batched search on the device (search mode). Between two rounds of the
 // fixpoint, one warp per slot decides: a slot whose node is at its fixpoint
 // (no table of it in the next round) or failed branches on the first-fail
-// variable (left: x = min D(x)), backtracks to the deepest frame whose right
-// branch (x != min) is untried, or, with its subtree done, takes the next
+// variable (left: x = min D(x)), backtracks to the right branch (x != min) of
+// its deepest frame, or, with its subtree done, goes idle and takes the next
 // open node from the device queue. Restores are queued and done by the whole
 // grid after a barrier: a table's trail entries above the level's mark are
 // undone (each chunk written once), its non-zero index comes from the level's
 // snapshot, and its last-seen domains from the level's domains (a level is
 // saved at a fixpoint, where every table has seen the domains of its scope).
+// Beside the restores, idle slots that found the queue empty take over the
+// lowest frame (the largest subtree) of slots that have one to give: they
+// start from the root state (where going idle put them) with the domains of
+// that right branch, as from an open node. Without this the last slots' deep
+// subtrees held the search: on 10-variable instances of 14 tables with 512
+// slots, 28,480 nodes took 3,540 rounds, about 8 nodes a round.
+// A right branch replaces its frame: its changes trail from the level below,
+// so the stack and the trail grow with the left branches of the path only.
 // ---------------------------------------------------------------------------
 constexpr unsigned FULLM = 0xffffffffu;
 
@@ -340,9 +348,9 @@ __device__ void save_level(const ModelDev& M, const SearchDev& S, int s, int L) 
     }
 }
 
-// Queue the restore of every table of slot s to level L; their calls trail
-// from that level's marks again.
-__device__ void queue_restore(const SearchDev& S, int s, int L) {
+// Queue the restore of every table of slot s to level L; their calls then trail
+// from level Lmark's marks.
+__device__ void queue_restore(const SearchDev& S, int s, int L, int Lmark) {
     const int lane = threadIdx.x & 31;
     int base = 0;
     if (lane == 0) base = atomicAdd(&S.ctr->nrestQ, S.T);
@@ -350,7 +358,7 @@ __device__ void queue_restore(const SearchDev& S, int s, int L) {
     // (at most one restore per slot and decision phase: the queue holds B * T)
     for (int k = lane; k < S.T; k += 32) {
         S.restQ[base + k] = make_int4(s * S.T + k, L, 0, 0);
-        S.calls[s * S.T + k].mark = S.markAt[lvl(S, s, L) * S.T + k];
+        S.calls[s * S.T + k].mark = S.markAt[lvl(S, s, Lmark) * S.T + k];
     }
 }
 
@@ -380,41 +388,94 @@ __device__ void append_var(const SearchDev& S, int s, int x, int32_t* next, int3
     }
 }
 
+// Branch taken at depth r below the slot's open node (one lane).
+__device__ __forceinline__ void set_path(const SearchDev& S, int s, int r, bool right) {
+    uint32_t* w = S.path + (size_t)s * S.pathWords + (r >> 5);
+    const uint32_t bit = 0x80000000u >> (r & 31);
+    *w = right ? (__ldcg(w) | bit) : (__ldcg(w) & ~bit);
+}
+
+// A solution of slot s, the first of its current subtree: kept if it comes
+// before the slot's first one in depth-first order (the open node, then the
+// path below it; two solutions' paths differ before either ends).
+__device__ void keep_first(const SearchDev& S, int s, const uint32_t* dom) {
+    const int lane = threadIdx.x & 31;
+    const int o = __ldcg(&S.openIdx[s]), fo = __ldcg(&S.firstOpen[s]), len = __ldcg(&S.rel[s]);
+    if (o > fo) return;
+    uint32_t* best = S.firstPath + (size_t)s * S.pathWords;
+    const uint32_t* path = S.path + (size_t)s * S.pathWords;
+    auto word = [&](int w) {  // path bits at and beyond len are not the path's
+        const int left = len - 32 * w;
+        const uint32_t v = left > 0 ? __ldcg(path + w) : 0u;
+        return left >= 32 ? v : left > 0 ? v & ~(0xffffffffu >> left) : 0u;
+    };
+    bool first = o < fo;
+    for (int w0 = 0; o == fo && w0 < S.pathWords; w0 += 32) {
+        const int w = w0 + lane;
+        const uint32_t mine = w < S.pathWords ? word(w) : 0u, theirs = w < S.pathWords ? __ldcg(best + w) : 0u;
+        const unsigned diff = __ballot_sync(FULLM, mine != theirs);
+        if (!diff) continue;
+        first = __shfl_sync(FULLM, mine < theirs, __ffs(diff) - 1);
+        break;
+    }
+    if (!first) return;
+    for (int w = lane; w < S.pathWords; w += 32) best[w] = word(w);
+    for (int q = lane; q < S.DWs; q += 32) S.firstSol[(size_t)s * S.DWs + q] = __ldcg(dom + q);
+    __syncwarp();
+    if (lane == 0) S.firstOpen[s] = o;
+}
+
+// Slot s starts on the node whose domains are already in its domain words, at
+// depth rel below open node o, from the root state (one lane).
+__device__ __forceinline__ void start_slot(const ModelDev& M, const SearchDev& S, int s, int o, int rel) {
+    S.active[s] = 1;
+    S.depth[s] = 0;
+    S.given[s] = 0;
+    S.openIdx[s] = o;
+    S.rel[s] = rel;
+    S.subSol[s] = 0;
+    S.busy[s] = 0;
+    M.nodeStatus[s] = CT_OK;
+}
+
 // One warp: move slot s on when its node is done. Returns after issuing a
 // node (its tables are in the next round) or with the slot idle; at most one
-// restore of the slot is queued.
+// restore of the slot is queued. An idle slot's tables are at the root, or
+// queued to go there.
 __device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, int32_t* next, int32_t* nnext) {
     const int lane = threadIdx.x & 31;
     uint32_t* dom = M.dom + (size_t)s * S.DWs;
+    // a slot that goes on offers its lowest frame when slots are idle
+    auto offer = [&](int frames) {
+        if (frames > 0 && lane == 0 && __ldcg(&S.ctr->want)) S.giveList[atomicAdd(&S.ctr->nGive, 1)] = s;
+    };
     for (int guard = 0; guard < 2; ++guard) {
-        if (!S.active[s]) {
-            // an idle slot takes the next open node (its tables back at level 0, the root)
+        if (!__ldcg(&S.active[s])) {
+            // an idle slot takes the next open node
             if (__ldcg(&S.ctr->error) != CT_OK) return;
-            int o = 0;
-            if (lane == 0) o = atomicAdd(&S.ctr->nextOpen, 1);
+            int o = S.nopen;
+            if (lane == 0 && __ldcg(&S.ctr->nextOpen) < S.nopen) o = atomicAdd(&S.ctr->nextOpen, 1);
             o = __shfl_sync(FULLM, o, 0);
-            if (o >= S.nopen) return;
-            if (!issue_node(S, S.openDepth[o])) return;
-            queue_restore(S, s, 0);
-            for (int q = lane; q < S.DWs; q += 32) dom[q] = S.openDom[(size_t)o * S.DWs + q];
-            if (lane == 0) {
-                S.active[s] = 1;
-                S.depth[s] = 0;
-                S.openIdx[s] = o;
-                S.depth0[s] = S.openDepth[o];
-                S.busy[s] = 0;
-                M.nodeStatus[s] = CT_OK;
+            if (o >= S.nopen) {
+                if (lane == 0) S.idleList[atomicAdd(&S.ctr->nIdle, 1)] = s;
+                return;
             }
+            if (!issue_node(S, S.openDepth[o])) return;
+            for (int q = lane; q < S.DWs; q += 32) dom[q] = S.openDom[(size_t)o * S.DWs + q];
+            if (lane == 0) start_slot(M, S, s, o, 0);
             append_tables(S, s, nullptr, S.T, next, nnext);
             return;
         }
+        const int d = __ldcg(&S.depth[s]), given = __ldcg(&S.given[s]);
         if (__ldcg(&S.busy[s])) {  // its node is still propagating
             if (lane == 0) S.busy[s] = 0;
+            offer(d - given);
             return;
         }
         const bool failed = __ldcg(&M.nodeStatus[s]) != CT_OK;
+        const int rel = __ldcg(&S.rel[s]), depth0 = S.openDepth[__ldcg(&S.openIdx[s])];
+        __syncwarp();
         if (lane == 0) M.nodeStatus[s] = CT_OK;
-        int d = S.depth[s];
         if (!failed) {
             const int x = warp_first_fail(S, dom);
             if (x >= 0) {
@@ -424,7 +485,7 @@ __device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, int32_
                     if (lane == 0) S.active[s] = 0;
                     return;
                 }
-                if (!issue_node(S, S.depth0[s] + d + 1)) {
+                if (!issue_node(S, depth0 + rel + 1)) {
                     if (lane == 0) S.active[s] = 0;
                     return;
                 }
@@ -433,55 +494,80 @@ __device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, int32_
                 __syncwarp();
                 for (int q = lane; q < S.varNW[x]; q += 32) dom[S.varOff[x] + q] = q == (a >> 5) ? 1u << (a & 31) : 0u;
                 if (lane == 0) {
-                    S.frames[(size_t)s * S.maxLevels + d] = make_int4(x, a, 0, 0);
+                    S.frames[(size_t)s * S.maxLevels + d] = make_int4(x, a, rel, 0);
                     S.depth[s] = d + 1;
+                    S.rel[s] = rel + 1;
+                    set_path(S, s, rel, false);
                 }
                 append_var(S, s, x, next, nnext);
+                offer(d + 1 - given);
                 return;
             }
-            // every variable fixed: a solution. A slot takes open nodes in
-            // increasing (depth-first) order and searches each subtree
-            // depth-first, so its first solution is the first of its subtrees;
-            // it is kept for the host.
-            bool first = false;
-            if (lane == 0) {
-                atomicAdd(&S.ctr->solutions, 1ull);
-                first = S.openIdx[s] < S.firstOpen[s];
-                if (first) S.firstOpen[s] = S.openIdx[s];
+            // every variable fixed: a solution; within a subtree the slot's
+            // first is the first in depth-first order
+            if (lane == 0) atomicAdd(&S.ctr->solutions, 1ull);
+            if (!__ldcg(&S.subSol[s])) {
+                keep_first(S, s, dom);
+                __syncwarp();
+                if (lane == 0) S.subSol[s] = 1;
             }
-            first = __shfl_sync(FULLM, first, 0);
-            if (first)
-                for (int q = lane; q < S.DWs; q += 32) S.firstSol[(size_t)s * S.DWs + q] = __ldcg(dom + q);
         } else if (lane == 0) {
             atomicAdd(&S.ctr->fails, 1ull);
         }
-        // backtrack: the deepest frame with an untried right branch
-        while (d > 0 && S.frames[(size_t)s * S.maxLevels + d - 1].z != 0) --d;
-        if (d == 0) {
-            if (lane == 0) {
-                S.depth[s] = 0;
-                S.active[s] = 0;
-            }
+        if (d == given) {
+            // the subtree is done: idle, back to the root
+            queue_restore(S, s, 0, 0);
             __syncwarp();
-            continue;  // the subtree is done: take the next open node
+            if (lane == 0) S.active[s] = 0;
+            __syncwarp();
+            continue;  // take the next open node
         }
+        // backtrack: the deepest frame's right branch, in the frame's place
         const int4 f = S.frames[(size_t)s * S.maxLevels + d - 1];
-        if (!issue_node(S, S.depth0[s] + d)) {
+        if (!issue_node(S, depth0 + f.z + 1)) {
             if (lane == 0) S.active[s] = 0;
             return;
         }
-        queue_restore(S, s, d);
+        queue_restore(S, s, d, d - 1);
         const uint32_t* ld = S.levelDom + lvl(S, s, d) * S.DWs;
         for (int q = lane; q < S.DWs; q += 32) dom[q] = ld[q];
         __syncwarp();
         if (lane == 0) {
             dom[S.varOff[f.x] + (f.y >> 5)] &= ~(1u << (f.y & 31));
-            S.frames[(size_t)s * S.maxLevels + d - 1] = make_int4(f.x, f.y, 1, 0);
-            S.depth[s] = d;
+            S.depth[s] = d - 1;
+            S.rel[s] = f.z + 1;
+            set_path(S, s, f.z, true);
         }
         append_var(S, s, f.x, next, nnext);
+        offer(d - 1 - given);
         return;
     }
+}
+
+// One warp, beside the restores: idle slot s takes the right branch of slot
+// v's lowest frame (no decision runs; a slot is at most once in either list).
+__device__ void take_frame(const ModelDev& M, const SearchDev& S, int s, int v, int32_t* next, int32_t* nnext) {
+    const int lane = threadIdx.x & 31;
+    const int g = __ldcg(&S.given[v]), o = __ldcg(&S.openIdx[v]);
+    const int4 f = __ldcg(&S.frames[(size_t)v * S.maxLevels + g]);
+    if (!issue_node(S, S.openDepth[o] + f.z + 1)) return;
+    uint32_t* dom = M.dom + (size_t)s * S.DWs;
+    const uint32_t* ld = S.levelDom + lvl(S, v, g + 1) * S.DWs;
+    const int at = S.varOff[f.x] + (f.y >> 5);
+    for (int q = lane; q < S.DWs; q += 32) {
+        const uint32_t w = __ldcg(ld + q);
+        dom[q] = q == at ? w & ~(1u << (f.y & 31)) : w;
+    }
+    for (int w = lane; w <= (f.z >> 5); w += 32) {
+        const uint32_t p = __ldcg(S.path + (size_t)v * S.pathWords + w);
+        S.path[(size_t)s * S.pathWords + w] = w == (f.z >> 5) ? p | (0x80000000u >> (f.z & 31)) : p;
+    }
+    if (lane == 0) {
+        S.given[v] = g + 1;
+        start_slot(M, S, s, o, f.z + 1);
+        atomicAdd(&S.ctr->steals, 1);
+    }
+    append_tables(S, s, nullptr, S.T, next, nnext);
 }
 
 // One warp per queued restore: table j back to level L of its slot.
@@ -595,8 +681,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
             const int4 e = __ldcg(&Sd.restQ[q]);
             restore_table(M, Sd, e.x, e.y);
         }
+        // (the last warps first: the first ones hold the restores)
+        const int ns = min(__ldcg(&Sd.ctr->nIdle), __ldcg(&Sd.ctr->nGive));
+        for (int q = nwarps - 1 - gwarp; q < ns; q += nwarps)
+            take_frame(M, Sd, __ldcg(&Sd.idleList[q]), __ldcg(&Sd.giveList[q]), nl, nc);
         if (!sync()) return false;
-        if (blockIdx.x == 0 && tid == 0) Sd.ctr->nrestQ = 0;  // read by no CTA before the next decisions
+        if (blockIdx.x == 0 && tid == 0) {  // read by no CTA before the next decisions
+            Sd.ctr->nrestQ = 0;
+            Sd.ctr->want = __ldcg(&Sd.ctr->nIdle) > 0;
+            Sd.ctr->nIdle = 0;
+            Sd.ctr->nGive = 0;
+        }
         return true;
     };
     if (kSearch) {
@@ -1201,8 +1296,11 @@ __global__ void ct_search_init_kernel(const __grid_constant__ ModelDev M, const 
     }
     if (tid == 0) {
         S.depth[s] = 0;
+        S.given[s] = 0;
         S.active[s] = 0;
         S.busy[s] = 0;
+        S.rel[s] = 0;
+        S.subSol[s] = 0;
         S.firstOpen[s] = 0x7fffffff;
         M.nodeStatus[s] = CT_OK;
     }

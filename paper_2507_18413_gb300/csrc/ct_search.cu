@@ -361,11 +361,9 @@ int d_alloc(DevSearch* d, T** p, size_t n) {
 
 // First capacities of the device search, doubled (up to the maxima) and the
 // search run again when a subtree needs more.
-constexpr int kDevLevels = 64, kDevLevelsMax = 1024;        // levels below an open node
+constexpr int kDevLevels = 64, kDevLevelsMax = 1024;        // levels: left branches on a path below an open node
 constexpr int kDevTrailFactor = 16, kDevTrailFactorMax = 128;  // trail entries per table: factor x chunks + 1024
 constexpr int kDevRoundBudget = 1024;  // rounds per launch
-constexpr int kDevOpenPerSlot = 2;      // the device search splits until this many open nodes per slot
-constexpr int kMaxSplitDepth = 48;      // ... or this depth
 
 // The device search's buffers for the B slots of b (kept with b).
 int build_dsearch(ct_model* m, ct_batch* b, int levels, int trailFactor, DevSearch** out) {
@@ -390,12 +388,19 @@ int build_dsearch(ct_model* m, ct_batch* b, int levels, int trailFactor, DevSear
     S.maxLevels = L;
     S.segTotal = segOff[T];
     S.roundBudget = kDevRoundBudget;
+    // every branch takes a value off a variable's domain or fixes the variable
+    int64_t values = 1;
+    for (int v = 0; v < nv; ++v) values += m->size[v];
+    S.pathWords = (int32_t)((values + 31) / 32);
     const size_t lv = (size_t)B * (L + 1);
     int st = CT_OK;
     int32_t *vOff, *vNW, *vTS, *vTL, *sOff, *sTab;
     uint32_t** sPtr;
     if ((st = d_alloc(d, &S.ctr, 1)) || (st = d_alloc(d, &S.depth, B)) || (st = d_alloc(d, &S.active, B)) ||
-        (st = d_alloc(d, &S.busy, B)) || (st = d_alloc(d, &S.openIdx, B)) || (st = d_alloc(d, &S.depth0, B)) ||
+        (st = d_alloc(d, &S.given, B)) || (st = d_alloc(d, &S.rel, B)) || (st = d_alloc(d, &S.subSol, B)) ||
+        (st = d_alloc(d, &S.path, (size_t)B * S.pathWords)) || (st = d_alloc(d, &S.firstPath, (size_t)B * S.pathWords)) ||
+        (st = d_alloc(d, &S.idleList, B)) || (st = d_alloc(d, &S.giveList, B)) ||
+        (st = d_alloc(d, &S.busy, B)) || (st = d_alloc(d, &S.openIdx, B)) ||
         (st = d_alloc(d, &S.frames, (size_t)B * L)) || (st = d_alloc(d, &S.levelDom, lv * DWs)) ||
         (st = d_alloc(d, &S.markAt, lv * T)) || (st = d_alloc(d, &S.liveAt, lv * T)) ||
         (st = d_alloc(d, &S.snapSeg, lv * S.segTotal)) || (st = d_alloc(d, &S.firstOpen, B)) ||
@@ -454,7 +459,6 @@ struct Search {
     ct_batch* b = nullptr;
     int B = 0, splitDepth = 0;
     bool splitAssign = false;  // splitDepth counts assignments (left branches) on a node's path
-    int64_t minOpen = 0;       // the breadth-first split goes on below splitDepth while fewer open nodes
     int64_t limit = 0;
     bool countAll = true;
     bool anyStop = false;  // stop at the first solution any slot finds
@@ -648,8 +652,7 @@ struct Search {
         std::vector<OpenNode> F, G;
         children(F, m->h_dom, x, 1, std::vector<uint8_t>());
         for (int depth = 1; !F.empty() && !stopIssue; ++depth) {
-            if (!splitAssign && depth >= splitDepth && ((int64_t)F.size() >= minOpen || depth >= kMaxSplitDepth))
-                break;
+            if (!splitAssign && depth >= splitDepth) break;
             if (splitAssign) {
                 // nodes with splitDepth assignments on their path are open nodes
                 std::vector<OpenNode> rest;
@@ -1022,7 +1025,8 @@ struct Search {
         int L1 = 0;
         if ((rc = ct_model_save(m, &L1)) != CT_OK) return rc;
         rc = ct_model_propagate(m);  // the root fixpoint, for the state copies
-        int levels = b && b->dsearch ? b->dsearch->maxLevels : kDevLevels;
+        // (a left branch fixes a variable: a path holds at most as many as there are variables)
+        int levels = b && b->dsearch ? b->dsearch->maxLevels : std::min(kDevLevels, m->nvars);
         int factor = b && b->dsearch ? b->dsearch->trailFactor : kDevTrailFactor;
         for (;;) {
             if (rc == CT_OK) rc = ensure_copies();
@@ -1034,7 +1038,7 @@ struct Search {
             // a subtree deeper, or a trail fuller, than the capacities: larger
             // ones, from the start again (the counts are the same)
             if (rc == CT_ERR_LEVEL && levels < kDevLevelsMax) {
-                levels *= 2;
+                levels = std::min(2 * levels, kDevLevelsMax);
             } else if (rc == CT_ERR_OOM && devTrailFull && factor < kDevTrailFactorMax) {
                 factor *= 2;
             } else {
@@ -1187,15 +1191,24 @@ struct Search {
         st.max_depth = std::max(st.max_depth, c.maxDepth);
         info.slot_nodes += issued;
         info.open_nodes += std::min(c.nextOpen, nopen);
+        info.steals += c.steals;
         if (c.solutions > 0) {
             // the first solution in depth-first order: the slots' first
-            // solutions in their lowest open node, against the split's
+            // solutions by open node and path below it, against the split's
             std::vector<int32_t> fo(B);
+            std::vector<uint32_t> fp((size_t)B * S.pathWords);
             CT_CUDA(cudaMemcpyAsync(fo.data(), S.firstOpen, (size_t)B * 4, cudaMemcpyDeviceToHost, str));
+            CT_CUDA(cudaMemcpyAsync(fp.data(), S.firstPath, fp.size() * 4, cudaMemcpyDeviceToHost, str));
             CT_CUDA(cudaStreamSynchronize(str));
             int bs = -1;
-            for (int q = 0; q < B; ++q)
-                if (fo[q] < nopen && (bs < 0 || fo[q] < fo[bs])) bs = q;
+            for (int q = 0; q < B; ++q) {
+                if (fo[q] >= nopen) continue;
+                const uint32_t* p = fp.data() + (size_t)q * S.pathWords;
+                const uint32_t* best = fp.data() + (size_t)std::max(bs, 0) * S.pathWords;
+                if (bs < 0 || fo[q] < fo[bs] ||
+                    (fo[q] == fo[bs] && std::lexicographical_compare(p, p + S.pathWords, best, best + S.pathWords)))
+                    bs = q;
+            }
             if (bs >= 0 && (!haveBest || after(bestPath, open[fo[bs]].path))) {
                 std::vector<uint32_t> sol(DWs);
                 CT_CUDA(cudaMemcpyAsync(sol.data(), S.firstSol + (size_t)bs * DWs, (size_t)DWs * 4,
@@ -1329,9 +1342,6 @@ int search_batch(ct_model* m, int slots, int split_depth, bool split_assign, int
     S.limit = node_limit;
     S.countAll = count_all == 1;
     S.anyStop = count_all == 2;
-    // the device search keeps no slot waiting for another's right branches:
-    // it splits on until every slot has several open nodes to take
-    if (on_device) S.minOpen = (int64_t)kDevOpenPerSlot * slots;
     // any solution: the model first searches alone for 4 nodes per slot; easy
     // instances end there, the others continue from the frontier it leaves
     if (S.anyStop) S.splitBudget = 4 * (int64_t)slots;
