@@ -120,7 +120,6 @@ struct TableDev {
                                 // other scope domains' sizes (saturated), written by the plan
     int32_t* hardRow;        // [R] values left for the full scan
     int32_t* foundChunk;     // [R]
-    uint32_t* removed;       // [DW] one-table kernel: values found unsupported by the call's probes (zero between calls)
     const int32_t* rowVar;   // [R] scope position of each row
     const int32_t* varRow0;  // [arity+1] first row of each variable (_supportJmp)
     const int32_t* varNW;    // [arity] words of each domain
@@ -132,13 +131,14 @@ struct TableDev {
     int32_t negative;        // 1: the tuples are forbidden (negative table)
     int32_t shard;           // 1: a word-range shard (one-table kernel only): no failure on an
                              // empty currTable, lastDom keeps the call's input domains
-    int32_t wordLanesLog;    // log2 of the lanes that share one variable's domain words (the widest domain's
-                             // words rounded up to a power of two, at most a warp; 0 up to two words)
     int32_t warpPlan;        // 1: the network kernel plans it with one warp (positive, arity
                              // <= 32, every domain <= kWarpPlanWords words)
     // Scopes of at most kParamArity variables: words, lastDom offset and first
     // supports row of each variable, so that the plan reads no global table.
     int32_t pNW[kParamArity], pLD[kParamArity], pRow0[kParamArity];
+    int32_t wordLanesLog;    // log2 of the lanes that share one variable's domain words (the widest domain's
+                             // words rounded up to a power of two, at most a warp; 0 up to two words)
+    uint32_t* removed;       // [DW] one-table kernel: values found unsupported by the call's probes (zero between calls)
 };
 
 // Per-call parameters of the propagation kernel.
