@@ -98,6 +98,7 @@ struct Ctrl {
     // counters above.
     alignas(128) uint32_t bar_count;  // grid barrier arrivals (only grows)
     uint32_t bar_base;                // grid barrier count at the start of the next launch
+    uint32_t bank[2][4];  // small-network kernel: live, live_in, words_in of a round by its parity (zero between launches)
 };
 
 // Everything a kernel needs, passed by value.
@@ -300,6 +301,8 @@ struct ModelDev {
     int4* missQ;                // [sum of the tables' rows] residue misses of a round: (table, row, residue)
     uint32_t spinLimit;         // polls of a grid-barrier wait before it gives up (0: kBarrierSpinLimit)
     SearchDev* search;          // device copy of the search state (search mode only)
+    int32_t netCodes;           // small-network kernel: row codes a warp holds (the largest table's rows)
+    int32_t nscope;             // ... and the scope entries of all tables
 };
 constexpr int kModelPhases = 8;  // prologue, plan, update, probe, scan, apply, next round, publish
 constexpr int kRestoreBatch = 256;
@@ -311,6 +314,13 @@ struct RestoreBatch {
 // The fixpoint kernel's variant depends on the launch's table count (M.ntables).
 int max_coresident_model_blocks(int ntables);
 cudaError_t launch_model(const ModelDev& M, int grid, cudaStream_t s);
+// The fixpoint of one small network of positive tables (ct_net.cu): at most
+// kNetMaxTables tables, each with a one-warp plan and at most kNetMaxRows rows,
+// and net_smem_bytes(M) <= kNetSmemMax (two CTAs per SM).
+constexpr int kNetMaxTables = 512, kNetMaxRows = 1024, kNetTabSmem = 64, kNetSmemMax = 112 << 10;
+int net_smem_bytes(const ModelDev& M);
+int max_coresident_net_blocks(const ModelDev& M);
+cudaError_t launch_net(const ModelDev& M, int grid, cudaStream_t s);
 // The fixpoint kernel in search mode (M.search set): decision and restore
 // phases between rounds, until the search is done or the launch's round budget
 // is spent. The grid is max_coresident_model_blocks()-bounded as for launch_model.

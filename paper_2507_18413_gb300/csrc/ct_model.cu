@@ -50,6 +50,11 @@ int sync_dom(ct_model* m) {
     return CT_OK;
 }
 
+// Resident CTAs of the kernel that runs the model's fixpoints.
+int model_max_blocks(const ct_model* m) {
+    return m->net ? max_coresident_net_blocks(m->md) : max_coresident_model_blocks((int)m->tables.size());
+}
+
 // Device descriptors of the network for the one-launch fixpoint (built once,
 // after the last table was added).
 int batch_setup(ct_model* m) {
@@ -131,22 +136,31 @@ int batch_setup(ct_model* m) {
     for (int v = 0; v < m->nvars; ++v) domBits += m->size[v];
     M.maxRounds = (int)std::min<int64_t>(domBits + 2, 1 << 30);
     m->tabVersion.assign(n, -1);
-    const int maxCo = max_coresident_model_blocks(n);
+    int64_t segs = 0, rows = 0;
+    int maxR = 1;
+    m->net = n >= 1 && n <= kNetMaxTables;
+    for (ct_table* tab : m->tables) {
+        const TableDev& d = ct_table_dev(tab);
+        segs += d.nseg;
+        rows += d.R;
+        maxR = std::max(maxR, d.R);
+        m->net = m->net && d.warpPlan && !d.negative;
+    }
+    M.netCodes = (maxR + 31) / 32 * 32;
+    M.nscope = base[n];
+    m->net = m->net && maxR <= kNetMaxRows && net_smem_bytes(M) <= kNetSmemMax;
+    const int maxCo = model_max_blocks(m);
     if (maxCo <= 0) {
         ct_set_error("model: the fixpoint kernel cannot be made resident on this device");
         return CT_ERR_CUDA;
-    }
-    int64_t segs = 0, rows = 0;
-    for (ct_table* tab : m->tables) {
-        segs += ct_table_dev(tab).nseg;
-        rows += ct_table_dev(tab).R;
     }
     if ((st = m_alloc(m, &M.missQ, (size_t)std::max<int64_t>(rows, 1))) != CT_OK) return st;
     if (m->opt.profile) {
         if ((st = m_alloc(m, &M.phaseNs, kModelPhases)) != CT_OK) return st;
         CT_CUDA(cudaMemsetAsync(M.phaseNs, 0, kModelPhases * sizeof(uint64_t), m->stream));
     }
-    int64_t want = std::max<int64_t>({(int64_t)n, (segs + kWarps - 1) / kWarps, (rows + 2 * kWarps - 1) / (2 * kWarps), 1});
+    const int rowsPer = m->net ? kWarps : 2 * kWarps;  // rows per CTA: the small-network kernel's barriers are few
+    int64_t want = std::max<int64_t>({(int64_t)n, (segs + kWarps - 1) / kWarps, (rows + rowsPer - 1) / rowsPer, 1});
     if (m->opt.grid_blocks > 0) want = m->opt.grid_blocks;
     m->grid = (int)std::min<int64_t>(want, maxCo);
     CT_CUDA(cudaStreamSynchronize(m->stream));
@@ -161,7 +175,7 @@ int set_var(ct_model* m, int v, const uint32_t* words);
 // CTA count of the fixpoint launch chosen by trial fixpoints (ct_options.autotune):
 // half of the 4 largest domains removed, propagated, restored; best of 3 per candidate.
 int tune_grid(ct_model* m) {
-    const int maxCo = max_coresident_model_blocks((int)m->tables.size());
+    const int maxCo = model_max_blocks(m);
     if (maxCo <= 0 || m->tables.empty()) return CT_OK;
     const int want = m->grid;
     std::vector<int> cands;
@@ -245,7 +259,7 @@ int batch_propagate(ct_model* m) {
     volatile int32_t* H = m->h_mstatus;
     H[0] = kNoChunk;
     const auto t0 = std::chrono::steady_clock::now();
-    CT_CUDA(launch_model(m->md, m->grid, m->stream));
+    CT_CUDA(m->net ? launch_net(m->md, m->grid, m->stream) : launch_model(m->md, m->grid, m->stream));
     bool seen = false;
     for (uint64_t it = 0;; ++it) {
         if (H[0] != kNoChunk) {

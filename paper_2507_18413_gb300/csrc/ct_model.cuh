@@ -49,6 +49,7 @@ struct ct_model {
     std::vector<int> tabVersion;
     std::vector<void*> allocs;
     int grid = 1;
+    bool net = false;  // the small-network kernel runs the fixpoints
     ct_batch* bsearch = nullptr;  // built by the first batched search, kept for the next ones
     bool hasNegative = false;     // a negative table: no ordering features or lookahead labels
     // learned branching order

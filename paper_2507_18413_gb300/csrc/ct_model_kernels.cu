@@ -26,45 +26,6 @@ static_assert(offsetof(Ctrl, live_in) == offsetof(Ctrl, live) + 4 * kCntLiveIn &
                   offsetof(Ctrl, words_in) == offsetof(Ctrl, live) + 4 * kCntWords && kCntLive == 0,
               "counter block layout");
 
-// Entry k of a round's prefix array: the shared-memory copy, or the global
-// array itself (read through L2) when the round is too long for the copy.
-__device__ __forceinline__ int pre_at(const int32_t* pre, int k, bool global) {
-    return global ? __ldcg(pre + k) : pre[k];
-}
-
-// Position k of the work list whose prefix range holds u: the largest k < n
-// with pre[k] <= u (pre is non-decreasing, pre[0] = 0 <= u). The whole warp
-// calls it with the same u. The answer stays in [lo, hi] with pre[lo] <= u;
-// each pass samples lo + j * step for j < 32, with 32 * step covering the
-// hi - lo + 1 candidates, and keeps the stretch from the last sample <= u to
-// the next sample.
-__device__ __forceinline__ int find_prefix(const int32_t* pre, int n, int u, bool global) {
-    const int lane = threadIdx.x & 31;
-    int lo = 0, hi = n - 1;
-    while (hi - lo >= 32) {
-        const int step = (hi - lo + 32) >> 5;
-        const int k = lo + lane * step;
-        const unsigned b = __ballot_sync(0xffffffffu, k <= hi && pre_at(pre, k, global) <= u);
-        lo += (31 - __clz(b)) * step;
-        hi = min(hi, lo + step - 1);
-    }
-    const int k = lo + lane;
-    const unsigned b = __ballot_sync(0xffffffffu, k <= hi && pre_at(pre, k, global) <= u);
-    return lo + (31 - __clz(b));
-}
-
-// The same search by one lane for its own u (binary search: the lanes of a
-// warp look up different units at once).
-__device__ __forceinline__ int lane_find_prefix(const int32_t* pre, int n, int u, bool global) {
-    int lo = 0, hi = n - 1;  // pre[lo] <= u
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (pre_at(pre, mid, global) <= u) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 // Exclusive prefixes of the segments and of the supports rows of work[k] over
 // k < n into unitOut[0..n] and rowOut[0..n] (one CTA): each thread sums a run
 // of entries, warps scan by shuffles, warp totals go through shared memory.
