@@ -320,7 +320,11 @@ cudaError_t launch_model(const ModelDev& M, int grid, cudaStream_t s);
 constexpr int kNetMaxTables = 512, kNetMaxRows = 1024, kNetTabSmem = 64, kNetSmemMax = 112 << 10;
 int net_smem_bytes(const ModelDev& M);
 int max_coresident_net_blocks(const ModelDev& M);
-cudaError_t launch_net(const ModelDev& M, int grid, cudaStream_t s);
+// block: the launch's host block [count, 3 pad | calls | domains | work list]; up
+// to kNetCallWords words travel in the kernel's parameters, a longer one (or
+// null) has been copied to M's arrays by the caller.
+constexpr int kNetCallWords = 512;
+cudaError_t launch_net(const ModelDev& M, const int32_t* block, int words, int grid, cudaStream_t s);
 // The fixpoint kernel in search mode (M.search set): decision and restore
 // phases between rounds, until the search is done or the launch's round budget
 // is spent. The grid is max_coresident_model_blocks()-bounded as for launch_model.

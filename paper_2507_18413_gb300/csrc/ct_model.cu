@@ -161,6 +161,14 @@ int batch_setup(ct_model* m) {
     }
     const int rowsPer = m->net ? kWarps : 2 * kWarps;  // rows per CTA: the small-network kernel's barriers are few
     int64_t want = std::max<int64_t>({(int64_t)n, (segs + kWarps - 1) / kWarps, (rows + rowsPer - 1) / rowsPer, 1});
+    if (m->net) {
+        // one CTA per SM while that leaves a warp per segment: a second one made
+        // the update 1.5 us per node longer on 200 segments and won nothing
+        int dev = 0, sms = 0;
+        CT_CUDA(cudaGetDevice(&dev));
+        CT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (segs <= (int64_t)sms * kWarps) want = std::min<int64_t>(want, sms);
+    }
     if (m->opt.grid_blocks > 0) want = m->opt.grid_blocks;
     m->grid = (int)std::min<int64_t>(want, maxCo);
     CT_CUDA(cudaStreamSynchronize(m->stream));
@@ -253,13 +261,16 @@ int batch_propagate(ct_model* m) {
     // round's tables in one copy
     m->h_blk[0] = nwork;
     std::memcpy(m->h_blk + 4 + 4 * (size_t)n, m->h_dom.data(), (size_t)m->DWg * sizeof(uint32_t));
-    CT_CUDA(cudaMemcpyAsync(m->d_blk, m->h_blk, (4 + 4 * (size_t)n + (size_t)m->DWg + (size_t)nwork) * sizeof(int32_t),
-                            cudaMemcpyHostToDevice, m->stream));
+    const size_t blkWords = 4 + 4 * (size_t)n + (size_t)m->DWg + (size_t)nwork;
+    const bool inl = m->net && blkWords <= (size_t)kNetCallWords;  // ... or in the launch's parameters
+    if (!inl)
+        CT_CUDA(cudaMemcpyAsync(m->d_blk, m->h_blk, blkWords * sizeof(int32_t), cudaMemcpyHostToDevice, m->stream));
     m->domStale = false;
     volatile int32_t* H = m->h_mstatus;
     H[0] = kNoChunk;
     const auto t0 = std::chrono::steady_clock::now();
-    CT_CUDA(m->net ? launch_net(m->md, m->grid, m->stream) : launch_model(m->md, m->grid, m->stream));
+    CT_CUDA(m->net ? launch_net(m->md, inl ? m->h_blk : nullptr, (int)blkWords, m->grid, m->stream)
+                   : launch_model(m->md, m->grid, m->stream));
     bool seen = false;
     for (uint64_t it = 0;; ++it) {
         if (H[0] != kNoChunk) {

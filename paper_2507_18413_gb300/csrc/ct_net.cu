@@ -28,12 +28,19 @@
 // and propagations as ct_model_kernel).
 #include <cstddef>
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 #include "ct_device.cuh"
 
 namespace ctk {
 namespace {
+
+// The block of a launch in the kernel's parameters.
+struct NetCall {
+    int32_t words;
+    alignas(16) int32_t w[kNetCallWords];
+};
 
 constexpr int kDirectRows = 4;  // rows per warp up to which a warp searches its own misses
 
@@ -96,11 +103,11 @@ __device__ __forceinline__ NetPlan net_plan(const TableDev& T, const int32_t* of
     if (own) {
         nw = V.nw(lane);
         ld = V.ld(lane);
-        const uint32_t* dp = dom + off[lane];
+        const uint32_t* dp = dom + off[lane];  // (parameters or global memory)
         const uint32_t* lp = last + ld;
 #pragma unroll
         for (int q = 0; q < kWarpPlanWords; ++q) {
-            d[q] = q < nw ? __ldcg(dp + q) : 0u;
+            d[q] = q < nw ? *reinterpret_cast<const volatile uint32_t*>(dp + q) : 0u;
             l[q] = q < nw ? __ldcg(lp + q) : 0u;
         }
 #pragma unroll
@@ -158,7 +165,10 @@ __device__ __forceinline__ NetPlan net_plan(const TableDev& T, const int32_t* of
     return P;
 }
 
-__global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_constant__ ModelDev M) {
+// in.words > 0: the launch's block (count, calls, domains, first work list) in
+// the parameters; round 0 plans from those domains while they are stored.
+__global__ void __launch_bounds__(kThreads, 2)
+ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCall in) {
     extern __shared__ __align__(16) int32_t dyn[];
     __shared__ uint32_t s_cnt[12];
     __shared__ int s_flag, s_sum[2 * kWarps];
@@ -187,13 +197,17 @@ __global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_consta
         }
     };
     // the launch's constants, the first work list, and the marks of round 0
+    const bool inl = in.words > 0;
+    const uint32_t* dom0 = inl ? reinterpret_cast<const uint32_t*>(in.w) + 4 + 4 * n : M.dom;
     for (int t = tid; t < n; t += kThreads) {
         dyn[L.nseg + t] = __ldg(&M.tabs[t].nseg);
         dyn[L.rows + t] = __ldg(&M.tabs[t].R);
-        dyn[L.mark + t] = __ldcg(&M.calls[t].mark);
-        const int from = __ldcg(&M.calls[t].snapFrom);
-        dyn[L.snap + t] = from < __ldcg(&M.calls[t].snapTo) ? from : -1;
+        const ModelTabCall cl = inl ? reinterpret_cast<const ModelTabCall*>(in.w + 4)[t] : M.calls[t];
+        dyn[L.mark + t] = cl.mark;
+        dyn[L.snap + t] = cl.snapFrom < cl.snapTo ? cl.snapFrom : -1;
     }
+    if (inl)
+        for (int q = gtid; q < M.DWg; q += gth) M.dom[q] = dom0[q];
     for (int t = tid; t <= n; t += kThreads) dyn[L.base + t] = __ldg(&M.scopeBase[t]);
     for (int q = tid; q < M.nscope; q += kThreads) {
         dyn[L.var + q] = __ldg(&M.scopeVar[q]);
@@ -207,8 +221,8 @@ __global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_consta
     for (int v = gtid; v < M.nvars; v += gth) M.prunedBy[v] = -1;
     if (tid < 12) s_cnt[tid] = 0u;
     if (tid < 2) s_bytes[tid] = 0ull;
-    int nwork = M.nworkIn ? __ldcg(M.nworkIn) : __ldcg(&C->nwork);
-    for (int k = tid; k < nwork; k += kThreads) work[k] = __ldcg(&M.work[k]);
+    int nwork = inl ? in.w[0] : __ldcg(M.nworkIn);
+    for (int k = tid; k < nwork; k += kThreads) work[k] = inl ? in.w[4 + 4 * n + M.DWg + k] : __ldcg(&M.work[k]);
     __syncthreads();
     auto bit_of = [&](const uint32_t* bits, int t) { return (bits[t >> 5] >> (t & 31)) & 1u; };
     // a table's last-seen domains, and where the round's domains go
@@ -263,6 +277,37 @@ __global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_consta
         }
         const int totalUnits = preU[nwork], totalRows = preR[nwork];
 
+        // the first row of the warp's lanes, what does not depend on the update:
+        // its residue is on the way while the warp updates, then the supports chunk
+        const int rpw = min(32, max(1, (totalRows + nwarps - 1) / nwarps));
+        const bool direct = totalRows <= kDirectRows * nwarps;
+        struct RowRef {
+            int t, r, res, word, bit, var;
+            uint4 sup;
+        };
+        auto row_ref = [&](int u) {
+            RowRef R;
+            const int k = lane_find_prefix(preR, nwork, u, false);
+            R.t = work[k];
+            R.r = u - preR[k];
+            const TableDev& T = tabs[R.t];
+            R.res = T.useResidues ? __ldcg(&T.residue[R.r]) : 0;
+            R.var = __ldg(&T.rowVar[R.r]);
+            return R;
+        };
+        auto row_sup = [&](RowRef& R) {
+            const TableDev& T = tabs[R.t];
+            R.sup = ld_sup(T.sup + (size_t)R.r * T.W4 + R.res);
+            const VarLayout V(T, nullptr, nullptr);
+            const int a = R.r - V.row0(R.var);
+            R.word = V.ld(R.var) + (a >> 5);
+            R.bit = a & 31;
+        };
+        RowRef R0{};
+        const int u00 = gwarp * rpw;
+        const bool row0 = lane < rpw && u00 + lane < totalRows;
+        if (row0) R0 = row_ref(u00 + lane);
+
         // update: unit u to warp u % nwarps
         int planned = -1;
         NetPlan P{};
@@ -275,7 +320,7 @@ __global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_consta
             const bool first = seg == 0;
             const int snap = s_snap[t] >= 0 && !bit_of(done, t) ? s_snap[t] : -1;
             if (t != planned || first) {
-                P = net_plan(T, s_off + s_base[t], M.dom, last_of(T, t, false), last_of(T, t, true), codes, first,
+                P = net_plan(T, s_off + s_base[t], round == 0 ? dom0 : M.dom, last_of(T, t, false), last_of(T, t, true), codes, first,
                              first ? snap : -1);
                 planned = t;
                 if (first && lane == 0) {
@@ -295,38 +340,13 @@ __global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_consta
                 trail_warp(T, it, __ldcg(&T.ctrl->trail_cap), &C->status);
             }
         }
-        // the first row of the warp's lanes: what does not depend on the update
-        const int rpw = min(32, max(1, (totalRows + nwarps - 1) / nwarps));
-        const bool direct = totalRows <= kDirectRows * nwarps;
-        struct RowRef {
-            int t, r, res, word, bit, var;
-            uint4 sup;
-        };
-        auto row_ref = [&](int u) {
-            RowRef R;
-            const int k = lane_find_prefix(preR, nwork, u, false);
-            R.t = work[k];
-            R.r = u - preR[k];
-            const TableDev& T = tabs[R.t];
-            R.res = T.useResidues ? __ldcg(&T.residue[R.r]) : 0;
-            const int i = __ldg(&T.rowVar[R.r]);
-            const VarLayout V(T, nullptr, nullptr);
-            const int a = R.r - V.row0(i);
-            R.var = i;
-            R.word = V.ld(i) + (a >> 5);
-            R.bit = a & 31;
-            R.sup = ld_sup(T.sup + (size_t)R.r * T.W4 + R.res);
-            return R;
-        };
-        RowRef R0{};
-        const int u00 = gwarp * rpw;
-        if (lane < rpw && u00 + lane < totalRows) R0 = row_ref(u00 + lane);
+        if (row0) row_sup(R0);
         if (!sync()) return;
         phase(2);
 
         // failure test (Algorithm 1 line 5) beside the first rows' loads
         uint4 cur0 = make_uint4(0u, 0u, 0u, 0u);
-        if (lane < rpw && u00 + lane < totalRows) cur0 = __ldcg(tabs[R0.t].curr + R0.res);
+        if (row0) cur0 = __ldcg(tabs[R0.t].curr + R0.res);
         bool stop = false;
         for (int k = tid; k < nwork; k += kThreads) {
             Ctrl* Tc = tabs[work[k]].ctrl;
@@ -382,6 +402,7 @@ __global__ void __launch_bounds__(kThreads, 2) ct_net_kernel(const __grid_consta
                 uint4 cur = cur0;
                 if (u0 != u00) {
                     R = row_ref(u);
+                    row_sup(R);
                     cur = __ldcg(tabs[R.t].curr + R.res);
                 }
                 const TableDev& T = tabs[R.t];
@@ -573,9 +594,12 @@ int max_coresident_net_blocks(const ModelDev& M) {
     return per * sms;
 }
 
-cudaError_t launch_net(const ModelDev& M, int grid, cudaStream_t s) {
+cudaError_t launch_net(const ModelDev& M, const int32_t* block, int words, int grid, cudaStream_t s) {
     ModelDev m = M;
-    void* args[] = {&m};
+    NetCall in;
+    in.words = block && words <= kNetCallWords ? words : 0;
+    if (in.words > 0) std::memcpy(in.w, block, (size_t)words * sizeof(int32_t));
+    void* args[] = {&m, &in};
     return cudaLaunchCooperativeKernel((const void*)ct_net_kernel, dim3(grid), dim3(kThreads), args,
                                        (size_t)net_smem_bytes(M), s);
 }
