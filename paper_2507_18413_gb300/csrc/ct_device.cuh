@@ -251,22 +251,26 @@ __device__ void plan(const TableDev& T, const VarLayout& V, const uint32_t* __re
     } else {
         constexpr int kAhead = 4;
         for (int b0 = 0; b0 < T.arity; b0 += kAhead * ngrp) {
+            // (indices clamped, not branched on: each level of loads issues at once)
             uint32_t dv[kAhead], lv[kAhead];
-            int nwv[kAhead];
-    #pragma unroll
+            int nwv[kAhead], offv[kAhead], ldv[kAhead];
+#pragma unroll
             for (int u = 0; u < kAhead; ++u) {
-                const int i = b0 + u * ngrp + grp;
-                nwv[u] = 0;
-                dv[u] = lv[u] = 0u;
-                if (i < T.arity) {
-                    nwv[u] = V.nw(i);
-                    if (sub < nwv[u]) {
-                        dv[u] = dom[V.off(i) + sub];
-                        lv[u] = T.lastDom[V.ld(i) + sub];
-                    }
-                }
+                const int i = min(b0 + u * ngrp + grp, T.arity - 1);
+                nwv[u] = V.nw(i);
+                offv[u] = V.off(i);
+                ldv[u] = V.ld(i);
             }
-    #pragma unroll
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u) {
+                const int q = min(sub, nwv[u] - 1);
+                dv[u] = dom[offv[u] + q];
+                lv[u] = T.lastDom[ldv[u] + q];
+            }
+#pragma unroll
+            for (int u = 0; u < kAhead; ++u)
+                if (b0 + u * ngrp + grp >= T.arity) nwv[u] = 0;
+#pragma unroll
             for (int u = 0; u < kAhead; ++u) {
                 if (b0 + u * ngrp >= T.arity) break;  // the same for every thread
                 const int i = b0 + u * ngrp + grp;
@@ -274,14 +278,14 @@ __device__ void plan(const TableDev& T, const VarLayout& V, const uint32_t* __re
                 uint32_t grow = 0u;
                 for (int q = sub; q < nwv[u]; q += gl) {
                     if (q != sub) {
-                        dv[u] = dom[V.off(i) + q];
-                        lv[u] = T.lastDom[V.ld(i) + q];
+                        dv[u] = dom[offv[u] + q];
+                        lv[u] = T.lastDom[ldv[u] + q];
                     }
                     grow |= dv[u] & ~lv[u];
                     nd += __popc(dv[u]);
                     ndel += __popc(lv[u] & ~dv[u]);
-                    if (domCopy) domCopy[V.ld(i) + q] = dv[u];
-                    for (int v = snapFrom; v < snapTo; ++v) T.levelDom[(size_t)v * T.DW + V.ld(i) + q] = lv[u];
+                    if (domCopy) domCopy[ldv[u] + q] = dv[u];
+                    for (int v = snapFrom; v < snapTo; ++v) T.levelDom[(size_t)v * T.DW + ldv[u] + q] = lv[u];
                 }
                 for (int o = gl >> 1; o > 0; o >>= 1) {
                     nd += __shfl_xor_sync(0xffffffffu, nd, o);
@@ -723,7 +727,7 @@ __device__ __forceinline__ uint4 chunk_after(const TableDev& T, const int32_t* c
 template <int kE>
 __device__ __forceinline__ uint4 probe_chunk(const TableDev& T, const int32_t* codes, int nrows, int c) {
     if constexpr (kE > 0) return chunk_after<kE>(T, codes, nrows, c);
-    else return __ldcg(T.curr + c);
+    else return T.curr[c];  // (a plain load: after the barrier nobody writes it, and every warp of the SM reads it)
 }
 
 // Position of the k-th (0-based) set bit of m (k < popcount(m)): halve the
@@ -740,6 +744,17 @@ __device__ __forceinline__ int nth_set_bit(uint32_t m, int k) {
         }
     }
     return pos;
+}
+
+// Chunk c of [0, 2^31) taken cyclically in a table of W4 < 2^30 chunks (32-bit,
+// a division only for tables of less than a window: the 64-bit remainder it
+// replaces was most of a window's instructions).
+__device__ __forceinline__ int wrap_chunk(int c, int W4) {
+    if (c >= W4) {
+        c -= W4;
+        if (c >= W4) c %= W4;
+    }
+    return c;
 }
 
 // Outcomes of the window search of a residue miss.
@@ -773,8 +788,8 @@ __device__ __forceinline__ int probe_windows(const TableDev& T, int r, int res, 
         constexpr int kStep = kE > 4 ? 1 : 2;
         for (int b = 0; b < kProbes; b += kStep) {
             if (complete && b * 32 >= W4) break;
-            const int c0 = (int)(((long long)res + 1 + b * 32 + lane) % W4);
-            const int c1 = (int)(((long long)res + 1 + (b + 1) * 32 + lane) % W4);
+            const int c0 = wrap_chunk(res + 1 + b * 32 + lane, W4);
+            const int c1 = wrap_chunk(res + 1 + (b + 1) * 32 + lane, W4);
             const bool two = kStep == 2 && b + 1 < kProbes;
             const uint4 s0 = ld_sup(row + c0), t0 = probe_chunk<kE>(T, codes, nrows, c0);
             uint4 s1 = make_uint4(0u, 0u, 0u, 0u), t1 = s1;
@@ -894,7 +909,9 @@ __device__ __forceinline__ void probe_miss(const TableDev& T, int r, int word, i
 // Residue misses of a warp (lanes `miss`, each holding its value r and residue
 // res) searched over the chunks that follow the residues, dead or alive, K
 // values at a time so that K rows' loads are in flight (after the update's
-// barrier only). Returns the lane's own outcome.
+// barrier only; currTable through L1: a table of few chunks is the same few
+// lines for every warp of the grid, and read past L1 the L2 slices that hold
+// them bound the search). Returns the lane's own outcome.
 template <int K>
 __device__ __forceinline__ int probe_dense_lanes(const TableDev& T, unsigned miss, int r, int res, uint32_t* s_cnt) {
     const unsigned FULL = 0xffffffffu;
@@ -912,7 +929,7 @@ __device__ __forceinline__ int probe_dense_lanes(const TableDev& T, unsigned mis
             if (miss) open |= 1u << k;
             miss &= miss - 1u;
             row[k] = T.sup + (size_t)__shfl_sync(FULL, r, ln[k]) * W4;
-            c[k] = (int)(((long long)__shfl_sync(FULL, res, ln[k]) + 1 + lane) % W4);
+            c[k] = wrap_chunk(__shfl_sync(FULL, res, ln[k]) + 1 + lane, W4);
         }
         for (int b = 0; b < nwin && open; ++b) {
             if (lane == 0) atomicAdd(&s_cnt[kCntWin], (uint32_t)__popc(open));
@@ -921,7 +938,7 @@ __device__ __forceinline__ int probe_dense_lanes(const TableDev& T, unsigned mis
             for (int k = 0; k < K; ++k) {
                 if ((open >> k) & 1u) {
                     s[k] = ld_sup(row[k] + c[k]);
-                    t[k] = __ldcg(T.curr + c[k]);
+                    t[k] = T.curr[c[k]];
                 }
             }
 #pragma unroll
@@ -937,8 +954,7 @@ __device__ __forceinline__ int probe_dense_lanes(const TableDev& T, unsigned mis
                     }
                     open &= ~(1u << k);
                 }
-                c[k] += 32;
-                if (c[k] >= W4) c[k] %= W4;
+                c[k] = wrap_chunk(c[k] + 32, W4);
             }
         }
     }

@@ -139,6 +139,7 @@ struct TableDev {
     int32_t pNW[kParamArity], pLD[kParamArity], pRow0[kParamArity];
     int32_t wordLanesLog;    // log2 of the lanes that share one variable's domain words (the widest domain's
                              // words rounded up to a power of two, at most a warp; 0 up to two words)
+    const int32_t* wordVar;  // [DW] scope position of each domain word
     uint32_t* removed;       // [DW] one-table kernel: values found unsupported by the call's probes (zero between calls)
 };
 
@@ -154,6 +155,7 @@ struct CallParams {
     int32_t domInParams;          // 1: the domains are domWords (local plan only); the result
                                   // leaves through the status block alone
     uint32_t domWords[kParamDomWords];
+    int32_t packed;    // 1: the domains lie in the table's packed layout (offset i = varLD[i])
     int32_t early;     // calls of at most min(early, U) rows filter beside the update (0: never; local plan)
 };
 

@@ -90,31 +90,35 @@ static_assert(kSlotStatus == 0 && kSlotLiveOut == 1 && kSlotWordsIn == 2 && kSlo
 // left for a full scan the CTA returns false without publishing.
 // The values the probes found unsupported are bits of T.removed, loaded in the
 // same round as the header (and, in the global plan, as the domain words); a
-// removal is a bit there too, so the work is per domain word, not per value,
-// with 2^wordLanesLog adjacent lanes on one variable's words. localDom: sm.dom
-// already holds the call's domains (local plan). early: the filter ran beside
+// removal is a bit there too, so the work is per domain word, not per value.
+// localDom: sm.dom already holds the call's domains (local plan). packed: the
+// caller's domains lie in the packed layout. early: the filter ran beside
 // the update (reported in the header; the failure is decided here).
 // Nobody else writes the domains or lastDom during a call: both are written
 // here, on CT_OK only.
 __device__ bool finalize(const TableDev& T, const VarLayout& V, uint32_t* __restrict__ dom, Smem& sm, int nh,
-                         uint64_t t3, bool localDom, bool early = false) {
+                         uint64_t t3, bool localDom, bool packed, bool early = false) {
     Ctrl* C = T.ctrl;
     const int tid = threadIdx.x;
     int32_t* H = T.statusBlk;
     __syncthreads();  // counters thread 0 of this CTA may have written just before
     const bool smemDom = localDom || T.DW <= kLocalMaxDW;
     uint32_t* rm = smemDom ? reinterpret_cast<uint32_t*>(sm.codes) : T.removed;  // (sm.codes is free by now)
-    const int lg = T.wordLanesLog, gl = 1 << lg, sub = tid & (gl - 1), ngrp = kThreads >> lg;
     int preRow = 0, preFc = 0;
     if (tid < nh) {
         preRow = __ldcg(&T.hardRow[tid]);
         preFc = __ldcg(&T.foundChunk[tid]);
     }
     const uint32_t preRm = tid < T.DW ? __ldcg(&T.removed[tid]) : 0u;  // used only if the call has hard values
+    // word w of the packed layout: its place in the caller's domains
+    auto at = [&](int w) {
+        if (packed) return w;
+        const int i = __ldg(&T.wordVar[w]);
+        return V.off(i) + w - V.ld(i);
+    };
     if (!localDom && smemDom) {
-#pragma unroll 4
-        for (int i = tid >> lg; i < T.arity; i += ngrp)
-            for (int q = sub; q < V.nw(i); q += gl) sm.dom[V.ld(i) + q] = __ldcg(&dom[V.off(i) + q]);
+#pragma unroll 8
+        for (int w = tid; w < T.DW; w += kThreads) sm.dom[w] = __ldcg(&dom[at(w)]);
     }
     if (tid < kStatusHdr) {
         // one predicated load (two for a stamp difference) per slot, no
@@ -168,33 +172,27 @@ __device__ bool finalize(const TableDev& T, const VarLayout& V, uint32_t* __rest
         // supported by another shard
         const bool keepLast = T.negative || T.shard;
         uint32_t pruned = 0;
-        for (int i = tid >> lg; i < T.arity; i += ngrp) {
-            for (int q = sub; q < V.nw(i); q += gl) {
-                const int w = V.ld(i) + q;
-                const uint32_t r = smemDom ? rm[w] : __ldcg(&rm[w]);
-                const uint32_t d = smemDom ? sm.dom[w] : __ldcg(&dom[V.off(i) + q]);
-                T.lastDom[w] = keepLast ? d : d & ~r;
-                if (r) {
-                    if (dom) dom[V.off(i) + q] = d & ~r;
-                    if (smemDom) sm.dom[w] = d & ~r;
-                    T.removed[w] = 0u;
-                    atomicOr(reinterpret_cast<unsigned*>(&sm.scan[kChgBase + (i >> 5)]), 1u << (i & 31));
-                    pruned += __popc(r);
-                }
+        for (int w = tid; w < T.DW; w += kThreads) {
+            const uint32_t r = smemDom ? rm[w] : __ldcg(&rm[w]);
+            const uint32_t d = smemDom ? sm.dom[w] : __ldcg(&dom[at(w)]);
+            T.lastDom[w] = keepLast ? d : d & ~r;
+            if (r) {
+                const int i = __ldg(&T.wordVar[w]);
+                if (dom) dom[at(w)] = d & ~r;
+                if (smemDom) sm.dom[w] = d & ~r;
+                T.removed[w] = 0u;
+                atomicOr(reinterpret_cast<unsigned*>(&sm.scan[kChgBase + (i >> 5)]), 1u << (i & 31));
+                pruned += __popc(r);
             }
         }
         if (pruned) atomicAdd(&sm.cnt[kCntPruned], pruned);
         __syncthreads();
         if (sm.cnt[kCntPruned]) {
-            // The changed mask and the domains of the variables that lost values
-            // go to the host.
+            // The changed mask and the domains go to the host (which takes the
+            // variables that lost values).
             uint32_t* outDom = reinterpret_cast<uint32_t*>(H + kStatusHdr + T.nChangedWords);
             for (int q = tid; q < T.nChangedWords; q += kThreads) H[kStatusHdr + q] = sm.scan[kChgBase + q];
-            for (int i = tid >> lg; i < T.arity; i += ngrp) {
-                if (!((sm.scan[kChgBase + (i >> 5)] >> (i & 31)) & 1)) continue;
-                for (int q = sub; q < V.nw(i); q += gl)
-                    outDom[V.ld(i) + q] = smemDom ? sm.dom[V.ld(i) + q] : __ldcg(&dom[V.off(i) + q]);
-            }
+            for (int w = tid; w < T.DW; w += kThreads) outDom[w] = smemDom ? sm.dom[w] : __ldcg(&dom[at(w)]);
         }
     } else if (any) {
         // what the probes beside a failed update marked is void
@@ -359,7 +357,13 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
         }
     } else {
         if (blockIdx.x == 0) {
-            plan(T, V, dom, T.planK, T.planRowOff, T.varSup, T.codes, nullptr, sm, P.snapFrom, P.snapTo);
+            // (scopes that fit keep the plan's own arrays in shared memory; the
+            // other CTAs need s_sup and the row codes only)
+            const bool own = T.arity <= kLocalMaxArity;
+            plan(T, V, dom, own ? sm.k : T.planK, own ? sm.rowOff : T.planRowOff, own ? sm.sup : T.varSup, T.codes,
+                 nullptr, sm, P.snapFrom, P.snapTo);
+            if (own)
+                for (int i = tid; i < T.arity; i += kThreads) T.varSup[i] = sm.sup[i];
             if (tid == 0) {
                 C->nval = sm.flags[2]; C->ndelta = sm.flags[3]; C->nreset = sm.flags[4]; C->nsup = sm.flags[5];
                 C->nrows = sm.flags[6];
@@ -398,7 +402,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
         }
         if (!ok) {
             // Domain error or empty domain: publish without filtering.
-            if (blockIdx.x == 0) finalize(T, V, domOut, sm, 0, 0ull, kLocal);
+            if (blockIdx.x == 0) finalize(T, V, domOut, sm, 0, 0ull, kLocal, P.packed);
             return;
         }
         if (blockIdx.x == 0 && tid == 0) {
@@ -515,7 +519,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             if (r1 == 2) {
                 if (tid == 0 && st1 == CT_OK) C->status = CT_INFEASIBLE;
                 __syncthreads();
-                finalize(T, V, domOut, sm, 0, 0ull, kLocal);
+                finalize(T, V, domOut, sm, 0, 0ull, kLocal, P.packed);
             }
             return;
         }
@@ -605,7 +609,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
                     if (b0 != gwarp * rpw) {
                         res = T.residue[r];
                         sr = ld_sup(T.sup + (size_t)r * T.W4 + res);
-                        cr = __ldcg(T.curr + res);
+                        cr = T.curr[res];
                     }
                     hit = nz(and4(sr, cr));
                     need = !hit;
@@ -654,7 +658,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     // it publishes: with none left undecided (every value kept its support,
     // or its windows covered every live chunk) it removes the unsupported
     // values and publishes, and the others are done.
-    if (r2 == 2 && finalize(T, V, domOut, sm, -1, t3, kLocal, early)) {
+    if (r2 == 2 && finalize(T, V, domOut, sm, -1, t3, kLocal, P.packed, early)) {
         CT_STAMP(6);
         return;
     }
@@ -692,7 +696,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     CT_STAMP(14);
     if (!sm.flag[1]) return;
     __threadfence();
-    finalize(T, V, domOut, sm, nh, 0ull, kLocal, early);
+    finalize(T, V, domOut, sm, nh, 0ull, kLocal, P.packed, early);
     CT_STAMP(7);
 }
 

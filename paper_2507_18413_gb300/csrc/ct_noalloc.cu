@@ -46,6 +46,7 @@ struct NaScratch {
     int32_t foundChunk[kNaMaxRows];
     int32_t residue[kNaMaxRows];
     uint32_t removed[kNaMaxDW];
+    int32_t wordVar[kNaMaxDW];
     int32_t rowVar[kNaMaxRows];
     int32_t varSup[kNaMaxArity];
     int32_t planK[kNaMaxArity];
@@ -59,6 +60,7 @@ static __device__ __align__(256) unsigned char g_ct_noalloc_scratch[sizeof(NaScr
 // kernel parameters, so no host buffer is read after the launch.
 struct NaInit {
     int32_t rowVar[kNaMaxRows];  // scope position of each supports row
+    int32_t wordVar[kNaMaxDW];   // ... and of each domain word
     int32_t R;
     int32_t nseg;
     int32_t W4;                  // 128-bit chunks of currTable
@@ -92,7 +94,10 @@ __global__ void ct_noalloc_init_kernel(const __grid_constant__ NaInit p) {
         const uint32_t m = __ballot_sync(0xffffffffu, live);
         if (lane == 0) S->segMask[seg0 >> 5] = m;
     }
-    if (tid < kNaMaxDW) S->removed[tid] = 0u;
+    if (tid < kNaMaxDW) {
+        S->removed[tid] = 0u;
+        S->wordVar[tid] = p.wordVar[tid];
+    }
     if (tid == 0) {
         S->status[kSlotStatus] = kNaPending;
     }
@@ -197,6 +202,7 @@ extern "C" int ct_propagate_noalloc(int arity, const int32_t* dom_size, int64_t 
     T.hardRow = S->hardRow;
     T.foundChunk = S->foundChunk;
     T.removed = S->removed;
+    T.wordVar = S->wordVar;
     T.rowVar = S->rowVar;
     T.statusBlk = S->status;
     T.arity = arity;
@@ -220,8 +226,10 @@ extern "C" int ct_propagate_noalloc(int arity, const int32_t* dom_size, int64_t 
     // non-zero index from the caller's currTable, reload the row -> variable
     // map, reset the status word.
     NaInit init;
-    for (int i = 0; i < arity; ++i)
+    for (int i = 0; i < arity; ++i) {
         for (int a = 0; a < dom_size[i]; ++a) init.rowVar[row0[i] + a] = i;
+        for (int q = 0; q < nw[i]; ++q) init.wordVar[ld[i] + q] = i;
+    }
     init.R = R;
     init.nseg = nseg;
     init.W4 = (int32_t)W4;
@@ -238,6 +246,7 @@ extern "C" int ct_propagate_noalloc(int arity, const int32_t* dom_size, int64_t 
     P.prevLive = (int32_t)W4;
     P.spinLimit = armed ? armed : kBarrierSpinLimit;
     P.maxSplit = 1;
+    P.packed = 1;
     for (int i = 0; i < arity; ++i) P.domOff[i] = ld[i];
     const int variant = nseg > nd->maxCo[1] * kWarps ? 3 : 1;
     int grid = (nseg + kWarps - 1) / kWarps;

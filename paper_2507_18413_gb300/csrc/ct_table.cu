@@ -465,7 +465,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
 
     TableDev& d = ct->dev;
     uint4* sup = nullptr;
-    int32_t *rowVar = nullptr, *varRow0 = nullptr, *varNW = nullptr, *varLD = nullptr;
+    int32_t *wordVar = nullptr, *rowVar = nullptr, *varRow0 = nullptr, *varNW = nullptr, *varLD = nullptr;
     if ((st = dalloc(ct, &sup, (size_t)R * W4)) != CT_OK) return st;
     uint4* supDel = sup;
     if (nShort > 0 && (st = dalloc(ct, &supDel, (size_t)R * W4)) != CT_OK) return st;
@@ -485,6 +485,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     if ((st = dalloc(ct, &d.hardRow, (size_t)R)) != CT_OK) return st;
     if ((st = dalloc(ct, &d.foundChunk, (size_t)R)) != CT_OK) return st;
     if ((st = dalloc(ct, &d.removed, (size_t)DW)) != CT_OK) return st;
+    if ((st = dalloc(ct, &wordVar, (size_t)DW)) != CT_OK) return st;
     if ((st = dalloc(ct, &rowVar, (size_t)R)) != CT_OK) return st;
     if ((st = dalloc(ct, &varRow0, (size_t)n + 1)) != CT_OK) return st;
     if ((st = dalloc(ct, &varNW, (size_t)n)) != CT_OK) return st;
@@ -495,6 +496,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     d.supDelta = supDel;
     d.negative = ct->negative ? 1 : 0;
     d.shard = (opt && opt->shard) ? 1 : 0;
+    d.wordVar = wordVar;
     d.rowVar = rowVar;
     d.varRow0 = varRow0;
     d.varNW = varNW;
@@ -565,6 +567,10 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     }
     CT_CUDA(launch_build_state(d, ct->t, ct->stream));
     if ((st = upload(ct, d.lastDom, hdom)) != CT_OK) return st;
+    std::vector<int32_t> hWordVar;
+    hWordVar.reserve(DW);
+    for (int i = 0; i < n; ++i) hWordVar.insert(hWordVar.end(), ct->nw[i], i);
+    if ((st = upload(ct, wordVar, hWordVar)) != CT_OK) return st;
     if ((st = upload(ct, rowVar, ct->rowVar)) != CT_OK) return st;
     if ((st = upload(ct, varRow0, ct->row0)) != CT_OK) return st;
     if ((st = upload(ct, varNW, ct->nw)) != CT_OK) return st;
@@ -696,6 +702,7 @@ int ct_table_propagate_on(ct_table* ct, uint32_t* dom, const int32_t* domOffDev,
     P.prevLive = ct->live;
     P.spinLimit = kBarrierSpinLimit;
     P.maxSplit = ct->maxSplit;
+    P.packed = domOffHost == ct->ld.data() ? 1 : 0;
     P.early = ct->early ? 16 : 0;
     for (int i = 0; i < ct->arity && i < kParamArity; ++i) P.domOff[i] = domOffHost[i];
     if (domHost) {
