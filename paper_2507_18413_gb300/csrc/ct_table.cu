@@ -9,6 +9,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <unordered_map>
 #include <vector>
 
@@ -92,9 +93,18 @@ namespace {
 // ---------------------------------------------------------------------------
 constexpr size_t kGuardBytes = 256;       // before and after a guarded buffer (keeps its 256-byte alignment)
 constexpr unsigned char kGuardFill = 0xA5;
+// One device allocation holding the buffers that were asked for together
+// (cudaMalloc takes about 33 us and cudaFree 28 us here, whatever the size: a
+// table's 25 buffers one by one made most of its construction); freed with the
+// last of them.
+struct DevBlock {
+    char* base;
+    int used;  // buffers still held
+};
 struct DevBuf {
     size_t bytes;
     bool guarded;
+    DevBlock* block;
 };
 std::mutex g_bufMu;
 std::unordered_map<void*, DevBuf> g_bufs;  // buffer as the table sees it -> size
@@ -102,33 +112,50 @@ int64_t g_bufBytes = 0;
 bool g_guardNew = false;                   // ct_debug_guard_buffers
 long long g_failAfter = -1;                // ct_debug_fail_alloc: allocations left before one fails
 
-cudaError_t table_malloc(void** p, size_t bytes) {
+struct BufAsk {
+    void** p;
+    size_t bytes;
+};
+
+// The buffers of `ask` in one allocation, all or none (each counts as one
+// allocation of the failure countdown).
+cudaError_t table_malloc_all(const std::vector<BufAsk>& ask) {
     std::lock_guard<std::mutex> lk(g_bufMu);
-    *p = nullptr;
+    for (const BufAsk& a : ask) *a.p = nullptr;
     if (g_failAfter >= 0) {
-        if (g_failAfter == 0) {
+        if (g_failAfter < (long long)ask.size()) {
             g_failAfter = -1;
             return cudaErrorMemoryAllocation;
         }
-        --g_failAfter;
+        g_failAfter -= (long long)ask.size();
     }
     const bool guarded = g_guardNew;
+    const size_t guard = guarded ? kGuardBytes : 0;
+    auto room = [&](size_t bytes) { return ((bytes + 255) & ~size_t(255)) + 2 * guard; };
+    size_t total = 0;
+    for (const BufAsk& a : ask) total += room(a.bytes);
     char* base = nullptr;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), bytes + (guarded ? 2 * kGuardBytes : 0));
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), total);
     if (e != cudaSuccess) return e;
     if (guarded) {
-        e = cudaMemset(base, kGuardFill, kGuardBytes);
-        if (e == cudaSuccess) e = cudaMemset(base + kGuardBytes + bytes, kGuardFill, kGuardBytes);
+        // (the guard behind a buffer begins at its last byte; the rounding behind
+        // it is filled too, as nobody writes there)
+        e = cudaMemset(base, kGuardFill, total);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();  // the guards are set before any use
         if (e != cudaSuccess) {
             cudaFree(base);
             return e;
         }
     }
-    void* user = base + (guarded ? kGuardBytes : 0);
-    g_bufs[user] = DevBuf{bytes, guarded};
-    g_bufBytes += (int64_t)bytes;
-    *p = user;
+    DevBlock* block = new DevBlock{base, (int)ask.size()};
+    size_t at = 0;
+    for (const BufAsk& a : ask) {
+        void* user = base + at + guard;
+        g_bufs[user] = DevBuf{a.bytes, guarded, block};
+        g_bufBytes += (int64_t)a.bytes;
+        *a.p = user;
+        at += room(a.bytes);
+    }
     return cudaSuccess;
 }
 
@@ -141,24 +168,111 @@ void table_free(void* p) {
         return;
     }
     g_bufBytes -= (int64_t)it->second.bytes;
-    cudaFree(static_cast<char*>(p) - (it->second.guarded ? kGuardBytes : 0));
+    DevBlock* block = it->second.block;
     g_bufs.erase(it);
+    if (--block->used == 0) {
+        cudaFree(block->base);
+        delete block;
+    }
 }
 
-template <typename T>
-int dalloc(ct_table* ct, T** p, size_t count) {
-    const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-    void* q = nullptr;
-    const cudaError_t e = table_malloc(&q, bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        ct_set_error("cudaMalloc(%zu bytes): %s", bytes, cudaGetErrorString(e));
-        return CT_ERR_OOM;
+// A table's buffers, asked for one by one and allocated together by take().
+struct TableBufs {
+    ct_table* ct;
+    std::vector<BufAsk> ask;
+    template <typename T>
+    void want(T** p, size_t count) {
+        ask.push_back({reinterpret_cast<void**>(const_cast<std::remove_const_t<T>**>(p)), std::max<size_t>(count, 1) * sizeof(T)});
     }
-    ct->allocs.push_back(q);
-    ct->deviceBytes += (int64_t)bytes;
-    *p = static_cast<T*>(q);
-    return CT_OK;
+    int take() {
+        size_t bytes = 0;
+        for (const BufAsk& a : ask) bytes += a.bytes;
+        const cudaError_t e = table_malloc_all(ask);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            ct_set_error("device buffers of a table (%zu bytes): %s", bytes, cudaGetErrorString(e));
+            return CT_ERR_OOM;
+        }
+        for (const BufAsk& a : ask) ct->allocs.push_back(*a.p);
+        ct->deviceBytes += (int64_t)bytes;
+        return CT_OK;
+    }
+};
+
+// ---------------------------------------------------------------------------
+// status blocks: mapped host memory, in slabs shared by the tables of the
+// process (cudaHostAlloc and cudaFreeHost take 110-250 us and 160 us here).
+// Blocks of up to kSlabBytes / 4 come from a slab of kSlabUnit units; a slab is
+// given back with its last block, but for one empty slab that is kept for the
+// next table. Larger blocks are allocations of their own.
+// ---------------------------------------------------------------------------
+constexpr size_t kSlabBytes = 64 << 10, kSlabUnit = 256;
+constexpr int kSlabUnits = (int)(kSlabBytes / kSlabUnit);
+struct Slab {
+    char* base = nullptr;
+    std::vector<bool> taken = std::vector<bool>(kSlabUnits, false);
+    int blocks = 0;
+};
+std::mutex g_slabMu;
+std::vector<Slab*> g_slabs;
+std::unordered_map<void*, std::pair<Slab*, int>> g_statusBlocks;  // block -> (slab, units); slab null: its own
+
+cudaError_t status_alloc(void** p, size_t bytes) {
+    std::lock_guard<std::mutex> lk(g_slabMu);
+    *p = nullptr;
+    if (bytes > kSlabBytes / 4) {
+        const cudaError_t e = cudaHostAlloc(p, bytes, cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e == cudaSuccess) g_statusBlocks[*p] = {nullptr, 0};
+        return e;
+    }
+    const int units = (int)((bytes + kSlabUnit - 1) / kSlabUnit);
+    for (size_t k = 0; k <= g_slabs.size(); ++k) {
+        if (k == g_slabs.size()) {
+            Slab* s = new Slab();
+            const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&s->base), kSlabBytes,
+                                                cudaHostAllocMapped | cudaHostAllocPortable);
+            if (e != cudaSuccess) {
+                delete s;
+                return e;
+            }
+            g_slabs.push_back(s);
+        }
+        Slab* s = g_slabs[k];
+        for (int u = 0, run = 0; u < kSlabUnits; ++u) {
+            run = s->taken[u] ? 0 : run + 1;
+            if (run < units) continue;
+            const int first = u + 1 - units;
+            std::fill(s->taken.begin() + first, s->taken.begin() + u + 1, true);
+            s->blocks += 1;
+            *p = s->base + (size_t)first * kSlabUnit;
+            g_statusBlocks[*p] = {s, units};
+            return cudaSuccess;
+        }
+    }
+    return cudaErrorMemoryAllocation;  // (a new slab has room for any block)
+}
+
+void status_free(void* p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lk(g_slabMu);
+    const auto it = g_statusBlocks.find(p);
+    if (it == g_statusBlocks.end()) return;
+    Slab* s = it->second.first;
+    const int units = it->second.second;
+    g_statusBlocks.erase(it);
+    if (!s) {
+        cudaFreeHost(p);
+        return;
+    }
+    const int first = (int)((static_cast<char*>(p) - s->base) / kSlabUnit);
+    std::fill(s->taken.begin() + first, s->taken.begin() + first + units, false);
+    if (--s->blocks > 0) return;
+    int empty = 0;
+    for (const Slab* o : g_slabs) empty += o->blocks == 0;
+    if (empty < 2) return;  // the one empty slab that is kept
+    g_slabs.erase(std::find(g_slabs.begin(), g_slabs.end(), s));
+    cudaFreeHost(s->base);
+    delete s;
 }
 
 template <typename T>
@@ -191,11 +305,10 @@ int ensure_trail(ct_table* ct, int64_t need) {
     if (cap > 0x7fffffffLL) cap = 0x7fffffffLL;
     int2* nk = nullptr;
     uint4* no = nullptr;
-    cudaError_t e = table_malloc(reinterpret_cast<void**>(&nk), (size_t)cap * sizeof(int2));
-    if (e == cudaSuccess) e = table_malloc(reinterpret_cast<void**>(&no), (size_t)cap * sizeof(uint4));
+    const cudaError_t e = table_malloc_all({{reinterpret_cast<void**>(&nk), (size_t)cap * sizeof(int2)},
+                                            {reinterpret_cast<void**>(&no), (size_t)cap * sizeof(uint4)}});
     if (e != cudaSuccess) {
         cudaGetLastError();
-        table_free(nk);
         ct_set_error("trail growth to %lld entries: %s", (long long)cap, cudaGetErrorString(e));
         return CT_ERR_OOM;
     }
@@ -226,12 +339,11 @@ int ensure_levels(ct_table* ct, int need) {
     const int cap = std::max(need, 2 * ct->levelCap);
     uint32_t* ns = nullptr;
     uint32_t* nd = nullptr;
-    cudaError_t e = table_malloc(reinterpret_cast<void**>(&ns), (size_t)cap * std::max(ct->nseg, 1) * sizeof(uint32_t));
-    if (e == cudaSuccess)
-        e = table_malloc(reinterpret_cast<void**>(&nd), (size_t)cap * std::max(ct->DW, 1) * sizeof(uint32_t));
+    const cudaError_t e =
+        table_malloc_all({{reinterpret_cast<void**>(&ns), (size_t)cap * std::max(ct->nseg, 1) * sizeof(uint32_t)},
+                          {reinterpret_cast<void**>(&nd), (size_t)cap * std::max(ct->DW, 1) * sizeof(uint32_t)}});
     if (e != cudaSuccess) {
         cudaGetLastError();
-        table_free(ns);
         ct_set_error("level stack growth: %s", cudaGetErrorString(e));
         return CT_ERR_OOM;
     }
@@ -268,7 +380,7 @@ void free_table(ct_table* ct) {
         table_free(ct->dev.levelSeg);
         table_free(ct->dev.levelDom);
     }
-    if (ct->h_status) cudaFreeHost(ct->h_status);
+    status_free(ct->h_status);
     if (ct->h_curr) cudaFreeHost(ct->h_curr);
     for (auto& e : ct->ev)
         if (e) cudaEventDestroy(e);
@@ -466,32 +578,35 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     TableDev& d = ct->dev;
     uint4* sup = nullptr;
     int32_t *wordVar = nullptr, *rowVar = nullptr, *varRow0 = nullptr, *varNW = nullptr, *varLD = nullptr;
-    if ((st = dalloc(ct, &sup, (size_t)R * W4)) != CT_OK) return st;
-    uint4* supDel = sup;
-    if (nShort > 0 && (st = dalloc(ct, &supDel, (size_t)R * W4)) != CT_OK) return st;
+    uint4* supDel = nullptr;
     // currTable and lastpos are padded to whole 32-chunk segments.
     const size_t padChunks = (size_t)ct->nseg * 32;
-    if ((st = dalloc(ct, &d.curr, padChunks)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.segMask, (size_t)ct->nseg)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.lastpos, padChunks)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.residue, (size_t)R)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.lastDom, (size_t)DW)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.ctrl, 1)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.codes, (size_t)R)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.planK, (size_t)n)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.planRowOff, (size_t)n)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.varSup, (size_t)n)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.other, (size_t)n)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.hardRow, (size_t)R)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.foundChunk, (size_t)R)) != CT_OK) return st;
-    if ((st = dalloc(ct, &d.removed, (size_t)DW)) != CT_OK) return st;
-    if ((st = dalloc(ct, &wordVar, (size_t)DW)) != CT_OK) return st;
-    if ((st = dalloc(ct, &rowVar, (size_t)R)) != CT_OK) return st;
-    if ((st = dalloc(ct, &varRow0, (size_t)n + 1)) != CT_OK) return st;
-    if ((st = dalloc(ct, &varNW, (size_t)n)) != CT_OK) return st;
-    if ((st = dalloc(ct, &varLD, (size_t)n)) != CT_OK) return st;
+    TableBufs bufs{ct, {}};
+    bufs.want(&sup, (size_t)R * W4);
+    if (nShort > 0) bufs.want(&supDel, (size_t)R * W4);
+    bufs.want(&d.curr, padChunks);
+    bufs.want(&d.segMask, (size_t)ct->nseg);
+    bufs.want(&d.lastpos, padChunks);
+    bufs.want(&d.residue, (size_t)R);
+    bufs.want(&d.lastDom, (size_t)DW);
+    bufs.want(&d.ctrl, 1);
+    bufs.want(&d.codes, (size_t)R);
+    bufs.want(&d.planK, (size_t)n);
+    bufs.want(&d.planRowOff, (size_t)n);
+    bufs.want(&d.varSup, (size_t)n);
+    bufs.want(&d.other, (size_t)n);
+    bufs.want(&d.hardRow, (size_t)R);
+    bufs.want(&d.foundChunk, (size_t)R);
+    bufs.want(&d.removed, (size_t)DW);
+    bufs.want(&wordVar, (size_t)DW);
+    bufs.want(&rowVar, (size_t)R);
+    bufs.want(&varRow0, (size_t)n + 1);
+    bufs.want(&varNW, (size_t)n);
+    bufs.want(&varLD, (size_t)n);
+    bufs.want(&ct->d_domScratch, (size_t)DW);
+    if ((st = bufs.take()) != CT_OK) return st;
+    if (nShort == 0) supDel = sup;
     ct->statusInts = (size_t)kStatusHdr + ct->nChW + DW;
-    if ((st = dalloc(ct, &ct->d_domScratch, (size_t)DW)) != CT_OK) return st;
     d.sup = sup;
     d.supDelta = supDel;
     d.negative = ct->negative ? 1 : 0;
@@ -523,8 +638,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
 
     // The status block lives in mapped host memory: the kernel's last CTA writes
     // it directly and the host reads it after the stream synchronises.
-    if (cudaHostAlloc((void**)&ct->h_status, ct->statusInts * sizeof(int32_t), cudaHostAllocMapped) !=
-        cudaSuccess) {
+    if (status_alloc((void**)&ct->h_status, ct->statusInts * sizeof(int32_t)) != cudaSuccess) {
         cudaGetLastError();
         ct->h_status = nullptr;
         ct_set_error("cudaHostAlloc of the status block failed");
@@ -931,32 +1045,38 @@ ct_table* ct_table_clone(const ct_table* src, cudaStream_t stream, DeviceArena* 
         ct->levelsInArena = true;
         ct->trailCap = (int)clone_trail_entries(src);
         ct->trailInArena = true;
-        int st = CT_OK;
-        if (ctrl) d.ctrl = ctrl;
-        else if ((st = dalloc(ct, &d.ctrl, 1)) != CT_OK) {
-            free_table(ct);
-            *status = st;
-            return nullptr;
+        if (ctrl) {
+            d.ctrl = ctrl;
+        } else {
+            TableBufs bufs{ct, {}};
+            bufs.want(&d.ctrl, 1);
+            const int st = bufs.take();
+            if (st != CT_OK) {
+                free_table(ct);
+                *status = st;
+                return nullptr;
+            }
         }
         *status = CT_OK;
         return ct;
     }
     const size_t padChunks = (size_t)ct->nseg * 32;
-    int st = CT_OK;
-    if ((st = dalloc(ct, &d.curr, padChunks)) != CT_OK || (st = dalloc(ct, &d.segMask, (size_t)ct->nseg)) != CT_OK ||
-        (st = dalloc(ct, &d.lastpos, padChunks)) != CT_OK || (st = dalloc(ct, &d.residue, (size_t)ct->R)) != CT_OK ||
-        (st = dalloc(ct, &d.lastDom, (size_t)ct->DW)) != CT_OK || (st = dalloc(ct, &d.codes, (size_t)ct->R)) != CT_OK ||
-        (st = dalloc(ct, &d.planK, (size_t)ct->arity)) != CT_OK ||
-        (st = dalloc(ct, &d.planRowOff, (size_t)ct->arity)) != CT_OK ||
-        (st = dalloc(ct, &d.varSup, (size_t)ct->arity)) != CT_OK ||
-        (st = dalloc(ct, &d.other, (size_t)ct->arity)) != CT_OK ||
-        (st = dalloc(ct, &d.hardRow, (size_t)ct->R)) != CT_OK || (st = dalloc(ct, &d.foundChunk, (size_t)ct->R)) != CT_OK) {
-        free_table(ct);
-        *status = st;
-        return nullptr;
-    }
+    TableBufs bufs{ct, {}};
+    bufs.want(&d.curr, padChunks);
+    bufs.want(&d.segMask, (size_t)ct->nseg);
+    bufs.want(&d.lastpos, padChunks);
+    bufs.want(&d.residue, (size_t)ct->R);
+    bufs.want(&d.lastDom, (size_t)ct->DW);
+    bufs.want(&d.codes, (size_t)ct->R);
+    bufs.want(&d.planK, (size_t)ct->arity);
+    bufs.want(&d.planRowOff, (size_t)ct->arity);
+    bufs.want(&d.varSup, (size_t)ct->arity);
+    bufs.want(&d.hardRow, (size_t)ct->R);
+    bufs.want(&d.foundChunk, (size_t)ct->R);
     if (ctrl) d.ctrl = ctrl;
-    else if ((st = dalloc(ct, &d.ctrl, 1)) != CT_OK) {
+    else bufs.want(&d.ctrl, 1);
+    int st = bufs.take();
+    if (st != CT_OK) {
         free_table(ct);
         *status = st;
         return nullptr;
@@ -1317,14 +1437,20 @@ extern "C" int ct_get_currtable(ct_table* ct, uint32_t* words_host, int64_t* non
         if (nonzero_words_out) *nonzero_words_out = 0;
         return CT_OK;
     }
-    std::vector<uint32_t> buf((size_t)ct->W4 * 4);
-    CT_CUDA(cudaMemcpyAsync(buf.data(), ct->dev.curr, buf.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost,
+    // straight into the caller's words; the non-zero ones are counted there
+    std::vector<uint32_t> buf;
+    if (!words_host) {
+        buf.resize((size_t)ct->W);
+        words_host = buf.data();
+    }
+    CT_CUDA(cudaMemcpyAsync(words_host, ct->dev.curr, (size_t)ct->W * sizeof(uint32_t), cudaMemcpyDeviceToHost,
                             ct->stream));
     CT_CUDA(cudaStreamSynchronize(ct->stream));
-    int64_t nz = 0;
-    for (int64_t w = 0; w < ct->W; ++w) nz += buf[(size_t)w] != 0u;
-    if (words_host) std::memcpy(words_host, buf.data(), (size_t)ct->W * sizeof(uint32_t));
-    if (nonzero_words_out) *nonzero_words_out = nz;
+    if (nonzero_words_out) {
+        int64_t nz = 0;
+        for (int64_t w = 0; w < ct->W; ++w) nz += words_host[w] != 0u;
+        *nonzero_words_out = nz;
+    }
     return CT_OK;
 }
 
