@@ -174,7 +174,8 @@ struct Smem {
     int32_t nd[kLocalMaxArity];     // |dom| (local plan)
     unsigned long long other[kLocalMaxArity];  // negative tables: product of the other domain sizes (saturated)
     int32_t scan[kThreads];
-    uint32_t cnt[12];
+    uint32_t cnt[12];               // counters of the update
+    uint32_t pcnt[12];              // ... and of the probes (which may run while thread 0 flushes the update's)
     int flags[8];                   // grow, empty, nval, ndelta, nreset, nsup, nrows
     int flag[4];
     int trw[kWarps];  // trail slots of each warp's segment, then their offsets in the CTA's block

@@ -301,6 +301,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     bar_init(bar, &C->bar_count, &C->bar_base, &C->status, P.spinLimit ? P.spinLimit : kBarrierSpinLimit);
     if (blockIdx.x == 0 && tid == 0) C->t[0] = gtimer();
     CT_STAMP(0);
+    if (tid < 12) sm.pcnt[tid] = 0u;  // (the plan's barriers come before the probes)
 
     // Prologue loads that do not depend on the plan: the first segment of the
     // warp when every warp takes a whole segment, and the residue (with its
@@ -494,12 +495,19 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
         }
         __syncthreads();
         CT_STAMP(2);
-        if (tid == 0) flush_update_counters(C, sm);
-        if (early) {
-            __syncthreads();  // the counters are read before the probes clear them
-            // this CTA's part of the update and its counts, released to the
-            // probes that wait for the whole update (wait_update_done)
-            if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&C->upd_done) : "memory");
+        // (the other warps go on to the probes meanwhile)
+        if (tid == 0) {
+            flush_update_counters(C, sm);
+            if (early) {
+                // this CTA's part of the update and its counts, released to the
+                // probes that wait for the whole update (wait_update_done); a CTA
+                // without a part has nothing to release, and a release would hold
+                // its first warp up for a round trip
+                if (blockIdx.x * kWarps < (unsigned)units)
+                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&C->upd_done) : "memory");
+                else
+                    asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(&C->upd_done) : "memory");
+            }
         }
     }
     if (ok && (nrows > 0 || T.negative) && !early) {
@@ -526,8 +534,6 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
     }
 
     // residue probes (Algorithm 3)
-    if (tid < 12) sm.cnt[tid] = 0u;
-    __syncthreads();
     // Tables of at most kLocalProbes windows: the windows after the residue
     // cover every chunk, so the live chunks need no index walk and no value is
     // left for the full scan (a 2-chunk table's calls with an unsupported value
@@ -551,7 +557,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             int m = 0;
             if (lane == 0) {
                 m = atomicAdd(&C->nscan, __popc(bal));
-                atomicAdd(&sm.cnt[kCntHard], (uint32_t)__popc(bal));
+                atomicAdd(&sm.pcnt[kCntHard], (uint32_t)__popc(bal));
             }
             m = __shfl_sync(0xffffffffu, m, 0) + __popc(bal & lanemask_lt());
             if (need) {
@@ -569,9 +575,9 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             if (r != pfirstE && present && lane == 0) res = T.residue[r];
             res = __shfl_sync(0xffffffffu, res, 0);
             if (nrows <= 4)
-                probe_early<4>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.cnt);
+                probe_early<4>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.pcnt);
             else
-                probe_early<U>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.cnt);
+                probe_early<U>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.pcnt);
         }
     } else if (kLocal) {
         for (int r = gwarp; r < T.R; r += nwarps) {
@@ -587,7 +593,7 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
                 cr = __ldcg(T.curr + res);
             }
             res = __shfl_sync(0xffffffffu, res, 0);
-            probe_loaded(T, r, word, a & 31, present, res, sr, cr, sparse, sm.cnt);
+            probe_loaded(T, r, word, a & 31, present, res, sr, cr, sparse, sm.pcnt);
         }
     } else {
         // one value per lane: its residue chunk; the warp then searches the
@@ -617,29 +623,29 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             }
             const unsigned nhit = __popc(__ballot_sync(0xffffffffu, hit));
             unsigned miss = __ballot_sync(0xffffffffu, need);
-            if (lane == 0 && nhit) atomicAdd(&sm.cnt[kCntHits], nhit);
+            if (lane == 0 && nhit) atomicAdd(&sm.pcnt[kCntHits], nhit);
             int o = kProbeUndecided;  // the lane's outcome
             if (T.useResidues && !sparse) {
-                o = probe_dense_lanes<4>(T, miss, r, res, sm.cnt);
+                o = probe_dense_lanes<4>(T, miss, r, res, sm.pcnt);
             } else if (T.useResidues) {
                 while (miss) {
                     const int l = __ffs(miss) - 1;
                     miss &= miss - 1u;
                     const int ol = probe_windows<true, kModelProbes>(T, __shfl_sync(0xffffffffu, r, l),
-                                                                     __shfl_sync(0xffffffffu, res, l), sm.cnt);
+                                                                     __shfl_sync(0xffffffffu, res, l), sm.pcnt);
                     if (lane == l) o = ol;
                 }
             }
-            if (need) note_probe(T, r, word, bit, o, sm.cnt);
+            if (need) note_probe(T, r, word, bit, o, sm.pcnt);
         }
     }
     __syncthreads();
     if (tid == 0) {
-        if (sm.cnt[kCntHits]) atomicAdd(&C->hits, (int)sm.cnt[kCntHits]);
-        if (sm.cnt[kCntLocal]) atomicAdd(&C->local_found, (int)sm.cnt[kCntLocal]);
-        if (sm.cnt[kCntMiss]) atomicAdd(&C->misses, (int)sm.cnt[kCntMiss]);
-        if (sm.cnt[kCntWin]) atomicAdd(&C->windows, (int)sm.cnt[kCntWin]);
-        if (sm.cnt[kCntHard]) atomicAdd(&C->nhard, sm.cnt[kCntHard]);
+        if (sm.pcnt[kCntHits]) atomicAdd(&C->hits, (int)sm.pcnt[kCntHits]);
+        if (sm.pcnt[kCntLocal]) atomicAdd(&C->local_found, (int)sm.pcnt[kCntLocal]);
+        if (sm.pcnt[kCntMiss]) atomicAdd(&C->misses, (int)sm.pcnt[kCntMiss]);
+        if (sm.pcnt[kCntWin]) atomicAdd(&C->windows, (int)sm.pcnt[kCntWin]);
+        if (sm.pcnt[kCntHard]) atomicAdd(&C->nhard, sm.pcnt[kCntHard]);
     }
     CT_STAMP(4);
     const int r2 = bar_sync(bar, &sm.flag[0]);
