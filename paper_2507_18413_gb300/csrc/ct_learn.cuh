@@ -30,6 +30,11 @@ struct FeatView {
     int32_t* deg = nullptr;       // [nv] tables holding each variable
     int32_t* scopeBase = nullptr; // [nt + 1] prefix of the arities
     int32_t* scopeOff = nullptr;  // word offset of every scope variable's domain
+    int32_t* pairVar = nullptr;   // [pairs] variable of every entry of adj
+    float4* pairStat = nullptr;   // [pairs] one-kernel path: the entry's part of the features
+    unsigned* ticket = nullptr;   // [nodes] ... and the node's entries done (zero between calls)
+    int32_t pairs = 0;            // entries of adj per node
+    bool small = false;           // the one-kernel path takes the network
     // per call
     uint32_t* counts = nullptr;   // [rowBase[nt]] valid tuples per supports row
     uint32_t* live = nullptr;     // [nt] valid tuples per table
