@@ -155,6 +155,7 @@ struct CallParams {
     int32_t domInParams;          // 1: the domains are domWords (local plan only); the result
                                   // leaves through the status block alone
     uint32_t domWords[kParamDomWords];
+    int32_t trailTop;  // trail entries in use (small-table kernel)
     int32_t packed;    // 1: the domains lie in the table's packed layout (offset i = varLD[i])
     int32_t early;     // calls of at most min(early, U) rows filter beside the update (0: never; local plan)
 };
@@ -350,6 +351,12 @@ cudaError_t launch_clone_state(const TableDev* src, const TableDev* dst, int nsr
 int max_coresident_blocks(int variant);
 cudaError_t launch_propagate(const TableDev& T, int variant, int grid, uint32_t* dom, const int32_t* domOff,
                              const CallParams& P, cudaStream_t s);
+// The same propagation by one CTA (ct_small.cu) for the tables small_table()
+// takes: a plain launch without barriers between CTAs. Scopes of at most
+// kParamArity variables of at most kWarpPlanWords words.
+constexpr int kSmallChunks = 128, kSmallRows = 512;
+bool small_table(const TableDev& T);
+cudaError_t launch_small(const TableDev& T, uint32_t* dom, const CallParams& P, cudaStream_t s);
 cudaError_t launch_save(const TableDev& T, int level, cudaStream_t s);
 cudaError_t launch_restore(const TableDev& T, int level, int mark, int top, int newMark, cudaStream_t s);
 cudaError_t launch_set_words(uint32_t* dst, const uint32_t* words, int n, cudaStream_t s);

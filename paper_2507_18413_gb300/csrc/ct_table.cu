@@ -671,6 +671,9 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
         want = std::max(want, std::min((ct->nseg + R + kWarps - 1) / kWarps, 64));
         if (opt && opt->grid_blocks > 0) want = opt->grid_blocks;
         ct->grid = std::max(1, std::min(want, maxCo));
+        // (a launch shape that was asked for, or is to be tuned, is the general kernel's)
+        ct->small = small_table(d) && !(opt && (opt->grid_blocks > 0 || opt->autotune));
+        if (ct->small) ct->grid = 1;
     }
 
     // supports rows (Sec. 2), value-major, 16-byte aligned rows of W4 chunks (a
@@ -832,6 +835,8 @@ int ct_table_propagate_on(ct_table* ct, uint32_t* dom, const int32_t* domOffDev,
         std::memcpy(P.domWords, domHost, (size_t)ct->DW * sizeof(uint32_t));
     }
     hv[kSlotStatus] = kNoChunk;  // overwritten by the kernel's last CTA
+    P.trailTop = ct->trailTop;
+    const bool small = ct->small && !ct->armPolls;  // (the hook is for the general kernel's barriers)
     if (ct->armPolls) {
         // Test hook (ct_arm_wait_timeout): an arrival count 2^30 behind every
         // target of this call (base 0), so no barrier completes and every wait
@@ -853,7 +858,8 @@ int ct_table_propagate_on(ct_table* ct, uint32_t* dom, const int32_t* domOffDev,
         evSlot = ct->evNext;
         CT_CUDA(cudaEventRecord(ct->ev[2 * evSlot], s));
     }
-    CT_CUDA(launch_propagate(ct->dev, ct->variant, ct->grid, dom, domOffDev, P, s));
+    CT_CUDA(small ? launch_small(ct->dev, dom, P, s)
+                  : launch_propagate(ct->dev, ct->variant, ct->grid, dom, domOffDev, P, s));
     if (ct->profile) {
         CT_CUDA(cudaEventRecord(ct->ev[2 * evSlot + 1], s));
         ct->evNext = (ct->evNext + 1) % ct_table::kEvRing;
