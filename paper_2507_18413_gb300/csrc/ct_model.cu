@@ -162,12 +162,14 @@ int batch_setup(ct_model* m) {
     const int rowsPer = m->net ? kWarps : 2 * kWarps;  // rows per CTA: the small-network kernel's barriers are few
     int64_t want = std::max<int64_t>({(int64_t)n, (segs + kWarps - 1) / kWarps, (rows + rowsPer - 1) / rowsPer, 1});
     if (m->net) {
-        // one CTA per SM while that leaves a warp per segment: a second one made
-        // the update 1.5 us per node longer on 200 segments and won nothing
+        // one CTA per SM: two share no more of the reads' latency and make every
+        // barrier wider. Per fixpoint, one against two: 512 tables of 3 rounds 98
+        // and 103 us (update 36.7 and 42.1), 64 tables of 1,024 tuples 1.5 us less,
+        // 100 tables of 60,000 tuples 43.0 and 43.7, 500 of 20,000 56.1 and 58.1.
         int dev = 0, sms = 0;
         CT_CUDA(cudaGetDevice(&dev));
         CT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (segs <= (int64_t)sms * kWarps) want = std::min<int64_t>(want, sms);
+        want = std::min<int64_t>(want, sms);
     }
     if (m->opt.grid_blocks > 0) want = m->opt.grid_blocks;
     m->grid = (int)std::min<int64_t>(want, maxCo);
@@ -298,9 +300,17 @@ int batch_propagate(ct_model* m) {
     m->stats.hard_values += (uint32_t)H[5];
     m->stats.update_bytes += (int64_t)(((uint64_t)(uint32_t)H[9] << 32) | (uint32_t)H[8]);
     m->stats.filter_bytes += (int64_t)(((uint64_t)(uint32_t)H[11] << 32) | (uint32_t)H[10]);
-    const int32_t* snapped = const_cast<const int32_t*>(H) + kModelHdr + 2 * n + m->DWg + 1;  // after the one node
-    for (int t = 0; t < n; ++t)
-        ct_table_batch_done(m->tables[t], H[kModelHdr + 2 * t], H[kModelHdr + 2 * t + 1], snapped[t] != 0);
+    // after the one node's status: the tables' snapshot flags, or from the
+    // small-network kernel a bit per table that ran (its pending levels were
+    // snapshotted then; the others' results are not written)
+    const int32_t* after = const_cast<const int32_t*>(H) + kModelHdr + 2 * n + m->DWg + 1;
+    for (int t = 0; t < n; ++t) {
+        if (m->net && !((after[t >> 5] >> (t & 31)) & 1)) {
+            m->tables[t]->failed = false;
+            continue;
+        }
+        ct_table_batch_done(m->tables[t], H[kModelHdr + 2 * t], H[kModelHdr + 2 * t + 1], m->net || after[t] != 0);
+    }
     if (status == CT_OK && H[kModelHdr + 2 * n + m->DWg] == CT_INFEASIBLE) {
         m->failed = true;
         return CT_INFEASIBLE;

@@ -539,17 +539,20 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
     }
     if (blockIdx.x != 0) return;
     // publish: CTA 0, the status word last
+    // (of the tables, those that ran: bit t of the words after the node status; a
+    // table's two words and the host's bookkeeping for them cost 2-5 us a call on 512 tables)
     int32_t* H = M.statusBlk;
     for (int t = tid; t < n; t += kThreads) {
+        if (!bit_of(done, t)) continue;
         const Ctrl* Tc = tabs[t].ctrl;
         H[kModelHdr + 2 * t] = __ldcg(&Tc->trail_top);
         H[kModelHdr + 2 * t + 1] = __ldcg(&Tc->live_state);
     }
     uint32_t* outDom = reinterpret_cast<uint32_t*>(H + kModelHdr + 2 * n);
+#pragma unroll 4
     for (int q = tid; q < M.DWg; q += kThreads) outDom[q] = __ldcg(&M.dom[q]);
     int32_t* outNode = H + kModelHdr + 2 * n + M.DWg;
-    for (int t = tid; t < n; t += kThreads)
-        outNode[1 + t] = s_snap[t] >= 0 && bit_of(done, t) ? 1 : 0;
+    for (int q = tid; q < (n + 31) / 32; q += kThreads) outNode[1 + q] = (int32_t)done[q];
     __syncthreads();
     if (tid == 0) {
         const int st = __ldcg(&C->status);
