@@ -164,7 +164,7 @@ int batch_setup(ct_model* m) {
     if (m->net) {
         // one CTA per SM: two share no more of the reads' latency and make every
         // barrier wider. Per fixpoint, one against two: 512 tables of 3 rounds 98
-        // and 103 us (update 36.7 and 42.1), 64 tables of 1,024 tuples 1.5 us less,
+        // and 103 us (update 36.7 and 42.1), 8 of 100,000 tuples 1.5 us less,
         // 100 tables of 60,000 tuples 43.0 and 43.7, 500 of 20,000 56.1 and 58.1.
         int dev = 0, sms = 0;
         CT_CUDA(cudaGetDevice(&dev));

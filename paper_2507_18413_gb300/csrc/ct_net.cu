@@ -167,7 +167,9 @@ __device__ __forceinline__ NetPlan net_plan(const TableDev& T, const int32_t* of
 
 // in.words > 0: the launch's block (count, calls, domains, first work list) in
 // the parameters; round 0 plans from those domains while they are stored.
-__global__ void __launch_bounds__(kThreads, 2)
+// One CTA per SM, so up to 255 registers: at 128 (two CTAs) the batches of rows
+// spilled, 53.2 us a search node (8 tables of 100,000 tuples) and 51.1 without.
+__global__ void __launch_bounds__(kThreads, 1)
 ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCall in) {
     extern __shared__ __align__(16) int32_t dyn[];
     __shared__ uint32_t s_cnt[12];
@@ -317,6 +319,7 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
             const TableDev& T = tabs[t];
             const int mark = s_mark[t];
             const SegState S = load_segment(T, seg, mark);
+            const int cap = __ldcg(&T.ctrl->trail_cap);
             const bool first = seg == 0;
             const int snap = s_snap[t] >= 0 && !bit_of(done, t) ? s_snap[t] : -1;
             if (t != planned || first) {
@@ -333,20 +336,28 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
                 TrailItem it;
                 it.need = false;
                 if (S.mask != 0u) {
-                    const uint4 acc = slice_rows<16, false, false>(T, seg, (S.mask >> lane) & 1u, S.cur, 0, P.nrows,
+                    const uint4 acc = slice_rows<16, false, false, 4>(T, seg, (S.mask >> lane) & 1u, S.cur, 0, P.nrows,
                                                                    codes, nullptr, 0);
                     finish_segment(T, mark, seg, S, acc, T.ctrl->bank[par], &T.ctrl->tuples, it);
                 }
-                trail_warp(T, it, __ldcg(&T.ctrl->trail_cap), &C->status);
+                trail_warp(T, it, cap, &C->status);
             }
         }
         if (row0) row_sup(R0);
         if (!sync()) return;
         phase(2);
 
-        // failure test (Algorithm 1 line 5) beside the first rows' loads
+        // failure test (Algorithm 1 line 5) beside the first rows' loads (all of
+        // them: read where they are used, each waited for the one before, 1.3 us a node)
         uint4 cur0 = make_uint4(0u, 0u, 0u, 0u);
-        if (row0) cur0 = __ldcg(tabs[R0.t].curr + R0.res);
+        int32_t in0 = 0;
+        uint32_t last0 = 0u;
+        if (row0) {
+            const TableDev& T = tabs[R0.t];
+            cur0 = __ldcg(T.curr + R0.res);
+            in0 = __ldcg(&T.varSup[R0.var]);
+            last0 = __ldcg(last_of(T, R0.t, true) + R0.word);
+        }
         bool stop = false;
         for (int k = tid; k < nwork; k += kThreads) {
             Ctrl* Tc = tabs[work[k]].ctrl;
@@ -400,14 +411,18 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
             RowRef R = R0;
             if (lane < rpw && u < totalRows) {
                 uint4 cur = cur0;
+                int32_t in = in0;
+                uint32_t last = last0;
                 if (u0 != u00) {
                     R = row_ref(u);
                     row_sup(R);
-                    cur = __ldcg(tabs[R.t].curr + R.res);
+                    const TableDev& T = tabs[R.t];
+                    cur = __ldcg(T.curr + R.res);
+                    in = __ldcg(&T.varSup[R.var]);
+                    last = __ldcg(last_of(T, R.t, true) + R.word);
                 }
                 const TableDev& T = tabs[R.t];
-                const bool present = __ldcg(&T.varSup[R.var]) != 0 &&
-                                     ((__ldcg(last_of(T, R.t, true) + R.word) >> R.bit) & 1u);
+                const bool present = in != 0 && ((last >> R.bit) & 1u);
                 hit = present && T.useResidues && nz(and4(R.sup, cur));
                 need = present && !hit;
             }
