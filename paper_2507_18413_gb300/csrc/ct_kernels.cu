@@ -470,9 +470,12 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             CT_STAMP(8);
             uint4 acc = make_uint4(~0u, ~0u, ~0u, ~0u);
             if (G == 1) {
+                const bool act = (S.mask >> lane) & 1u;
+                // (four rows or fewer: a batch of their size, not U rows predicated
+                // off; 100,000 tuples 675 -> 650 us for 32 calls, 4e6 855 -> 810)
                 if (S.mask != 0u)
-                    acc = slice_rows<U, false, false>(T, seg, (S.mask >> lane) & 1u, S.cur, 0, nrows, sm.codes,
-                                                      nullptr, 0);
+                    acc = nrows <= 4 ? slice_rows<4, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0)
+                                     : slice_rows<U, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0);
             } else {
                 if (S.mask != 0u) {
                     const int qa = min(nrows, slice * per);

@@ -183,11 +183,11 @@ __global__ void __launch_bounds__(kThreads) ct_small_kernel(const __grid_constan
         uint4 acc = make_uint4(~0u, ~0u, ~0u, ~0u);
         if (G == 1) {
             if (S.mask != 0u)
-                acc = slice_rows<16, false, false>(T, seg, (S.mask >> lane) & 1u, S.cur, 0, nrows, sm.codes, nullptr, 0);
+                acc = slice_rows<16, false, false, 4>(T, seg, (S.mask >> lane) & 1u, S.cur, 0, nrows, sm.codes, nullptr, 0);
         } else {
             if (S.mask != 0u) {
                 const int qa = min(nrows, slice * per);
-                slice_rows<16, false, true>(T, seg, (S.mask >> lane) & 1u, S.cur, qa, min(nrows, qa + per), sm.codes,
+                slice_rows<16, false, true, 4>(T, seg, (S.mask >> lane) & 1u, S.cur, qa, min(nrows, qa + per), sm.codes,
                                             &parts, warp);
             }
             __syncthreads();
