@@ -248,7 +248,6 @@ struct SearchDev {
     int32_t* depth;               // [B] frames on the stack
     int32_t* given;               // [B] of them, from the bottom, whose right branch another slot took
     int32_t* active;              // [B]
-    int32_t* busy;                // [B] the slot has tables in the next round (set by the collection)
     int32_t* openIdx;             // [B] open node the current subtree lies under
     int32_t* rel;                 // [B] depth of the current node below that open node
     int32_t* subSol;              // [B] a solution was found in the current subtree

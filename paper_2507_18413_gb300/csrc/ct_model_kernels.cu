@@ -44,8 +44,9 @@ __device__ void work_prefix(const ModelDev& M, const int32_t* work, int n, int32
 #pragma unroll
         for (int u = 0; u < kB; ++u)
             if (t[u] >= 0) {
-                su += M.tabs[t[u]].nseg;
-                sr += M.tabs[t[u]].R;
+                const TableDev& T = M.tabs[t[u] % M.nodeTables];
+                su += T.nseg;
+                sr += T.R;
             }
     }
     int iu = su, ir = sr;
@@ -79,8 +80,8 @@ __device__ void work_prefix(const ModelDev& M, const int32_t* work, int n, int32
         for (int u = 0; u < kB; ++u) t[u] = k0 + u < b1 ? __ldcg(&work[k0 + u]) : -1;
 #pragma unroll
         for (int u = 0; u < kB; ++u) {
-            ns[u] = t[u] >= 0 ? M.tabs[t[u]].nseg : 0;
-            nr[u] = t[u] >= 0 ? M.tabs[t[u]].R : 0;
+            ns[u] = t[u] >= 0 ? M.tabs[t[u] % M.nodeTables].nseg : 0;
+            nr[u] = t[u] >= 0 ? M.tabs[t[u] % M.nodeTables].R : 0;
         }
 #pragma unroll
         for (int u = 0; u < kB; ++u)
@@ -104,8 +105,11 @@ __device__ void work_prefix(const ModelDev& M, const int32_t* work, int n, int32
 // flags, first code of each variable, s_sup, row codes in variable order,
 // each variable's last code marked) and the table's call counters. A domain
 // that grew since the table's last propagation is a state error; an empty one
-// fails the table's node.
-__device__ void plan_warp(const ModelDev& M, const TableDev& T, const VarLayout& V, int t) {
+// fails the table's node. keep: the domains become the table's last-seen ones
+// here, where they are in registers (the search, whose domains never grow: a
+// launch that refuses one table's domains leaves every last-seen domain as it
+// was, so elsewhere they are copied once the plans have passed).
+__device__ void plan_warp(const ModelDev& M, const TableDev& T, const VarLayout& V, int t, bool keep) {
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     const bool own = lane < T.arity;
@@ -139,6 +143,11 @@ __device__ void plan_warp(const ModelDev& M, const TableDev& T, const VarLayout&
     if (own) {
         T.planK[lane] = delta ? (k | kCodeDelta) : k;
         T.varSup[lane] = nd > 1;
+        if (keep) {
+#pragma unroll
+            for (int q = 0; q < kWarpPlanWords; ++q)
+                if (q < nw) T.lastDom[V.ld(lane) + q] = d[q];
+        }
     }
     int rows = (bad || empty) ? 0 : k;
     int incl = rows;
@@ -200,9 +209,42 @@ __device__ __forceinline__ void remove_value(const ModelDev& M, const TableDev& 
     if (old != -1 && old != t) atomicExch(&pruned[v], -2);
 }
 
+// Table t's counters of the round, cleared for its next one; its live count and bytes kept.
+__device__ __forceinline__ void settle_table(ModelCtrl* C, Ctrl* Tc) {
+    const int nr = __ldcg(&Tc->nrows);
+    const unsigned long long live = nr > 0 ? __ldcg(&Tc->live) : (unsigned long long)__ldcg(&Tc->live_state);
+    const unsigned ns = (unsigned)__ldcg(&Tc->nscan);
+    if (nr > 0) {
+        Tc->live_state = (int32_t)live;
+        atomicAdd(&C->bytesUpdate, 4ull * __ldcg(&Tc->words_in) * (unsigned long long)(nr + 2));
+    }
+    if (ns) atomicAdd(&C->bytesFilter, 16ull * ns * live);
+    Tc->live = 0u; Tc->live_in = 0u; Tc->words_in = 0u; Tc->nhard = 0u; Tc->nrows = 0; Tc->nscan = 0;
+    Tc->tuples = 0u;
+}
+
+// Whether table t shares a variable that another table pruned: scope
+// variables eight at a time, their marks loaded together.
+__device__ __forceinline__ bool table_dirty(const ModelDev& M, int t, const int32_t* pruned) {
+    bool dirty = false;
+    const int j1 = M.scopeBase[t + 1];
+    for (int j = M.scopeBase[t]; j < j1; j += 8) {
+        int v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = j + u < j1 ? M.scopeVar[j + u] : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int p = v[u] >= 0 ? __ldcg(&pruned[v[u]]) : -1;
+            dirty |= p != -1 && p != t;
+        }
+    }
+    return dirty;
+}
+
 // ---------------------------------------------------------------------------
-// The batched search on the device (search mode). Between two rounds of the
-// fixpoint, one warp per slot decides: a slot whose node is at its fixpoint
+// The batched search on the device (search mode). At the end of a round of the
+// fixpoint, one warp per slot collects the slot's tables of the next round and
+// decides: a slot whose node is at its fixpoint
 // (no table of it in the next round) or failed branches on the first-fail
 // variable (left: x = min D(x)), backtracks to the right branch (x != min) of
 // its deepest frame, or, with its subtree done, goes idle and takes the next
@@ -326,13 +368,20 @@ __device__ void queue_restore(const SearchDev& S, int s, int L, int Lmark) {
 // A node is issued (counted) unless the node limit is reached.
 __device__ bool issue_node(const SearchDev& S, int depth) {
     const int lane = threadIdx.x & 31;
+    if (S.nodeLimit <= 0) {  // nothing waits for the count
+        if (lane == 0) {
+            atomicAdd(&S.ctr->nodes, 1ull);
+            atomicMax(&S.ctr->maxDepth, depth);
+        }
+        return true;
+    }
     unsigned long long o = 0;
     if (lane == 0) {
         o = atomicAdd(&S.ctr->nodes, 1ull);
-        if (S.nodeLimit <= 0 || (long long)o < S.nodeLimit) atomicMax(&S.ctr->maxDepth, depth);
+        if ((long long)o < S.nodeLimit) atomicMax(&S.ctr->maxDepth, depth);
     }
     o = __shfl_sync(FULLM, o, 0);
-    return S.nodeLimit <= 0 || (long long)o < S.nodeLimit;
+    return (long long)o < S.nodeLimit;
 }
 
 // The tables of variable x of slot s go to the next round; a variable in no
@@ -395,7 +444,6 @@ __device__ __forceinline__ void start_slot(const ModelDev& M, const SearchDev& S
     S.openIdx[s] = o;
     S.rel[s] = rel;
     S.subSol[s] = 0;
-    S.busy[s] = 0;
     M.nodeStatus[s] = CT_OK;
 }
 
@@ -403,7 +451,8 @@ __device__ __forceinline__ void start_slot(const ModelDev& M, const SearchDev& S
 // node (its tables are in the next round) or with the slot idle; at most one
 // restore of the slot is queued. An idle slot's tables are at the root, or
 // queued to go there.
-__device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, int32_t* next, int32_t* nnext) {
+// busy: tables of it are already in the next round (its node still propagates).
+__device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, bool busy, int32_t* next, int32_t* nnext) {
     const int lane = threadIdx.x & 31;
     uint32_t* dom = M.dom + (size_t)s * S.DWs;
     // a slot that goes on offers its lowest frame when slots are idle
@@ -411,7 +460,10 @@ __device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, int32_
         if (frames > 0 && lane == 0 && __ldcg(&S.ctr->want)) S.giveList[atomicAdd(&S.ctr->nGive, 1)] = s;
     };
     for (int guard = 0; guard < 2; ++guard) {
-        if (!__ldcg(&S.active[s])) {
+        // the slot's words, all on the way at once
+        const int active = __ldcg(&S.active[s]), d = __ldcg(&S.depth[s]), given = __ldcg(&S.given[s]);
+        const int rel = __ldcg(&S.rel[s]), open = __ldcg(&S.openIdx[s]), node = __ldcg(&M.nodeStatus[s]);
+        if (!active) {
             // an idle slot takes the next open node
             if (__ldcg(&S.ctr->error) != CT_OK) return;
             int o = S.nopen;
@@ -427,14 +479,12 @@ __device__ void decide_slot(const ModelDev& M, const SearchDev& S, int s, int32_
             append_tables(S, s, nullptr, S.T, next, nnext);
             return;
         }
-        const int d = __ldcg(&S.depth[s]), given = __ldcg(&S.given[s]);
-        if (__ldcg(&S.busy[s])) {  // its node is still propagating
-            if (lane == 0) S.busy[s] = 0;
+        if (busy) {
             offer(d - given);
             return;
         }
-        const bool failed = __ldcg(&M.nodeStatus[s]) != CT_OK;
-        const int rel = __ldcg(&S.rel[s]), depth0 = S.openDepth[__ldcg(&S.openIdx[s])];
+        const bool failed = node != CT_OK;
+        const int depth0 = S.openDepth[open];
         __syncwarp();
         if (lane == 0) M.nodeStatus[s] = CT_OK;
         if (!failed) {
@@ -632,19 +682,20 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
     // decisions, a barrier, the queued restores, a barrier)
     SearchDev Sd{};
     if (kSearch) Sd = *M.search;
+    // slot of the q-th turn of this warp: neighbours on different CTAs
+    const int spread = blockIdx.x + gridDim.x * warp;
     auto search_step = [&]() -> bool {
         int32_t* nl = M.work + (size_t)cur * M.ntables;
         int32_t* nc = &C->nnext[round & 1];
-        for (int s = gwarp; s < Sd.B; s += nwarps) decide_slot(M, Sd, s, nl, nc);
         if (!sync()) return false;
         const int nr = __ldcg(&Sd.ctr->nrestQ);
-        for (int q = gwarp; q < nr; q += nwarps) {
+        for (int q = spread; q < nr; q += nwarps) {
             const int4 e = __ldcg(&Sd.restQ[q]);
             restore_table(M, Sd, e.x, e.y);
         }
         // (the last warps first: the first ones hold the restores)
         const int ns = min(__ldcg(&Sd.ctr->nIdle), __ldcg(&Sd.ctr->nGive));
-        for (int q = nwarps - 1 - gwarp; q < ns; q += nwarps)
+        for (int q = nwarps - 1 - spread; q < ns; q += nwarps)
             take_frame(M, Sd, __ldcg(&Sd.idleList[q]), __ldcg(&Sd.giveList[q]), nl, nc);
         if (!sync()) return false;
         if (blockIdx.x == 0 && tid == 0) {  // read by no CTA before the next decisions
@@ -659,6 +710,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
         cur = __ldcg(&Sd.ctr->cur);
         round = __ldcg(&Sd.ctr->round);
         if (!__ldcg(&Sd.ctr->started)) {
+            for (int s = spread; s < Sd.B; s += nwarps)
+                decide_slot(M, Sd, s, false, M.work + (size_t)cur * M.ntables, &C->nnext[round & 1]);
             if (!search_step()) return;
             if (blockIdx.x == 0 && tid == 0) Sd.ctr->started = 1;
         }
@@ -704,7 +757,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
                         if (lane == 0) M.snapTaken[t] = 1;
                     }
                     __syncwarp();  // the snapshot reads lastDom before the plan's loads of it
-                    plan_warp(M, T, V, t);
+                    plan_warp(M, T, V, t, kSearch);
                 }
             }
         }
@@ -848,12 +901,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
             if (!T.negative && __ldcg(&T.ctrl->nrows) > 0 && __ldcg(&T.ctrl->live) == 0u)
                 M.nodeStatus[t / M.nodeTables] = CT_INFEASIBLE;
         }
-        // lastDom := the domains of this round (removals below clear their bits)
-        for (int k = blockIdx.x; k < nwork; k += gridDim.x) {
+        // lastDom := the domains of this round (removals below clear their bits):
+        // a warp per table, its domains' words over the lanes (a CTA per table
+        // took a chain of loads for each of its tables, 24 us of them with 7,168)
+        for (int k = gwarp; k < nwork; k += nwarps) {
             const int t = __ldcg(&work[k]);
             const TableDev& T = M.tabs[t];
+            if (kSearch && T.warpPlan) continue;  // (kept by the plan)
             const VarLayout V(T, nullptr, M.scopeOff + M.scopeBase[t]);
-            for (int i = tid; i < T.arity; i += kThreads)
+            for (int i = lane; i < T.arity; i += 32)
                 for (int q = 0; q < V.nw(i); ++q) T.lastDom[V.ld(i) + q] = __ldcg(&M.dom[V.off(i) + q]);
         }
         // filterDomains (Algorithm 3): the residue test of every (table, row) unit,
@@ -922,7 +978,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
         for (int q = gwarp; q < nm; q += nwarps) {
             const int4 e = __ldcg(&M.missQ[q]);
             const TableDev& T = M.tabs[e.x];
-            const int o = probe_windows<true, kModelProbes>(T, e.y, e.z, sm.cnt);
+            const int o = probe_network(T, e.y, e.z, sm.cnt);
             if (o != kProbeFound && lane == 0) {
                 if (o == kProbeGone) {
                     remove_value(M, T, e.x, e.y, pruned);
@@ -991,46 +1047,48 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
             int32_t* next = M.work + (size_t)(cur ^ 1) * M.ntables;
             int32_t* nnext = &C->nnext[(round + 1) & 1];
             const int gtid = blockIdx.x * kThreads + tid, gth = gridDim.x * kThreads;
-            for (int k = gtid; k < nwork; k += gth) {
-                Ctrl* Tc = M.tabs[__ldcg(&work[k])].ctrl;
-                const int nr = __ldcg(&Tc->nrows);
-                const unsigned long long live = nr > 0 ? __ldcg(&Tc->live) : (unsigned long long)__ldcg(&Tc->live_state);
-                if (nr > 0) {
-                    Tc->live_state = (int32_t)live;
-                    atomicAdd(&C->bytesUpdate, 4ull * __ldcg(&Tc->words_in) * (unsigned long long)(nr + 2));
-                }
-                const unsigned ns = (unsigned)__ldcg(&Tc->nscan);
-                if (ns) atomicAdd(&C->bytesFilter, 16ull * ns * live);
-                Tc->live = 0u; Tc->live_in = 0u; Tc->words_in = 0u; Tc->nhard = 0u; Tc->nrows = 0; Tc->nscan = 0;
-                Tc->tuples = 0u;
-            }
-            for (int t0 = gtid - lane; t0 < M.ntables; t0 += gth) {  // warp-uniform trip count
-                const int t = t0 + lane;
-                bool dirty = false;
-                if (t < M.ntables) {
-                    // scope variables eight at a time, their marks loaded together
-                    const bool alive = __ldcg(&M.nodeStatus[t / M.nodeTables]) == CT_OK;
-                    const int j1 = M.scopeBase[t + 1];
-                    for (int j = M.scopeBase[t]; j < j1; j += 8) {
-                        int v[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) v[u] = j + u < j1 ? M.scopeVar[j + u] : -1;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int p = v[u] >= 0 ? __ldcg(&pruned[v[u]]) : -1;
-                            dirty |= p != -1 && p != t;
+            if (kSearch) {
+                // a warp per slot: its tables' counters and which of them go on;
+                // with none, the slot's next step (no barrier in between: a
+                // slot's decision reads its own tables and marks alone; collected
+                // table by table over the grid and decided after a barrier, a
+                // round of 512 slots took 2.5 us longer)
+                for (int s = spread; s < Sd.B; s += nwarps) {
+                    bool busy = false;
+                    if (__ldcg(&Sd.active[s])) {
+                        const bool alive = __ldcg(&M.nodeStatus[s]) == CT_OK;
+                        for (int k0 = 0; k0 < Sd.T; k0 += 32) {
+                            const int t = s * Sd.T + k0 + lane;
+                            bool dirty = false;
+                            if (k0 + lane < Sd.T) {
+                                dirty = table_dirty(M, t, pruned) && alive;
+                                settle_table(C, M.tabs[t].ctrl);
+                            }
+                            const unsigned bal = __ballot_sync(0xffffffffu, dirty);
+                            if (!bal) continue;
+                            busy = true;
+                            int base = 0;
+                            if (lane == 0) base = atomicAdd(nnext, __popc(bal));
+                            base = __shfl_sync(0xffffffffu, base, 0);
+                            if (dirty) next[base + __popc(bal & lanemask_lt())] = t;
                         }
+                        __syncwarp();
                     }
-                    dirty &= alive;
+                    decide_slot(M, Sd, s, busy, next, nnext);
                 }
-                const unsigned bal = __ballot_sync(0xffffffffu, dirty);
-                if (bal) {
+            } else {
+                for (int k = gtid; k < nwork; k += gth) settle_table(C, M.tabs[__ldcg(&work[k])].ctrl);
+                for (int t0 = gtid - lane; t0 < M.ntables; t0 += gth) {  // warp-uniform trip count
+                    const int t = t0 + lane;
+                    const bool dirty = t < M.ntables && __ldcg(&M.nodeStatus[t / M.nodeTables]) == CT_OK &&
+                                       table_dirty(M, t, pruned);
+                    const unsigned bal = __ballot_sync(0xffffffffu, dirty);
+                    if (!bal) continue;
                     int base = 0;
                     if (lane == 0) base = atomicAdd(nnext, __popc(bal));
                     base = __shfl_sync(0xffffffffu, base, 0);
                     if (dirty) next[base + __popc(bal & lanemask_lt())] = t;
                 }
-                if (kSearch && dirty) Sd.busy[t / M.nodeTables] = 1;  // its node goes on next round
             }
             for (int v = gtid; v < M.nvars; v += gth) prunedNext[v] = -1;
             if (blockIdx.x == 0 && tid == 0) {
@@ -1040,7 +1098,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) ct_model_kernel(const __
         }
         cur ^= 1;
         ++round;
-        if (!sync()) return;
+        if (!kSearch && !sync()) return;
         if (kSearch) {
             if (!search_step()) return;
             if (++launchRounds >= Sd.roundBudget) {
@@ -1211,12 +1269,13 @@ cudaError_t launch_model(const ModelDev& M, int grid, cudaStream_t s) {
     return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, 0, s);
 }
 
-// Search mode: 4 CTAs per SM with 8 row loads in flight (twice the warps of
-// the fixpoint launch: a round's units are many and short).
+// Search mode: 3 CTAs per SM with 8 row loads in flight (a round's units are
+// many and short; 512 slots of 14 tables: 4 CTAs at 64 registers 9.2 ms, 3 at 80
+// 8.7, 2 at 128 8.75, 1 9.9).
 int max_coresident_search_blocks() {
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ct_model_kernel<8, true, 4>, kThreads, 0) != cudaSuccess) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ct_model_kernel<8, true, 3>, kThreads, 0) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1226,7 +1285,7 @@ int max_coresident_search_blocks() {
 cudaError_t launch_model_search(const ModelDev& M, int grid, cudaStream_t s) {
     ModelDev m = M;
     void* args[] = {&m};
-    return cudaLaunchCooperativeKernel((const void*)ct_model_kernel<8, true, 4>, dim3(grid), dim3(kThreads), args, 0, s);
+    return cudaLaunchCooperativeKernel((const void*)ct_model_kernel<8, true, 3>, dim3(grid), dim3(kThreads), args, 0, s);
 }
 
 // Level 0 of every slot (one CTA per slot): the root domains, and for every
@@ -1259,7 +1318,6 @@ __global__ void ct_search_init_kernel(const __grid_constant__ ModelDev M, const 
         S.depth[s] = 0;
         S.given[s] = 0;
         S.active[s] = 0;
-        S.busy[s] = 0;
         S.rel[s] = 0;
         S.subSol[s] = 0;
         S.firstOpen[s] = 0x7fffffff;

@@ -435,7 +435,7 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
                     miss &= miss - 1u;
                     const int t = __shfl_sync(0xffffffffu, R.t, l), r = __shfl_sync(0xffffffffu, R.r, l);
                     const TableDev& T = tabs[t];
-                    const int o = probe_windows<true, kModelProbes>(T, r, __shfl_sync(0xffffffffu, R.res, l), s_cnt);
+                    const int o = probe_network(T, r, __shfl_sync(0xffffffffu, R.res, l), s_cnt);
                     if (lane == 0 && o == kProbeGone) remove(T, t, r);
                     else if (lane == 0 && o != kProbeFound) undecided(T, r);
                 }
@@ -452,7 +452,7 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
             for (int q = gwarp; q < nm; q += nwarps) {
                 const int4 e = __ldcg(&M.missQ[q]);
                 const TableDev& T = tabs[e.x];
-                const int o = probe_windows<true, kModelProbes>(T, e.y, e.z, s_cnt);
+                const int o = probe_network(T, e.y, e.z, s_cnt);
                 if (lane == 0 && o == kProbeGone) remove(T, e.x, e.y);
                 else if (lane == 0 && o != kProbeFound) undecided(T, e.y);
             }

@@ -400,7 +400,7 @@ int build_dsearch(ct_model* m, ct_batch* b, int levels, int trailFactor, DevSear
         (st = d_alloc(d, &S.given, B)) || (st = d_alloc(d, &S.rel, B)) || (st = d_alloc(d, &S.subSol, B)) ||
         (st = d_alloc(d, &S.path, (size_t)B * S.pathWords)) || (st = d_alloc(d, &S.firstPath, (size_t)B * S.pathWords)) ||
         (st = d_alloc(d, &S.idleList, B)) || (st = d_alloc(d, &S.giveList, B)) ||
-        (st = d_alloc(d, &S.busy, B)) || (st = d_alloc(d, &S.openIdx, B)) ||
+        (st = d_alloc(d, &S.openIdx, B)) ||
         (st = d_alloc(d, &S.frames, (size_t)B * L)) || (st = d_alloc(d, &S.levelDom, lv * DWs)) ||
         (st = d_alloc(d, &S.markAt, lv * T)) || (st = d_alloc(d, &S.liveAt, lv * T)) ||
         (st = d_alloc(d, &S.snapSeg, lv * S.segTotal)) || (st = d_alloc(d, &S.firstOpen, B)) ||
