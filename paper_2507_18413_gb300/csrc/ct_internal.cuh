@@ -71,6 +71,7 @@ enum StatusSlot {
     kSlotT4 = 20,  // finalize
     kSlotScan = 21,  // hard values left undecided by the windows (the full scan's)
     kSlotEarly = 22,  // 1: the filter ran beside the update (one grid barrier)
+    kSlotWords = 23,  // non-zero words of currTable (launch_count_words)
 };
 
 // Per-table control block: persistent state and per-call counters.
@@ -98,6 +99,7 @@ struct Ctrl {
     // counters above.
     alignas(128) uint32_t bar_count;  // grid barrier arrivals (only grows)
     uint32_t bar_base;                // grid barrier count at the start of the next launch
+    uint32_t nzWords, nzTicket;  // count of currTable's non-zero words under way (zero between launches)
     uint32_t bank[2][4];  // small-network kernel: live, live_in, words_in of a round by its parity (zero between launches)
 };
 
@@ -360,6 +362,8 @@ cudaError_t launch_save(const TableDev& T, int level, cudaStream_t s);
 cudaError_t launch_restore(const TableDev& T, int level, int mark, int top, int newMark, cudaStream_t s);
 cudaError_t launch_set_words(uint32_t* dst, const uint32_t* words, int n, cudaStream_t s);
 cudaError_t launch_copy_words(uint32_t* dst, const uint32_t* src, int n, cudaStream_t s);
+// currTable's non-zero words into the table's status block (kSlotWords).
+cudaError_t launch_count_words(const TableDev& T, cudaStream_t s);
 cudaError_t launch_read_ceiling(const uint4* p, size_t n16, cudaStream_t s);
 
 // Launchers of a table's construction (ct_build.cu). tup: device copies of the
