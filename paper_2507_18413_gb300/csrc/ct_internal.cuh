@@ -348,7 +348,9 @@ cudaError_t launch_clone_state(const TableDev* src, const TableDev* dst, int nsr
 // The propagation kernel is a cooperative launch of `grid` CTAs that must all
 // be resident at once (grid <= max_coresident_blocks(variant)).
 // variant: bit 0 = every CTA plans in shared memory, bit 1 = batches of 8 rows
-// with 3 CTAs per SM (else batches of 16 rows with 2 CTAs per SM).
+// with 3 CTAs per SM (else batches of 16 rows with 2 CTAs per SM), bit 2 = 16
+// rows with 1 CTA per SM (local plans).
+constexpr int kLoneVariant = 5;
 int max_coresident_blocks(int variant);
 cudaError_t launch_propagate(const TableDev& T, int variant, int grid, uint32_t* dom, const int32_t* domOff,
                              const CallParams& P, cudaStream_t s);

@@ -824,10 +824,12 @@ int coresident() {
 
 }  // namespace
 
-// variant: bit 0 = local plan, bit 1 = wide (8 loads in flight, 3 CTAs per SM)
+// variant: bit 0 = local plan, bit 1 = wide (8 loads in flight, 3 CTAs per SM),
+// bit 2 (with bit 0 alone) = 16 loads at one CTA per SM: 255 registers, no spills
 int max_coresident_blocks(int variant) {
     int r = 0;
-    switch (variant & 3) {
+    switch (variant) {
+        case 5: r = coresident<true, 16, 1>(); break;
         case 0: r = coresident<false, 16, 2>(); break;
         case 1: r = coresident<true, 16, 2>(); break;
         case 2: r = coresident<false, 8, 3>(); break;
@@ -839,7 +841,8 @@ int max_coresident_blocks(int variant) {
 
 cudaError_t launch_propagate(const TableDev& T, int variant, int grid, uint32_t* dom, const int32_t* domOff,
                              const CallParams& P, cudaStream_t s) {
-    switch (variant & 3) {
+    switch (variant) {
+        case 5: return launch_coop<true, 16, 1>(T, grid, dom, domOff, P, s);
         case 0: return launch_coop<false, 16, 2>(T, grid, dom, domOff, P, s);
         case 1: return launch_coop<true, 16, 2>(T, grid, dom, domOff, P, s);
         case 2: return launch_coop<false, 8, 3>(T, grid, dom, domOff, P, s);

@@ -658,6 +658,14 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
         // more segments than one wave of warps at 2 CTAs per SM: 8 loads at 3 CTAs per SM
         const int maxNarrow = max_coresident_blocks(narrow);
         ct->variant = (ct->nseg > maxNarrow * kWarps) ? (narrow | 2) : narrow;
+        // A warp per segment and one per value at one CTA per SM: the second CTA's
+        // warps find nothing to do, and its registers are better used (32 calls,
+        // one and two CTAs per SM: 25 segments of 192 values 671 and 686 us, 245
+        // 701 and 735, 611 715 and 761, 977 725 and 768; a warp short of that, two
+        // are better again: 1,197 segments 779 and 774, 1,465 818 and 773).
+        if (ct->localPlan && !(opt && opt->grid_blocks > 0) &&
+            ct->nseg + R <= max_coresident_blocks(kLoneVariant) * kWarps)
+            ct->variant = kLoneVariant;
         const int maxCo = max_coresident_blocks(ct->variant);
         if (maxCo <= 0) {
             ct_set_error("ct_create: the propagation kernel cannot be made resident on this device");
@@ -1144,7 +1152,7 @@ int autotune(ct_table* ct) {
     const int base = std::max((ct->nseg * ct->maxSplit + kWarps - 1) / kWarps, (ct->R + 2 * kWarps - 1) / (2 * kWarps));
     std::vector<std::pair<int, int>> cands;
     for (int wide = 0; wide < 2; ++wide) {
-        const int var = narrow | (wide ? 2 : 0);
+        const int var = wide ? narrow | 2 : ct->variant == kLoneVariant ? kLoneVariant : narrow;
         const int maxCo = max_coresident_blocks(var);
         if (maxCo <= 0) continue;
         for (int g : {base / 4, base / 2, base, 2 * base, maxCo / 2, maxCo}) {
