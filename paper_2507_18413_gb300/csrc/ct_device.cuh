@@ -784,6 +784,7 @@ __device__ __forceinline__ int probe_windows(const TableDev& T, int r, int res, 
                                              const int32_t* codes = nullptr, int nrows = 0) {
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
+    static_assert(!kLive || kE == 0, "a filter beside the update searches dense states only");
     bool complete = false;
     if (!kLive && T.useResidues) {
         // the chunks that follow the residue, dead or alive: two windows per
@@ -875,7 +876,7 @@ __device__ __forceinline__ int probe_windows(const TableDev& T, int r, int res, 
                 int chunk = 0;
                 if (q < total) {
                     chunk = sj * 32 + nth_set_bit(mj, q - before);
-                    h = nz(and4(ld_sup(row + chunk), probe_chunk<kE>(T, codes, nrows, chunk)));
+                    h = nz(and4(ld_sup(row + chunk), probe_chunk<0>(T, codes, nrows, chunk)));
                 }
                 tested += min(32, total - q0);
                 const unsigned bal = __ballot_sync(FULL, h);
@@ -919,10 +920,9 @@ __device__ __forceinline__ void note_probe(const TableDev& T, int r, int word, i
     atomicAdd(&s_cnt[kCntMiss], 1u);
 }
 
-template <bool kLive, int kProbes = kLocalProbes, int kE = 0>
-__device__ __forceinline__ void probe_miss(const TableDev& T, int r, int word, int bit, int res, uint32_t* s_cnt,
-                                           const int32_t* codes = nullptr, int nrows = 0) {
-    const int o = probe_windows<kLive, kProbes, kE>(T, r, res, s_cnt, codes, nrows);
+template <bool kLive, int kProbes>
+__device__ __forceinline__ void probe_miss(const TableDev& T, int r, int word, int bit, int res, uint32_t* s_cnt) {
+    const int o = probe_windows<kLive, kProbes>(T, r, res, s_cnt);
     if ((threadIdx.x & 31) == 0) note_probe(T, r, word, bit, o, s_cnt);
 }
 

@@ -242,14 +242,14 @@ __device__ __forceinline__ void probe_loaded(const TableDev& T, int r, int word,
 
 // A value of s_sup probed beside the update (r and res uniform over the
 // warp): its residue chunk and, on a miss, the windows after it, every chunk
-// recomputed from the call's row codes (chunk_after, E >= nrows rows). The
-// sparse/dense choice of windows is the state's at entry; when they leave the
-// value undecided and the update has made currTable sparse (the live count is
+// recomputed from the call's row codes (chunk_after, E >= nrows rows); the state
+// at entry is dense (the rule of `early`). When the windows leave the value
+// undecided and the update has made currTable sparse (the live count is
 // final once every CTA has released its update), the value is searched again
 // over the live chunks of the index the update left, after waiting for it.
 template <int E>
 __device__ __forceinline__ void probe_early(const TableDev& T, int r, int word, int bit, bool present, int res,
-                                            const int32_t* codes, int nrows, bool sparse, unsigned limit,
+                                            const int32_t* codes, int nrows, unsigned limit,
                                             uint32_t* s_cnt) {
     const int lane = threadIdx.x & 31;
     if (!present) return;
@@ -259,8 +259,7 @@ __device__ __forceinline__ void probe_early(const TableDev& T, int r, int word, 
         if (lane == 0) atomicAdd(&s_cnt[kCntHits], 1u);
         return;
     }
-    int o = sparse ? probe_windows<true, kModelProbes, E>(T, r, res, s_cnt, codes, nrows)
-                   : probe_windows<false, kLocalProbes, E>(T, r, res, s_cnt, codes, nrows);
+    int o = probe_windows<false, kLocalProbes, E>(T, r, res, s_cnt, codes, nrows);
     if (o == kProbeUndecided && wait_update_done(T.ctrl, limit) && 2u * __ldcg(&T.ctrl->live) < (uint32_t)T.W4)
         o = probe_windows<true, kModelProbes>(T, r, res, s_cnt);
     if (lane == 0) note_probe(T, r, word, bit, o, s_cnt);
@@ -578,9 +577,9 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             if (r != pfirstE && present && lane == 0) res = T.residue[r];
             res = __shfl_sync(0xffffffffu, res, 0);
             if (nrows <= 4)
-                probe_early<4>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.pcnt);
+                probe_early<4>(T, r, word, a & 31, present, res, sm.codes, nrows, bar.limit, sm.pcnt);
             else
-                probe_early<U>(T, r, word, a & 31, present, res, sm.codes, nrows, sparse, bar.limit, sm.pcnt);
+                probe_early<U>(T, r, word, a & 31, present, res, sm.codes, nrows, bar.limit, sm.pcnt);
         }
     } else if (kLocal) {
         for (int r = gwarp; r < T.R; r += nwarps) {
