@@ -67,6 +67,7 @@ struct FeatArgs {
     float4* pairStat;
     unsigned* ticket;
     int32_t pairs;
+    float* publish;  // mapped host memory, or null
 };
 
 __device__ __forceinline__ uint32_t popc4(const uint4& v) {
@@ -283,8 +284,10 @@ __global__ void ct_features_kernel(const FeatArgs A, int perNode) {
 // CTA adds the parts up per variable, in the order and with the operations of
 // ct_features_kernel. What bounds it is the chain of round trips of one CTA:
 // the two kernels above with their two memsets took 42 us per node on 25
-// variables and 40 tables of up to 157 chunks, this one 10. Tables of more
-// than kFeatChunks chunks keep them (their counts spread over the grid).
+// variables and 40 tables of up to 157 chunks, this one 10. For one network the
+// last CTA also writes the features where the host reads them, and a word that
+// the host waits for (a copy and a stream synchronisation took 6 us more of
+// ct_model_features' 28). Tables of more than kFeatChunks chunks keep them (their counts spread over the grid).
 constexpr int kFeatChunks = 256, kFeatValues = 1024, kFeatVars = 2048, kFeatThreads = 256;
 
 __global__ void __launch_bounds__(kFeatThreads) ct_features_small_kernel(const FeatArgs A) {
@@ -410,7 +413,18 @@ __global__ void __launch_bounds__(kFeatThreads) ct_features_small_kernel(const F
         }
 #pragma unroll
         for (int k = 0; k < kNF; ++k) A.feat[(size_t)v * kNF + k] = f[k];
+        if (A.publish) {
+            float4* out = reinterpret_cast<float4*>(A.publish) + 2 * lx;
+            out[0] = make_float4(f[0], f[1], f[2], f[3]);
+            out[1] = make_float4(f[4], f[5], f[6], f[7]);
+        }
     }
+    if (!A.publish) return;
+    // every thread's rows before the word the host waits for
+    __threadfence_system();
+    __syncthreads();
+    if (tid == 0)
+        asm volatile("st.release.sys.global.s32 [%0], %1;" ::"l"(A.publish + (size_t)A.V * kNF), "r"(1) : "memory");
 }
 
 // Offsets of the layers in the flat weight vector.
@@ -974,10 +988,18 @@ int ct_feat_view_build(FeatView* f, int nodes, const std::vector<std::vector<int
         (st = f_upload(f->pairVar, pairVar)) != CT_OK)
         return st;
     CT_CUDA(cudaMemset(f->ticket, 0, (size_t)std::max(nodes, 1) * sizeof(unsigned)));
-    if (cudaHostAlloc((void**)&f->h_scores, std::max(nv, 1) * sizeof(float), cudaHostAllocDefault) != cudaSuccess) {
+    const size_t nscores = (size_t)(std::max(nv, 1) + 3) & ~(size_t)3;  // (the features on a 16-byte boundary)
+    const bool publish = f->small && nodes == 1;
+    if (cudaHostAlloc((void**)&f->h_scores, (nscores + (publish ? (size_t)nv * kNF + 1 : 0)) * sizeof(float),
+                      publish ? cudaHostAllocMapped : cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
+        f->h_scores = nullptr;
         ct_set_error("features: pinned scores");
         return CT_ERR_OOM;
+    }
+    if (publish) {
+        f->h_feat = f->h_scores + nscores;
+        CT_CUDA(cudaHostGetDevicePointer((void**)&f->d_hfeat, f->h_feat, 0));
     }
     return CT_OK;
 }
@@ -987,12 +1009,12 @@ void ct_feat_view_free(FeatView* f) {
     for (void* p : f->allocs) cudaFree(p);
     f->allocs.clear();
     if (f->h_scores) cudaFreeHost(f->h_scores);
-    f->h_scores = nullptr;
+    f->h_scores = f->h_feat = f->d_hfeat = nullptr;
     cudaGetLastError();
 }
 
 int ct_feat_compute(FeatView* f, const TableDev* d_tabs, const uint32_t* dom, const uint8_t* nodeActive,
-                    cudaStream_t s) {
+                    cudaStream_t s, bool publish) {
     if (!f->counts) {
         ct_set_error("features: view not built");
         return CT_ERR_STATE;
@@ -1024,6 +1046,7 @@ int ct_feat_compute(FeatView* f, const TableDev* d_tabs, const uint32_t* dom, co
     A.pairStat = f->pairStat;
     A.ticket = f->ticket;
     A.pairs = f->pairs;
+    A.publish = publish ? f->d_hfeat : nullptr;
     if (f->small) {
         ct_features_small_kernel<<<f->nodes * f->pairs, kFeatThreads, 0, s>>>(A);
         CT_CUDA(cudaGetLastError());

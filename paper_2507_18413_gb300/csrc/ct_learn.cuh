@@ -41,6 +41,10 @@ struct FeatView {
     float* feat = nullptr;        // [nv][kNF]
     float* scores = nullptr;      // [nv]
     float* h_scores = nullptr;    // pinned copy of scores
+    // one-kernel path of one node, pinned and mapped: the features as the kernel
+    // publishes them, and behind them a word that it sets last
+    float* h_feat = nullptr;
+    float* d_hfeat = nullptr;     // (the device's address of it)
     int32_t nt = 0, nv = 0, nodes = 1, T = 0, V = 0, degmax = 1, totalUnits = 0, totalRows = 0;
     std::vector<void*> allocs;
 };
@@ -59,9 +63,10 @@ int ct_feat_view_build(ctk::FeatView* f, int nodes, const std::vector<std::vecto
 void ct_feat_view_free(ctk::FeatView* f);
 // Features of every variable of the view's nodes (node n only if nodeActive is
 // null or nodeActive[n] != 0), from the tables' current currTable and the
-// domains in `dom` (device). Stream-ordered; no synchronisation.
+// domains in `dom` (device). Stream-ordered; no synchronisation. publish (views
+// with h_feat): also into f->h_feat, its last word set when they are there.
 int ct_feat_compute(ctk::FeatView* f, const ctk::TableDev* d_tabs, const uint32_t* dom, const uint8_t* nodeActive,
-                    cudaStream_t s);
+                    cudaStream_t s, bool publish = false);
 // Scores of the view's variables with the network (after ct_feat_compute),
 // copied to f->h_scores; synchronises the stream.
 int ct_feat_scores(ctk::FeatView* f, const ct_mlp* mlp, cudaStream_t s);

@@ -12,6 +12,7 @@
 // schedules the other tables that share them. Either way one table pass is
 // GAC for that table, so a table is not re-queued by its own pruning.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cstring>
 #include <deque>
@@ -852,10 +853,32 @@ extern "C" int ct_model_features(ct_model* m, float* features_host) {
     }
     int st = ensure_features(m);
     if (st == CT_OK) st = sync_dom(m);
-    if (st == CT_OK) st = ct_feat_compute(m->fview, m->d_tabs, m->d_dom, nullptr, m->stream);
     if (st != CT_OK) return st;
-    CT_CUDA(cudaMemcpyAsync(features_host, m->fview->feat, (size_t)m->nvars * kNF * sizeof(float),
-                            cudaMemcpyDeviceToHost, m->stream));
+    // published by the kernel where it can, unless the stream is being captured
+    // (the launch would not run: the copy's synchronisation reports it)
+    FeatView* f = m->fview;
+    const size_t words = (size_t)m->nvars * kNF;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    bool seen = false;
+    if (f->h_feat) CT_CUDA(cudaStreamIsCapturing(m->stream, &capture));
+    const bool publish = f->h_feat && capture == cudaStreamCaptureStatusNone;
+    volatile int32_t* flag = reinterpret_cast<volatile int32_t*>(f->h_feat + (publish ? words : 0));
+    if (publish) *flag = 0;
+    if ((st = ct_feat_compute(f, m->d_tabs, m->d_dom, nullptr, m->stream, publish)) != CT_OK) return st;
+    if (publish) {
+        const auto t0 = std::chrono::steady_clock::now();
+        for (uint64_t it = 0; !seen; ++it) {
+            seen = *flag != 0;
+            if ((it & 1023u) == 1023u && std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(kHostWaitMs))
+                break;
+        }
+    }
+    if (seen) {
+        std::atomic_thread_fence(std::memory_order_acquire);
+        std::memcpy(features_host, f->h_feat, words * sizeof(float));
+        return CT_OK;
+    }
+    CT_CUDA(cudaMemcpyAsync(features_host, f->feat, words * sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     CT_CUDA(cudaStreamSynchronize(m->stream));
     return CT_OK;
 }

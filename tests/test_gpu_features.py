@@ -45,3 +45,26 @@ def test_features_match_the_oracle(sizes, t):
         if C.ct_model_propagate(m) != C.CT_OK:
             break
     C.ct_model_destroy(m)
+
+
+@pytest.mark.parametrize("nvars", [1, 2, 7, 255, 257, 601])
+def test_every_variable_is_published(nvars):
+    """One variable to several per thread, most of them in no table; called again without a change."""
+    torch = torch_cuda()
+    sizes = [3 + v % 4 for v in range(nvars)]
+    g = np.random.default_rng(nvars)
+    csp = O.Csp([0] * nvars, sizes)
+    st, m = C.ct_model_create([0] * nvars, sizes, stream=torch.cuda.current_stream())
+    assert st == C.CT_OK
+    for sc in {(0, nvars // 2, nvars - 1), (nvars - 1,)} if nvars > 2 else {(0,)}:
+        tup = np.stack([g.integers(0, sizes[v], 50) for v in sc], axis=1).astype(np.int32)
+        csp.add_table(list(sc), tup)
+        assert C.ct_model_add_table(m, list(sc), tup) >= 0
+    assert C.ct_model_propagate(m) == C.CT_OK
+    masks = C.words_to_masks(C.ct_model_get_domains(m, int(C.dom_layout(sizes)[0][-1]))[1], sizes)
+    want = L.features(csp, masks)
+    for _ in range(3):
+        st, got = C.ct_model_features(m, nvars)
+        assert st == C.CT_OK, C.last_error()
+        assert np.all(np.abs(got - want) <= 1e-5 * np.maximum(1.0, np.abs(want)))
+    C.ct_model_destroy(m)
