@@ -1244,16 +1244,16 @@ __global__ void ct_clone_state_kernel(const TableDev* __restrict__ src, const Ta
 
 }  // namespace
 
-// Launches of many tables (the batched searches' copies of a network) run 4
+// Launches of many tables (the batched searches' copies of a network) run 3
 // CTAs per SM with 8 row loads in flight: a round's units are many and short,
-// and twice the warps keep twice the loads in flight (batched search 1.2-1.3x
-// nodes/s); smaller networks keep 2 CTAs per SM with 16 loads (4 CTAs per SM
-// measured 6-7% slower there).
+// and more warps keep more loads in flight (4 CTAs per SM at 64 registers: 20.2
+// ms for a host-driven search of 512 slots where 3 at 80 take 19.2, 24.4 and
+// 22.8 with 128 slots); smaller networks keep 2 CTAs per SM with 16 loads.
 constexpr int kManyTables = 1024;
 
 int max_coresident_model_blocks(int ntables) {
     int dev = 0, sms = 0, per = 0;
-    const void* k = ntables >= kManyTables ? (const void*)ct_model_kernel<8, false, 4> : (const void*)ct_model_kernel<16, false>;
+    const void* k = ntables >= kManyTables ? (const void*)ct_model_kernel<8, false, 3> : (const void*)ct_model_kernel<16, false>;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kThreads, 0) != cudaSuccess) {
         cudaGetLastError();
@@ -1265,7 +1265,7 @@ int max_coresident_model_blocks(int ntables) {
 cudaError_t launch_model(const ModelDev& M, int grid, cudaStream_t s) {
     ModelDev m = M;
     void* args[] = {&m};
-    const void* k = M.ntables >= kManyTables ? (const void*)ct_model_kernel<8, false, 4> : (const void*)ct_model_kernel<16, false>;
+    const void* k = M.ntables >= kManyTables ? (const void*)ct_model_kernel<8, false, 3> : (const void*)ct_model_kernel<16, false>;
     return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, 0, s);
 }
 
