@@ -284,6 +284,7 @@ int batch_propagate(ct_model* m) {
             break;
     }
     if (!seen) CT_CUDA(cudaStreamSynchronize(m->stream));
+    std::atomic_thread_fence(std::memory_order_acquire);  // the results after the word that publishes them
     m->stats.wait_seconds += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     const int status = H[0];
     if (status == kNoChunk) {

@@ -16,6 +16,7 @@
 // only its own slot's node. A slot whose subtree is done takes the next open
 // node, or the untried right branch nearest the root of another slot.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -946,6 +947,7 @@ struct Search {
                 break;
         }
         if (!seen) CT_CUDA(cudaStreamSynchronize(b->stream));
+        std::atomic_thread_fence(std::memory_order_acquire);  // the results after the word that publishes them
         info.wait_seconds += std::chrono::duration<double>(std::chrono::steady_clock::now() - w0).count();
         const int status = H[0];
         if (status != CT_OK) {
@@ -1144,6 +1146,7 @@ struct Search {
                 }
             }
             if (!seen) CT_CUDA(cudaStreamSynchronize(str));
+            std::atomic_thread_fence(std::memory_order_acquire);  // the results after the word that publishes them
             info.wait_seconds += std::chrono::duration<double>(std::chrono::steady_clock::now() - w0).count();
             info.steps += 1;
             const int status = H[0];

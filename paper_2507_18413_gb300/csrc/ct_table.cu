@@ -2,6 +2,7 @@
 // device layout (Sec. 3 constructor, Sec. 4 device copies), propagation calls,
 // backtrack levels and inspection.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cstdarg>
 #include <cstddef>
@@ -894,6 +895,7 @@ int ct_table_propagate_on(ct_table* ct, uint32_t* dom, const int32_t* domOffDev,
         }
     }
     if (!seen) CT_CUDA(cudaStreamSynchronize(s));
+    std::atomic_thread_fence(std::memory_order_acquire);  // the results after the word that publishes them
     if (ct->copyState) {
         // ... and back to the host after it
         CT_CUDA(cudaMemcpyAsync(ct->h_curr, ct->dev.curr, (size_t)ct->W4 * sizeof(uint4), cudaMemcpyDeviceToHost, s));
