@@ -93,7 +93,9 @@ typedef struct ct_options {
                                  chunks are live filters beside the update, each probed chunk
                                  recomputed from its stored value and the call's rows (Algorithm 2 at
                                  one chunk), and one grid barrier ends both; positive tables with
-                                 residues and a plan in shared memory. Results are the same. */
+                                 residues and a plan in shared memory, of more than 128 chunks (below,
+                                 one CTA propagates the table and its filter always follows the
+                                 update). Results are the same. */
 } ct_options;
 
 /* Static shape and live state of a table (ct_get_info). */
@@ -112,7 +114,7 @@ typedef struct ct_table_info {
     int32_t grid_blocks;   /* CTAs of the propagation launch */
     int32_t short_tuples;  /* retained tuples with at least one CT_STAR component */
     int64_t device_bytes;  /* device memory held by the table */
-    int32_t loads_in_flight; /* 16 (2 CTAs per SM) or 8 (3 CTAs per SM) row loads per lane */
+    int32_t loads_in_flight; /* 16 (1 or 2 CTAs per SM) or 8 (3 CTAs per SM) row loads per lane */
     int32_t autotuned;     /* 1 if the launch shape was chosen by trial propagations */
 } ct_table_info;
 
@@ -126,7 +128,8 @@ typedef struct ct_call_stats {
     int32_t sup_vars;       /* |s_sup|: scope variables with more than one value */
     int32_t residue_hits;   /* values found supported by their residue chunk */
     int32_t local_found;    /* values found in the 32-chunk windows after a missed residue */
-    int32_t hard;           /* values that needed the full index scan */
+    int32_t hard;           /* values that neither the residue nor the windows support: removed where the
+                               windows covered every chunk, else decided by a scan of the whole index */
     int32_t windows;        /* 32-chunk windows probed */
     int32_t pruned;         /* values removed by filterDomains */
     int32_t trail_added;    /* trail entries appended */

@@ -44,6 +44,8 @@
 // waits (bounded) for the whole update and is searched again over the index
 // it left when currTable has become sparse; the finalizing CTA writes lastDom
 // (no CTA may write it before every plan is done).
+// Tables of at most 128 chunks and 512 values with narrow scopes run on one CTA
+// instead (ct_small.cu).
 // Grid barriers spin with a bounded iteration count; running out sets
 // CT_ERR_TIMEOUT in the control block and every CTA returns.
 #include <cstddef>

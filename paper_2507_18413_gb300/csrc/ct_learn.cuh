@@ -13,7 +13,7 @@ namespace ctk {
 constexpr int kNF = 8;    // features per variable
 constexpr int kNH = 64;   // hidden units per layer
 constexpr int kNW = kNH * kNF + kNH + kNH * kNH + kNH + kNH + 1;  // 4801 weights
-constexpr int kTrainBatch = 128;  // largest training batch (one CTA holds it in shared memory)
+constexpr int kTrainBatch = 128;  // largest training batch (held in shared memory over a cluster of 8 CTAs)
 
 // A network view for the feature kernels: `nodes` independent copies of a
 // network of T tables over V variables (table k of node n is n * T + k,
