@@ -431,6 +431,11 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
             }
         }
         const int units = T.nseg << lg;
+        // Rows per batch of the longest lists: at one CTA per SM a warp walks a list
+        // that two CTAs' warps shared (977 segments, 90 rows: update 13.1 us with
+        // batches of 16, 12.2 with 32; split lists, 23 rows on 245 segments, stay
+        // with 16: 6.9 us against 8.2).
+        constexpr int kLong = kMinBlocks == 1 ? 2 * U : U;
         const int per = (nrows + G - 1) >> lg;  // rows per slice
         __syncthreads();
         CT_STAMP(20);
@@ -474,9 +479,14 @@ ct_propagate_kernel(const __grid_constant__ TableDev T, uint32_t* __restrict__ d
                 const bool act = (S.mask >> lane) & 1u;
                 // (four rows or fewer: a batch of their size, not U rows predicated
                 // off; 100,000 tuples 675 -> 650 us for 32 calls, 4e6 855 -> 810)
-                if (S.mask != 0u)
-                    acc = nrows <= 4 ? slice_rows<4, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0)
-                                     : slice_rows<U, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0);
+                if (S.mask != 0u) {
+                    if (nrows <= 4)
+                        acc = slice_rows<4, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0);
+                    else if (kLong > U && nrows > kLong)
+                        acc = slice_rows<kLong, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0);
+                    else
+                        acc = slice_rows<U, false, false>(T, seg, act, S.cur, 0, nrows, sm.codes, nullptr, 0);
+                }
             } else {
                 if (S.mask != 0u) {
                     const int qa = min(nrows, slice * per);
