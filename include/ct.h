@@ -396,8 +396,17 @@ int ct_model_add_table(ct_model* m, const int32_t* scope, int arity,
 int ct_model_add_negative_table(ct_model* m, const int32_t* scope, int arity, const int32_t* tuples, int64_t t);
 
 /* ct_model_propagate: run table propagations until no domain changes
- * (fixpoint) or a table fails (CT_INFEASIBLE). */
+ * (fixpoint) or a table fails (CT_INFEASIBLE). CT_ERR_TIMEOUT when a bounded
+ * device-side wait ran out: the model is unusable then (every later
+ * propagation, restore and search of it fails; destroy it). */
 int ct_model_propagate(ct_model* m);
+
+/* ct_model_arm_wait_timeout: ct_arm_wait_timeout for a model's one-launch
+ * fixpoint: every barrier wait of the next launch runs out after `polls` polls
+ * (> 0), the kernel returns without publishing and that ct_model_propagate
+ * returns CT_ERR_TIMEOUT. CT_ERR_ARG for a model whose fixpoint runs on the
+ * host (ct_options.host_fixpoint). */
+int ct_model_arm_wait_timeout(ct_model* m, uint32_t polls);
 
 /* ct_model_get_domains / ct_model_set_domains: host copies of all domains
  * (sum over variables of ceil(dom_size/32) words). Set domains must be

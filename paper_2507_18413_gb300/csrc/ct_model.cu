@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cstddef>
 #include <cstring>
 #include <deque>
 #include <vector>
@@ -271,9 +272,19 @@ int batch_propagate(ct_model* m) {
     m->domStale = false;
     volatile int32_t* H = m->h_mstatus;
     H[0] = kNoChunk;
+    ModelDev M = m->md;
+    if (m->armPolls) {
+        // Test hook (ct_model_arm_wait_timeout): no barrier of this launch completes
+        // (an arrival count 2^30 behind every target), each wait ends after armPolls polls.
+        const uint32_t unreachable[2] = {0xC0000000u, 0u};  // bar_count, bar_base
+        static_assert(offsetof(ModelCtrl, bar_base) == offsetof(ModelCtrl, bar_count) + sizeof(uint32_t), "adjacent words");
+        CT_CUDA(cudaMemcpyAsync(&M.ctrl->bar_count, unreachable, sizeof(unreachable), cudaMemcpyHostToDevice, m->stream));
+        M.spinLimit = m->armPolls;
+        m->armPolls = 0;
+    }
     const auto t0 = std::chrono::steady_clock::now();
-    CT_CUDA(m->net ? launch_net(m->md, inl ? m->h_blk : nullptr, (int)blkWords, m->grid, m->stream)
-                   : launch_model(m->md, m->grid, m->stream));
+    CT_CUDA(m->net ? launch_net(M, inl ? m->h_blk : nullptr, (int)blkWords, m->grid, m->stream)
+                   : launch_model(M, m->grid, m->stream));
     bool seen = false;
     for (uint64_t it = 0;; ++it) {
         if (H[0] != kNoChunk) {
@@ -288,9 +299,12 @@ int batch_propagate(ct_model* m) {
     m->stats.wait_seconds += std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     const int status = H[0];
     if (status == kNoChunk) {
+        // The kernel returned half-way: its tables' trails, last-seen domains and
+        // counters are whatever its CTAs had reached, and the host has none of the
+        // results, so no table can be propagated or restored from here.
+        for (ct_table* tab : m->tables) tab->failed = tab->broken = true;
+        m->failed = m->broken = true;
         ct_set_error("model: the fixpoint kernel did not publish (a device-side wait ran out)");
-        m->batch = false;
-        m->failed = true;
         return CT_ERR_TIMEOUT;
     }
     m->propagations += H[2];
@@ -555,6 +569,10 @@ extern "C" int ct_model_propagate(ct_model* m) {
         ct_set_error("ct_model_propagate: null handle");
         return CT_ERR_ARG;
     }
+    if (m->broken) {
+        ct_set_error("ct_model_propagate: the model is unusable after a device-side timeout");
+        return CT_ERR_TIMEOUT;
+    }
     if (m->failed) {
         ct_set_error("ct_model_propagate: the model failed; restore a level first");
         return CT_ERR_STATE;
@@ -604,6 +622,15 @@ extern "C" int ct_model_propagate(ct_model* m) {
             mark_var(m, v, self, &q);
         }
     }
+    return CT_OK;
+}
+
+extern "C" int ct_model_arm_wait_timeout(ct_model* m, uint32_t polls) {
+    if (!m || polls == 0 || !m->batch || (int)m->tables.size() > kModelMaxTables) {
+        ct_set_error("ct_model_arm_wait_timeout: polls must be positive, and the model's fixpoint one launch");
+        return CT_ERR_ARG;
+    }
+    m->armPolls = polls;
     return CT_OK;
 }
 

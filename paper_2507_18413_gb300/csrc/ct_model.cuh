@@ -50,6 +50,8 @@ struct ct_model {
     std::vector<void*> allocs;
     int grid = 1;
     bool net = false;  // the small-network kernel runs the fixpoints
+    bool broken = false;    // a device-side wait ran out: the model is unusable
+    uint32_t armPolls = 0;  // test hook: the next launch's barrier waits run out after this many polls
     ct_batch* bsearch = nullptr;  // built by the first batched search, kept for the next ones
     bool hasNegative = false;     // a negative table: no ordering features or lookahead labels
     // learned branching order

@@ -123,6 +123,7 @@ _SIGS = {
     "ct_destroy": (ctypes.c_int, [_P]),
     "ct_propagate_noalloc": (ctypes.c_int, [ctypes.c_int, _I32P, ctypes.c_int64, _P, _P, _P, _P, _U32P, _P]),
     "ct_arm_wait_timeout": (ctypes.c_int, [_P, ctypes.c_uint32]),
+    "ct_model_arm_wait_timeout": (ctypes.c_int, [_P, ctypes.c_uint32]),
     "ct_read_ceiling": (ctypes.c_int, [_P, ctypes.c_int64, _P, ctypes.POINTER(ctypes.c_float)]),
     "ct_debug_guard_buffers": (ctypes.c_int, [ctypes.c_int]),
     "ct_debug_check_guards": (ctypes.c_int, [_P, ctypes.c_int, _I64P]),
@@ -420,6 +421,12 @@ def ct_arm_wait_timeout(h, polls):
     """Test hook: the next ct_propagate on h (None: the next ct_propagate_noalloc) runs
     its barrier waits out after `polls` polls and returns CT_ERR_TIMEOUT."""
     return load().ct_arm_wait_timeout(h, int(polls))
+
+
+def ct_model_arm_wait_timeout(m, polls):
+    """Test hook: the next fixpoint launch of model m runs its barrier waits out
+    after `polls` polls; that ct_model_propagate returns CT_ERR_TIMEOUT."""
+    return load().ct_model_arm_wait_timeout(m, int(polls))
 
 
 def ct_propagate_host(h, dom_words: np.ndarray, changed_words: int = 0):
