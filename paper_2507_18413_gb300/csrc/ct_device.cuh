@@ -136,31 +136,35 @@ __device__ __forceinline__ void bar_init(GridBarrier& b, unsigned* count, unsign
     b.target = threadIdx.x == 0 ? ld_relaxed(base) : 0u;
 }
 
+// The two halves of a barrier, for thread 0: the arrival (true: the last one)
+// and the bounded wait (false: it ran out, CT_ERR_TIMEOUT is set). A CTA with
+// nothing left to do after a barrier need not wait for it.
+__device__ __forceinline__ bool bar_arrive(GridBarrier& b) {
+    unsigned arrived;
+    b.target += gridDim.x;
+    // Release this CTA's writes (ordered before by the CTA barrier) and, for
+    // the last arrival, acquire everybody else's.
+    asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(b.count) : "memory");
+    if (arrived != b.target - 1u) return false;
+    *b.base = b.target;  // read by the next launch only
+    return true;
+}
+
+__device__ __forceinline__ bool bar_wait(const GridBarrier& b) {
+    unsigned it = 0;
+    while ((int)(ld_acquire(b.count) - b.target) < 0) {
+        if (++it > b.limit) {
+            atomicExch(b.status, CT_ERR_TIMEOUT);
+            return false;
+        }
+        if (it > 64) __nanosleep(32);
+    }
+    return true;
+}
+
 __device__ int bar_sync(GridBarrier& b, int* s_flag) {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int r = 1;
-        unsigned arrived;
-        b.target += gridDim.x;
-        // Release this CTA's writes (ordered before by the CTA barrier) and, for
-        // the last arrival, acquire everybody else's.
-        asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(b.count) : "memory");
-        if (arrived == b.target - 1u) {
-            *b.base = b.target;  // read by the next launch only
-            r = 2;
-        } else {
-            unsigned it = 0;
-            while ((int)(ld_acquire(b.count) - b.target) < 0) {
-                if (++it > b.limit) {
-                    r = 0;
-                    atomicExch(b.status, CT_ERR_TIMEOUT);
-                    break;
-                }
-                if (it > 64) __nanosleep(32);
-            }
-        }
-        *s_flag = r;
-    }
+    if (threadIdx.x == 0) *s_flag = bar_arrive(b) ? 2 : bar_wait(b) ? 1 : 0;
     __syncthreads();
     return *s_flag;
 }

@@ -543,71 +543,36 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
     if (failed) ++round;
     phase(6);
 
-    // publish: CTA 0, the status word last
-    // (of the tables, those that ran: bit t of the words after the node status; a
-    // table's two words and the host's bookkeeping for them cost 2-5 us a call on 512 tables)
-    if (blockIdx.x == 0) {
-        int32_t* H = M.statusBlk;
-        int st = CT_OK;
-        uint32_t hits = 0u, local = 0u, hard = 0u, windows = 0u;
-        unsigned long long bf = 0ull;
-        if (tid == 0) {  // (on the way with the rest)
-            st = __ldcg(&C->status);
-            hits = __ldcg(&C->hits);
-            local = __ldcg(&C->local);
-            hard = __ldcg(&C->hard);
-            windows = __ldcg(&C->windows);
-            bf = __ldcg(&C->bytesFilter);
-        }
-        uint32_t* outDom = reinterpret_cast<uint32_t*>(H + kModelHdr + 2 * n);
-        for (int q0 = tid; q0 < M.DWg; q0 += 8 * kThreads) {
-            uint32_t w[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (q0 + u * kThreads < M.DWg) w[u] = __ldcg(&M.dom[q0 + u * kThreads]);
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (q0 + u * kThreads < M.DWg) outDom[q0 + u * kThreads] = w[u];
-        }
-        for (int t = tid; t < n; t += kThreads) {
-            if (!bit_of(done, t)) continue;
-            const Ctrl* Tc = tabs[t].ctrl;
-            const int top = __ldcg(&Tc->trail_top), live = __ldcg(&Tc->live_state);
-            H[kModelHdr + 2 * t] = top;
-            H[kModelHdr + 2 * t + 1] = live;
-        }
-        int32_t* outNode = H + kModelHdr + 2 * n + M.DWg;
-        for (int q = tid; q < (n + 31) / 32; q += kThreads) outNode[1 + q] = (int32_t)done[q];
-        __syncthreads();
-        if (tid == 0) {
-            outNode[0] = failed && st == CT_OK ? CT_INFEASIBLE : CT_OK;
-            H[1] = round;
-            H[2] = props;
-            H[3] = (int32_t)hits;
-            H[4] = (int32_t)local;
-            H[5] = (int32_t)hard;
-            H[6] = (int32_t)windows;
-            bf += 4ull * hits + 512ull * windows;
-            const unsigned long long bu = s_bytes[0];
-            H[8] = (int32_t)(bu & 0xffffffffull);
-            H[9] = (int32_t)(bu >> 32);
-            H[10] = (int32_t)(bf & 0xffffffffull);
-            H[11] = (int32_t)(bf >> 32);
-            phase(7);
-            st_release_sys(&H[0], st);
-        }
-    }
-    // Behind the publication, before the next launch of the stream: the tables'
-    // state as other kernels expect it (last-seen domains in lastDom) and the
-    // counters clear; every CTA is past its last read of them.
-    for (int t = gwarp; t < n; t += nwarps) {
+    // The tables' state as other kernels expect it: last-seen domains in lastDom,
+    // counters clear (every CTA is past its last read of them). The host may
+    // start anything once it has the status word, so all of it is done before:
+    // by the CTAs that do not publish, beside the publication, which waits for
+    // their arrivals before its last store.
+    const int idle = gridDim.x > 1 ? kWarps : 0;  // warps of CTA 0, which publishes
+    for (int t = gwarp - idle; t < n; t += nwarps - idle) {
+        if (t < 0) break;
         const TableDev& T = tabs[t];
         if (bit_of(flip, t))
             for (int q = lane; q < T.DW; q += 32) T.lastDom[q] = __ldcg(reinterpret_cast<uint32_t*>(T.codes) + q);
         if (lane < 8) (&T.ctrl->bank[0][0])[lane] = 0u;
         if (lane == 8) T.ctrl->nrows = 0;
     }
-    if (gtid == 0) {
+    if (blockIdx.x != 0) {
+        __syncthreads();
+        if (tid == 0) bar_arrive(bar);
+        return;
+    }
+    // publish: CTA 0, the status word last
+    // (of the tables, those that ran: bit t of the words after the node status; a
+    // table's two words and the host's bookkeeping for them cost 2-5 us a call on 512 tables)
+    int32_t* H = M.statusBlk;
+    int st = CT_OK;
+    bool last = false;
+    if (tid == 0) {
+        st = __ldcg(&C->status);
+        const uint32_t hits = __ldcg(&C->hits), local = __ldcg(&C->local), hard = __ldcg(&C->hard);
+        const uint32_t windows = __ldcg(&C->windows);
+        const unsigned long long bf = __ldcg(&C->bytesFilter) + 4ull * hits + 512ull * windows, bu = s_bytes[0];
         C->hits = C->local = C->hard = C->windows = 0u;
         C->bytesFilter = 0ull;
         C->nmiss[0] = C->nmiss[1] = 0;
@@ -615,6 +580,43 @@ ct_net_kernel(const __grid_constant__ ModelDev M, const __grid_constant__ NetCal
         C->status = CT_OK;
         C->nwork = 0;
         M.nodeStatus[0] = CT_OK;
+        last = bar_arrive(bar);  // (the header's stores go to the host meanwhile)
+        H[kModelHdr + 2 * n + M.DWg] = failed && st == CT_OK ? CT_INFEASIBLE : CT_OK;
+        H[1] = round;
+        H[2] = props;
+        H[3] = (int32_t)hits;
+        H[4] = (int32_t)local;
+        H[5] = (int32_t)hard;
+        H[6] = (int32_t)windows;
+        H[8] = (int32_t)(bu & 0xffffffffull);
+        H[9] = (int32_t)(bu >> 32);
+        H[10] = (int32_t)(bf & 0xffffffffull);
+        H[11] = (int32_t)(bf >> 32);
+    }
+    uint32_t* outDom = reinterpret_cast<uint32_t*>(H + kModelHdr + 2 * n);
+    for (int q0 = tid; q0 < M.DWg; q0 += 8 * kThreads) {
+        uint32_t w[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (q0 + u * kThreads < M.DWg) w[u] = __ldcg(&M.dom[q0 + u * kThreads]);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (q0 + u * kThreads < M.DWg) outDom[q0 + u * kThreads] = w[u];
+    }
+    for (int t = tid; t < n; t += kThreads) {
+        if (!bit_of(done, t)) continue;
+        const Ctrl* Tc = tabs[t].ctrl;
+        const int top = __ldcg(&Tc->trail_top), live = __ldcg(&Tc->live_state);
+        H[kModelHdr + 2 * t] = top;
+        H[kModelHdr + 2 * t + 1] = live;
+    }
+    int32_t* outRan = H + kModelHdr + 2 * n + M.DWg + 1;
+    for (int q = tid; q < (n + 31) / 32; q += kThreads) outRan[q] = (int32_t)done[q];
+    if (tid == 0 && !last) last = bar_wait(bar);
+    __syncthreads();
+    if (tid == 0 && last) {
+        phase(7);
+        st_release_sys(&H[0], st);
     }
 }
 
