@@ -185,6 +185,8 @@ typedef struct ct_profile {
  * check, Sec. 3); the handle is still valid and every propagation of it
  * fails. The first ct_propagate starts from the initial domains, so values
  * already removed by the caller count as removed since the last call.
+ * While the table is built, device scratch for the tuples (up to 256 MB, less
+ * or host memory where the device is short) is held beside its buffers.
  */
 /* ct_create_negative: a negative table (the tuples are the FORBIDDEN ones), the
  * extension of Compact-Table to negative tables that the paper cites (Sec. 1)
@@ -650,12 +652,17 @@ int ct_search_collect(ct_model* m, int64_t node_limit, int slots, int64_t max_sa
  * returns CT_ERR_OOM and releases what it took); one failure per arming;
  * n < 0 disarms.
  *
+ * ct_debug_limit_bytes: as on a device with `bytes` bytes for table buffers and
+ * the scratch of constructions: what would take them beyond it fails as if the
+ * device were out of memory (bytes < 0: no limit).
+ *
  * ct_debug_device_bytes: bytes of device memory the table buffers hold now,
  * over all tables, counted by the library's allocator (CT_ERR_ARG if
  * bytes_out is null). */
 int ct_debug_guard_buffers(int on);
 int ct_debug_check_guards(ct_table* ct, int poke, int64_t* changed_out);
 int ct_debug_fail_alloc(int n);
+int ct_debug_limit_bytes(int64_t bytes);
 int ct_debug_device_bytes(int64_t* bytes_out);
 
 /* ---------------------------------------------------------------- misc -- */

@@ -110,6 +110,8 @@ struct DevBuf {
 std::mutex g_bufMu;
 std::unordered_map<void*, DevBuf> g_bufs;  // buffer as the table sees it -> size
 int64_t g_bufBytes = 0;
+int64_t g_stageBytes = 0;                  // device scratch of constructions under way
+int64_t g_limitBytes = -1;                 // ct_debug_limit_bytes: a device of this many bytes (-1: the real one)
 bool g_guardNew = false;                   // ct_debug_guard_buffers
 long long g_failAfter = -1;                // ct_debug_fail_alloc: allocations left before one fails
 
@@ -118,14 +120,18 @@ struct BufAsk {
     size_t bytes;
 };
 
+// Whether n more device bytes are beyond the test hook's limit (under g_bufMu).
+bool beyond_limit(int64_t n) { return g_limitBytes >= 0 && g_bufBytes + g_stageBytes + n > g_limitBytes; }
+
 // The buffers of `ask` in one allocation, all or none (each counts as one
-// allocation of the failure countdown).
-cudaError_t table_malloc_all(const std::vector<BufAsk>& ask) {
+// allocation of the failure countdown; *injected: it was the countdown that failed it).
+cudaError_t table_malloc_all(const std::vector<BufAsk>& ask, bool* injected = nullptr) {
     std::lock_guard<std::mutex> lk(g_bufMu);
     for (const BufAsk& a : ask) *a.p = nullptr;
     if (g_failAfter >= 0) {
         if (g_failAfter < (long long)ask.size()) {
             g_failAfter = -1;
+            if (injected) *injected = true;
             return cudaErrorMemoryAllocation;
         }
         g_failAfter -= (long long)ask.size();
@@ -133,8 +139,12 @@ cudaError_t table_malloc_all(const std::vector<BufAsk>& ask) {
     const bool guarded = g_guardNew;
     const size_t guard = guarded ? kGuardBytes : 0;
     auto room = [&](size_t bytes) { return ((bytes + 255) & ~size_t(255)) + 2 * guard; };
-    size_t total = 0;
-    for (const BufAsk& a : ask) total += room(a.bytes);
+    size_t total = 0, sum = 0;
+    for (const BufAsk& a : ask) {
+        total += room(a.bytes);
+        sum += a.bytes;
+    }
+    if (beyond_limit((int64_t)sum)) return cudaErrorMemoryAllocation;
     char* base = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), total);
     if (e != cudaSuccess) return e;
@@ -181,6 +191,7 @@ void table_free(void* p) {
 struct TableBufs {
     ct_table* ct;
     std::vector<BufAsk> ask;
+    bool injected = false;  // the last take() failed by the test hook's countdown
     template <typename T>
     void want(T** p, size_t count) {
         ask.push_back({reinterpret_cast<void**>(const_cast<std::remove_const_t<T>**>(p)), std::max<size_t>(count, 1) * sizeof(T)});
@@ -188,7 +199,7 @@ struct TableBufs {
     int take() {
         size_t bytes = 0;
         for (const BufAsk& a : ask) bytes += a.bytes;
-        const cudaError_t e = table_malloc_all(ask);
+        const cudaError_t e = table_malloc_all(ask, &injected);
         if (e != cudaSuccess) {
             cudaGetLastError();
             ct_set_error("device buffers of a table (%zu bytes): %s", bytes, cudaGetErrorString(e));
@@ -390,56 +401,111 @@ void free_table(ct_table* ct) {
     delete ct;
 }
 
-// The tuple list on the device while a table is built, with the layout its
-// kernels need: a bounded scratch buffer (kStageInts components; lists beyond it
-// go through in chunks), freed when the construction ends. Not one of the
-// table's buffers.
+// The tuple list while a table is built, with the layout its kernels need: a
+// bounded scratch buffer on the device (kStageInts components; lists beyond it go
+// through in chunks), given back when the rows are built. Not one of the table's
+// buffers, and never the reason that a table does not fit: it gets smaller where
+// memory is short, steps aside for the table's buffers (close, then open again),
+// and where the device has no room for 1,024 tuples it is mapped host memory,
+// which the kernels read.
 struct TupleStage {
     static constexpr int64_t kStageInts = 1LL << 26;  // 256 MB
-    char* base = nullptr;
+    char* base = nullptr;  // as the kernels address it
+    char* host = nullptr;  // ... and the host, when it is mapped host memory
+    int64_t bytes = 0;     // device bytes held
+    cudaStream_t stream = nullptr;
     int32_t* lo = nullptr;
     int32_t* row0 = nullptr;
     unsigned long long* counts = nullptr;
     int32_t* tup = nullptr;
     int64_t cap = 0;              // tuples per chunk (a multiple of 1,024)
-    const int32_t* held = nullptr;  // host list whose chunk at heldAt is on the device
+    const int32_t* held = nullptr;  // host list whose chunk at heldAt is in the stage
     int64_t heldAt = 0;
     std::vector<int32_t> meta;  // what lo and row0 are copied from (kept until the copy is done)
-    ~TupleStage() {
-        if (base) cudaFree(base);
+    ~TupleStage() { close(); }
+    void close() {
+        if (host) {
+            cudaStreamSynchronize(stream);  // (a kernel may still read it)
+            cudaFreeHost(host);
+        } else if (base) {
+            cudaFree(base);
+        }
+        if (bytes > 0) {
+            std::lock_guard<std::mutex> lk(g_bufMu);
+            g_stageBytes -= bytes;
+        }
+        base = host = nullptr;
+        held = nullptr;
+        bytes = 0;
+    }
+    cudaError_t take_device(size_t n) {
+        {
+            std::lock_guard<std::mutex> lk(g_bufMu);
+            if (beyond_limit((int64_t)n)) return cudaErrorMemoryAllocation;
+            g_stageBytes += (int64_t)n;
+        }
+        bytes = (int64_t)n;
+        const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), n);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            base = nullptr;
+            close();
+        }
+        return e;
     }
     // Room for t tuples of n components, or as many as memory allows.
     int open(const ct_table* ct, int64_t t) {
         const int n = ct->arity;
+        stream = ct->stream;
         const int64_t whole = (t + 1023) / 1024 * 1024;
         cap = std::max<int64_t>(1024, std::min(whole, kStageInts / n / 1024 * 1024));
         const size_t head = ((size_t)(2 * n + 1) * sizeof(int32_t) + 2 * sizeof(unsigned long long) + 511) & ~size_t(255);
-        for (;; cap = std::max<int64_t>(1024, cap / 2 / 1024 * 1024)) {
-            const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&base), head + (size_t)cap * n * sizeof(int32_t));
-            if (e == cudaSuccess) break;
-            cudaGetLastError();
-            base = nullptr;
+        while (take_device(head + (size_t)cap * n * sizeof(int32_t)) != cudaSuccess) {
             if (cap == 1024) {
-                ct_set_error("ct_create: device scratch for the tuples: %s", cudaGetErrorString(e));
-                return CT_ERR_OOM;
+                const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&host), head + (size_t)cap * n * sizeof(int32_t),
+                                                    cudaHostAllocMapped);
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    host = nullptr;
+                    ct_set_error("ct_create: scratch for the tuples: %s", cudaGetErrorString(e));
+                    return CT_ERR_OOM;
+                }
+                CT_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void**>(&base), host, 0));
+                break;
             }
+            cap = std::max<int64_t>(1024, cap / 2 / 1024 * 1024);
         }
         counts = reinterpret_cast<unsigned long long*>(base);
         lo = reinterpret_cast<int32_t*>(base + 2 * sizeof(unsigned long long));
         row0 = lo + n;
         tup = reinterpret_cast<int32_t*>(base + head);
-        meta = ct->lo;
+        meta.assign(2 * sizeof(unsigned long long) / sizeof(int32_t), 0);  // the counts start at zero
+        meta.insert(meta.end(), ct->lo.begin(), ct->lo.end());
         meta.insert(meta.end(), ct->row0.begin(), ct->row0.end());
-        CT_CUDA(cudaMemsetAsync(counts, 0, 2 * sizeof(unsigned long long), ct->stream));
-        CT_CUDA(cudaMemcpyAsync(lo, meta.data(), meta.size() * sizeof(int32_t), cudaMemcpyHostToDevice, ct->stream));
+        return put(ct, base, meta.data(), meta.size() * sizeof(int32_t));
+    }
+    int put(const ct_table* ct, void* dst, const void* src, size_t n) {
+        if (!host) {
+            CT_CUDA(cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, ct->stream));
+            return CT_OK;
+        }
+        CT_CUDA(cudaStreamSynchronize(ct->stream));  // the kernels before have read what is overwritten
+        std::memcpy(host + (static_cast<char*>(dst) - base), src, n);
+        return CT_OK;
+    }
+    // The counts of launch_check_tuples (waits for them).
+    int counted(const ct_table* ct, unsigned long long (&c)[2]) {
+        if (!host) CT_CUDA(cudaMemcpyAsync(c, counts, sizeof(c), cudaMemcpyDeviceToHost, ct->stream));
+        CT_CUDA(cudaStreamSynchronize(ct->stream));
+        if (host) std::memcpy(c, host, sizeof(c));
         return CT_OK;
     }
     // The chunk of `tuples` that starts at tuple j0 (nothing to do if it is there).
     int load(const ct_table* ct, const int32_t* tuples, int64_t t, int64_t j0) {
         if (held == tuples && heldAt == j0) return CT_OK;
         const int64_t m = std::min(cap, t - j0);
-        CT_CUDA(cudaMemcpyAsync(tup, tuples + j0 * ct->arity, (size_t)m * ct->arity * sizeof(int32_t),
-                                cudaMemcpyHostToDevice, ct->stream));
+        const int st = put(ct, tup, tuples + j0 * ct->arity, (size_t)m * ct->arity * sizeof(int32_t));
+        if (st != CT_OK) return st;
         held = tuples;
         heldAt = j0;
         return CT_OK;
@@ -489,8 +555,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
                                         ct->stream));
         }
         unsigned long long c[2] = {0, 0};
-        CT_CUDA(cudaMemcpyAsync(c, stage.counts, sizeof(c), cudaMemcpyDeviceToHost, ct->stream));
-        CT_CUDA(cudaStreamSynchronize(ct->stream));
+        if ((st = stage.counted(ct, c)) != CT_OK) return st;
         all = c[0] == 0;
         nShort = (int64_t)c[1];
     }
@@ -605,7 +670,13 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     bufs.want(&varNW, (size_t)n);
     bufs.want(&varLD, (size_t)n);
     bufs.want(&ct->d_domScratch, (size_t)DW);
-    if ((st = bufs.take()) != CT_OK) return st;
+    st = bufs.take();
+    if (st == CT_ERR_OOM && stage.base && !bufs.injected) {
+        // the stage may be what is in the way: it comes back with what is left
+        stage.close();
+        st = bufs.take();
+    }
+    if (st != CT_OK) return st;
     if (nShort == 0) supDel = sup;
     ct->statusInts = (size_t)kStatusHdr + ct->nChW + DW;
     d.sup = sup;
@@ -715,6 +786,7 @@ int build(ct_table* ct, const int32_t* dom_lo, const int32_t* dom_size, const in
     c.trail_cap = 0;
     CT_CUDA(cudaMemcpyAsync(d.ctrl, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, ct->stream));
     if ((st = sync(ct)) != CT_OK) return st;
+    stage.close();
     if ((st = ensure_levels(ct, 8)) != CT_OK) return st;
     if (ct->profile) {
         if ((st = create_events(ct)) != CT_OK) return st;
@@ -1236,6 +1308,12 @@ extern "C" int ct_debug_guard_buffers(int on) {
 extern "C" int ct_debug_fail_alloc(int n) {
     std::lock_guard<std::mutex> lk(g_bufMu);
     g_failAfter = n < 0 ? -1 : n;
+    return CT_OK;
+}
+
+extern "C" int ct_debug_limit_bytes(int64_t bytes) {
+    std::lock_guard<std::mutex> lk(g_bufMu);
+    g_limitBytes = bytes < 0 ? -1 : bytes;
     return CT_OK;
 }
 

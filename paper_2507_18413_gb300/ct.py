@@ -128,6 +128,7 @@ _SIGS = {
     "ct_debug_guard_buffers": (ctypes.c_int, [ctypes.c_int]),
     "ct_debug_check_guards": (ctypes.c_int, [_P, ctypes.c_int, _I64P]),
     "ct_debug_fail_alloc": (ctypes.c_int, [ctypes.c_int]),
+    "ct_debug_limit_bytes": (ctypes.c_int, [ctypes.c_int64]),
     "ct_debug_device_bytes": (ctypes.c_int, [_I64P]),
     "ct_shard_bounds": (ctypes.c_int, [ctypes.c_int64, ctypes.c_int, _I64P]),
     "ct_sharded_create": (ctypes.c_int, [ctypes.c_int, _I32P, _I32P, _I32P, ctypes.c_int64, ctypes.c_int,
@@ -398,6 +399,11 @@ def ct_debug_check_guards(h, poke=0):
 def ct_debug_fail_alloc(n):
     """Test hook: the table-buffer allocation after the next n fails (n < 0: disarm)."""
     return load().ct_debug_fail_alloc(int(n))
+
+
+def ct_debug_limit_bytes(nbytes):
+    """Test hook: a device of nbytes for table buffers and construction scratch (< 0: no limit)."""
+    return load().ct_debug_limit_bytes(int(nbytes))
 
 
 def ct_debug_device_bytes():
