@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThreads) ct_small_kernel(const __grid_constan
         H[kSlotT2] = (int32_t)((update ? t2 : t1) - t0);
         H[kSlotT3] = (int32_t)(t3 - t0);
         H[kSlotT4] = (int32_t)(gtimer() - t0);
-        H[kSlotScan] = 0;
+        H[kSlotScan] = T.negative ? (int)sm.cnt[kCntHard] : 0;
         H[kSlotEarly] = 0;
         if (sm.trail) T.ctrl->trail_top = P.trailTop + sm.trail;
         st_release_sys(&H[kSlotStatus], st);

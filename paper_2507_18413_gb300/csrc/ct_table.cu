@@ -815,9 +815,10 @@ void fill_stats(ct_table* ct) {
     // Algorithmic bytes (what CT itself must move, 4-byte words): updateTable
     // reads k rows and currTable and writes currTable over the N live words;
     // filterDomains reads one word per residue hit, the windows it probes and
-    // the whole live table for every value scanned in full.
+    // the whole live table for every value scanned (a negative table's: counted)
+    // in full; a value that its windows decide costs no more than they do.
     s.update_bytes = s.rows_ored > 0 ? 4LL * s.live_words_in * (s.rows_ored + 2) : 0;
-    s.filter_bytes = 4LL * s.residue_hits + 4LL * 128 * s.windows + 16LL * s.hard * s.live_chunks_out;
+    s.filter_bytes = 4LL * s.residue_hits + 4LL * 128 * s.windows + 16LL * h[kSlotScan] * s.live_chunks_out;
     s.phase_ns[0] = h[kSlotT1];
     s.phase_ns[1] = h[kSlotT2];
     s.phase_ns[2] = h[kSlotT3];
