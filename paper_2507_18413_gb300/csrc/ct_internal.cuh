@@ -415,9 +415,9 @@ struct DeviceArena {
 // Arena bytes one clone of src takes (dynamic buffers, 8 levels and a trail of
 // 2 * W4 + 64 entries, each piece rounded up to 256 bytes).
 size_t ct_table_clone_bytes(const ct_table* src);
-// A clone of src (see ct_table.cu); its dynamic buffers come from `arena` when
-// given (else from cudaMalloc), its Ctrl is `ctrl` when given.
-ct_table* ct_table_clone(const ct_table* src, cudaStream_t stream, DeviceArena* arena, ctk::Ctrl* ctrl, int* status);
+// A clone of src (see ct_table.cu): its dynamic buffers come from `arena`, its
+// control block is `ctrl`.
+ct_table* ct_table_clone(const ct_table* src, cudaStream_t stream, DeviceArena& arena, ctk::Ctrl* ctrl, int* status);
 void ct_table_free(ct_table* ct);
 int ct_table_depth(const ct_table* ct);
 void ct_table_adopt_state(ct_table* dst, const ct_table* src);

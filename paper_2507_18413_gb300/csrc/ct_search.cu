@@ -203,7 +203,7 @@ int build_batch(ct_model* m, int B, ct_batch** out) {
     for (int s = 0; s < B; ++s) {
         for (int k = 0; k < T; ++k) {
             const int j = s * T + k;
-            ct_table* c = ct_table_clone(m->tables[k], m->stream, &b->arena, dCtrls + j, &st);
+            ct_table* c = ct_table_clone(m->tables[k], m->stream, b->arena, dCtrls + j, &st);
             if (!c) return st;
             b->tabs.push_back(c);
             hc[j] = Ctrl{};

@@ -1066,10 +1066,10 @@ size_t ct_table_clone_bytes(const ct_table* src) {
 // A table that shares `src`'s static buffers (supports rows and the layout
 // tables, which stay owned by src) with dynamic buffers of its own (currTable,
 // index, lastDom, residues, trail, levels), filled by launch_clone_state. Used
-// for the independent search nodes of a batched search. With an arena the
-// dynamic buffers, 8 levels and a first trail come out of it in one piece;
-// a trail or level stack that outgrows them moves to its own allocation.
-ct_table* ct_table_clone(const ct_table* src, cudaStream_t stream, DeviceArena* arena, Ctrl* ctrl, int* status) {
+// for the independent search nodes of a batched search. The dynamic buffers, 8
+// levels and a first trail come out of the arena in one piece; a trail or level
+// stack that outgrows them moves to its own allocation.
+ct_table* ct_table_clone(const ct_table* src, cudaStream_t stream, DeviceArena& arena, Ctrl* ctrl, int* status) {
     *status = CT_ERR_ARG;
     if (!src || src->empty) return nullptr;
     ct_table* ct = new (std::nothrow) ct_table();
@@ -1106,79 +1106,38 @@ ct_table* ct_table_clone(const ct_table* src, cudaStream_t stream, DeviceArena* 
     d.levelSeg = nullptr;
     d.levelDom = nullptr;
     d.statusBlk = src->dev.statusBlk;  // never written by the batched path; kept valid
-    if (arena) {
-        const std::vector<size_t> pc = clone_pieces(src);
-        void* p[16];
-        for (int i = 0; i < 16; ++i) {
-            p[i] = arena->take(pc[i]);
-            if (!p[i]) {
-                free_table(ct);
-                ct_set_error("clone arena exhausted");
-                *status = CT_ERR_OOM;
-                return nullptr;
-            }
+    const std::vector<size_t> pc = clone_pieces(src);
+    void* p[16];
+    for (int i = 0; i < 16; ++i) {
+        p[i] = arena.take(pc[i]);
+        if (!p[i]) {
+            free_table(ct);
+            ct_set_error("clone arena exhausted");
+            *status = CT_ERR_OOM;
+            return nullptr;
         }
-        d.curr = static_cast<uint4*>(p[0]);
-        d.segMask = static_cast<uint32_t*>(p[1]);
-        d.lastpos = static_cast<int32_t*>(p[2]);
-        d.residue = static_cast<int32_t*>(p[3]);
-        d.lastDom = static_cast<uint32_t*>(p[4]);
-        d.codes = static_cast<int32_t*>(p[5]);
-        d.planK = static_cast<int32_t*>(p[6]);
-        d.planRowOff = static_cast<int32_t*>(p[7]);
-        d.varSup = static_cast<int32_t*>(p[8]);
-        d.other = static_cast<unsigned long long*>(p[9]);
-        d.hardRow = static_cast<int32_t*>(p[10]);
-        d.foundChunk = static_cast<int32_t*>(p[11]);
-        d.levelSeg = static_cast<uint32_t*>(p[12]);
-        d.levelDom = static_cast<uint32_t*>(p[13]);
-        d.trailKey = static_cast<int2*>(p[14]);
-        d.trailOld = static_cast<uint4*>(p[15]);
-        ct->levelCap = kCloneLevels;
-        ct->levelsInArena = true;
-        ct->trailCap = (int)clone_trail_entries(src);
-        ct->trailInArena = true;
-        if (ctrl) {
-            d.ctrl = ctrl;
-        } else {
-            TableBufs bufs{ct, {}};
-            bufs.want(&d.ctrl, 1);
-            const int st = bufs.take();
-            if (st != CT_OK) {
-                free_table(ct);
-                *status = st;
-                return nullptr;
-            }
-        }
-        *status = CT_OK;
-        return ct;
     }
-    const size_t padChunks = (size_t)ct->nseg * 32;
-    TableBufs bufs{ct, {}};
-    bufs.want(&d.curr, padChunks);
-    bufs.want(&d.segMask, (size_t)ct->nseg);
-    bufs.want(&d.lastpos, padChunks);
-    bufs.want(&d.residue, (size_t)ct->R);
-    bufs.want(&d.lastDom, (size_t)ct->DW);
-    bufs.want(&d.codes, (size_t)ct->R);
-    bufs.want(&d.planK, (size_t)ct->arity);
-    bufs.want(&d.planRowOff, (size_t)ct->arity);
-    bufs.want(&d.varSup, (size_t)ct->arity);
-    bufs.want(&d.hardRow, (size_t)ct->R);
-    bufs.want(&d.foundChunk, (size_t)ct->R);
-    if (ctrl) d.ctrl = ctrl;
-    else bufs.want(&d.ctrl, 1);
-    int st = bufs.take();
-    if (st != CT_OK) {
-        free_table(ct);
-        *status = st;
-        return nullptr;
-    }
-    if ((st = ensure_levels(ct, kCloneLevels)) != CT_OK) {
-        free_table(ct);
-        *status = st;
-        return nullptr;
-    }
+    d.curr = static_cast<uint4*>(p[0]);
+    d.segMask = static_cast<uint32_t*>(p[1]);
+    d.lastpos = static_cast<int32_t*>(p[2]);
+    d.residue = static_cast<int32_t*>(p[3]);
+    d.lastDom = static_cast<uint32_t*>(p[4]);
+    d.codes = static_cast<int32_t*>(p[5]);
+    d.planK = static_cast<int32_t*>(p[6]);
+    d.planRowOff = static_cast<int32_t*>(p[7]);
+    d.varSup = static_cast<int32_t*>(p[8]);
+    d.other = static_cast<unsigned long long*>(p[9]);
+    d.hardRow = static_cast<int32_t*>(p[10]);
+    d.foundChunk = static_cast<int32_t*>(p[11]);
+    d.levelSeg = static_cast<uint32_t*>(p[12]);
+    d.levelDom = static_cast<uint32_t*>(p[13]);
+    d.trailKey = static_cast<int2*>(p[14]);
+    d.trailOld = static_cast<uint4*>(p[15]);
+    ct->levelCap = kCloneLevels;
+    ct->levelsInArena = true;
+    ct->trailCap = (int)clone_trail_entries(src);
+    ct->trailInArena = true;
+    d.ctrl = ctrl;
     *status = CT_OK;
     return ct;
 }
