@@ -287,8 +287,22 @@ __global__ void ct_features_kernel(const FeatArgs A, int perNode) {
 // variables and 40 tables of up to 157 chunks, this one 10. For one network the
 // last CTA also writes the features where the host reads them, and a word that
 // the host waits for (a copy and a stream synchronisation took 6 us more of
-// ct_model_features' 28). Tables of more than kFeatChunks chunks keep them (their counts spread over the grid).
-constexpr int kFeatChunks = 256, kFeatValues = 1024, kFeatVars = 2048, kFeatThreads = 256;
+// ct_model_features' 28). The line to the two kernels, which spread the counts
+// and the sums over the grid, lies where those catch up (ct_model_features in us,
+// this kernel and those):
+//   an entry's values x chunks, all one CTA's: 128 x 256 57 and 60 us (3 tables)
+//   or 61 and 74 (40 tables), 512 x 64 57 and 62, 60 and 87; beyond, 192 x 256 68
+//   and 59, 125 and 94, 1,024 x 64 89 and 62;
+//   a node's variables, one per thread of its last CTA: 256 in 8 tables each 52
+//   and 75, in 24 each 95 and 105; beyond, 384 73 and 76, 140 and 118, 512 79 and
+//   78, 157 and 124, 2,048 221 and 117, 636 and 315.
+// Batches of nodes (the batched search with a policy, ms, this kernel and those):
+// many entries of short tables leave it bound by its CTAs, 600 of 16 chunks at 200
+// variables 60.6 and 59.9 on 8 nodes, 30.6 and 26.4 on 64; 300 of 94 chunks at
+// 100 variables 7.2 and 7.3 on 64; 192 of 40 chunks at 64 variables 12.2 and 12.8.
+constexpr int kFeatNodeVars = 64, kFeatEntries = 16384;
+constexpr int kFeatThreads = 256, kFeatVars = kFeatThreads;
+constexpr int kFeatChunks = 256, kFeatValues = 1024, kFeatTests = 32768;  // of a table, a variable, an entry
 
 __global__ void __launch_bounds__(kFeatThreads) ct_features_small_kernel(const FeatArgs A) {
     __shared__ uint4 cur[kFeatChunks];
@@ -962,12 +976,18 @@ int ct_feat_view_build(FeatView* f, int nodes, const std::vector<std::vector<int
     }
     f->pairs = nodes > 0 ? (int)adj.size() / nodes : 0;
     f->small = f->pairs > 0 && V <= kFeatVars;
-    for (int k = 0; k < T; ++k) f->small = f->small && tableSeg[k] * 32 <= kFeatChunks;
-    for (int v = 0; v < V; ++v) f->small = f->small && varNW[v] * 32 <= kFeatValues;
+    for (int k = 0; k < T; ++k) {
+        const int chunks = tableSeg[k] * 32;
+        for (int v : scopes[k])
+            f->small = f->small && chunks <= kFeatChunks && varNW[v] <= kFeatValues / 32 &&
+                       varNW[v] * 32 * chunks <= kFeatTests;
+    }
     std::vector<int32_t> pairVar(adj.size());
     for (int v = 0; v < nv; ++v) std::fill(pairVar.begin() + adjBase[v], pairVar.begin() + adjBase[v + 1], v);
     f->degmax = degmax;
     f->totalUnits = unitBase[nt];
+    const int64_t entries = (int64_t)nodes * f->pairs;
+    f->small = f->small && (nodes == 1 || V <= kFeatNodeVars || entries <= kFeatEntries || f->totalUnits >= 3 * entries);
     f->totalRows = rowBase[nt];
     int st;
     if ((st = f_alloc(f, &f->rowBase, nt + 1)) != CT_OK || (st = f_alloc(f, &f->unitBase, nt + 1)) != CT_OK ||
