@@ -322,6 +322,15 @@ cudaError_t launch_model(const ModelDev& M, int grid, cudaStream_t s);
 // kNetMaxTables tables, each with a one-warp plan and at most kNetMaxRows rows,
 // and net_smem_bytes(M) <= kNetSmemMax (two CTAs per SM).
 constexpr int kNetMaxTables = 512, kNetMaxRows = 1024, kNetTabSmem = 64, kNetSmemMax = 112 << 10;
+// A launch whose first round has more than this many tables x (table, segment)
+// units runs the general kernel all the same: it plans a table once where the
+// small-network kernel plans it again for each unit, and has twice its warps.
+// Per fixpoint in us, this kernel and the general one: 100 tables, 9,800 units
+// 117 and 120, 16,900 units of 69 tables 122 and 112; 200 tables, 5,000 units 95
+// and 98, 9,800 127 and 122, 19,600 193 and 176; 400 tables, 2,662 units of 106 67
+// and 77, 10,000 149 and 136; 512 tables, 25,088 265 and 220; few tables never
+// get there (50 tables, 19,804 units of 40: 135 and 156).
+constexpr int64_t kNetWork = 1 << 20;
 int net_smem_bytes(const ModelDev& M);
 int max_coresident_net_blocks(const ModelDev& M);
 // block: the launch's host block [count, 3 pad | calls | domains | work list]; up

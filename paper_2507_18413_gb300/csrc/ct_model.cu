@@ -161,8 +161,11 @@ int batch_setup(ct_model* m) {
         if ((st = m_alloc(m, &M.phaseNs, kModelPhases)) != CT_OK) return st;
         CT_CUDA(cudaMemsetAsync(M.phaseNs, 0, kModelPhases * sizeof(uint64_t), m->stream));
     }
-    const int rowsPer = m->net ? kWarps : 2 * kWarps;  // rows per CTA: the small-network kernel's barriers are few
-    int64_t want = std::max<int64_t>({(int64_t)n, (segs + kWarps - 1) / kWarps, (rows + rowsPer - 1) / rowsPer, 1});
+    // rows per CTA: the small-network kernel's barriers are few
+    auto ctas = [&](int rowsPer) {
+        return std::max<int64_t>({(int64_t)n, (segs + kWarps - 1) / kWarps, (rows + rowsPer - 1) / rowsPer, 1});
+    };
+    int64_t want = ctas(m->net ? kWarps : 2 * kWarps);
     if (m->net) {
         // one CTA per SM: two share no more of the reads' latency and make every
         // barrier wider. Per fixpoint, one against two: 512 tables of 3 rounds 98
@@ -172,6 +175,8 @@ int batch_setup(ct_model* m) {
         CT_CUDA(cudaGetDevice(&dev));
         CT_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         want = std::min<int64_t>(want, sms);
+        const int64_t general = m->opt.grid_blocks > 0 ? m->opt.grid_blocks : ctas(2 * kWarps);
+        m->generalGrid = (int)std::min<int64_t>(general, max_coresident_model_blocks(n));
     }
     if (m->opt.grid_blocks > 0) want = m->opt.grid_blocks;
     m->grid = (int)std::min<int64_t>(want, maxCo);
@@ -243,15 +248,24 @@ int batch_propagate(ct_model* m) {
     int st;
     if (!m->batchReady) {
         if ((st = batch_setup(m)) != CT_OK) return st;
-        if (m->opt.autotune && m->opt.grid_blocks <= 0 && (st = tune_grid(m)) != CT_OK) return st;
+        if (m->opt.autotune && m->opt.grid_blocks <= 0) {
+            m->tuning = true;
+            st = tune_grid(m);
+            m->tuning = false;
+            if (st != CT_OK) return st;
+        }
     }
     const int n = (int)m->tables.size();
     int nwork = 0;
+    int64_t units = 0;
     for (int t = 0; t < n; ++t) {
         if ((st = ct_table_batch_prepare(m->tables[t], &m->h_calls[t])) != CT_OK) return st;
-        if (m->dirty[t]) m->h_list[nwork++] = t;
+        if (!m->dirty[t]) continue;
+        m->h_list[nwork++] = t;
+        units += ct_table_dev(m->tables[t]).nseg;
     }
     if (nwork == 0) return CT_OK;
+    const bool net = m->net && (m->tuning || m->generalGrid < 1 || units * nwork <= kNetWork);
     // device copies of the tables whose buffers moved (trail or level growth)
     for (int t = 0; t < n; ++t) {
         const int v = ct_table_version(m->tables[t]);
@@ -266,7 +280,7 @@ int batch_propagate(ct_model* m) {
     m->h_blk[0] = nwork;
     std::memcpy(m->h_blk + 4 + 4 * (size_t)n, m->h_dom.data(), (size_t)m->DWg * sizeof(uint32_t));
     const size_t blkWords = 4 + 4 * (size_t)n + (size_t)m->DWg + (size_t)nwork;
-    const bool inl = m->net && blkWords <= (size_t)kNetCallWords;  // ... or in the launch's parameters
+    const bool inl = net && blkWords <= (size_t)kNetCallWords;  // ... or in the launch's parameters
     if (!inl)
         CT_CUDA(cudaMemcpyAsync(m->d_blk, m->h_blk, blkWords * sizeof(int32_t), cudaMemcpyHostToDevice, m->stream));
     m->domStale = false;
@@ -283,8 +297,10 @@ int batch_propagate(ct_model* m) {
         m->armPolls = 0;
     }
     const auto t0 = std::chrono::steady_clock::now();
-    CT_CUDA(m->net ? launch_net(M, inl ? m->h_blk : nullptr, (int)blkWords, m->grid, m->stream)
-                   : launch_model(M, m->grid, m->stream));
+    if (m->net && !net)  // the small-network kernel clears the variables' marks when it starts, this one when it ends
+        CT_CUDA(cudaMemsetAsync(M.prunedBy, 0xff, 2 * (size_t)m->nvars * sizeof(int32_t), m->stream));
+    CT_CUDA(net ? launch_net(M, inl ? m->h_blk : nullptr, (int)blkWords, m->grid, m->stream)
+                : launch_model(M, m->net ? m->generalGrid : m->grid, m->stream));
     bool seen = false;
     for (uint64_t it = 0;; ++it) {
         if (H[0] != kNoChunk) {
@@ -321,11 +337,11 @@ int batch_propagate(ct_model* m) {
     // snapshotted then; the others' results are not written)
     const int32_t* after = const_cast<const int32_t*>(H) + kModelHdr + 2 * n + m->DWg + 1;
     for (int t = 0; t < n; ++t) {
-        if (m->net && !((after[t >> 5] >> (t & 31)) & 1)) {
+        if (net && !((after[t >> 5] >> (t & 31)) & 1)) {
             m->tables[t]->failed = false;
             continue;
         }
-        ct_table_batch_done(m->tables[t], H[kModelHdr + 2 * t], H[kModelHdr + 2 * t + 1], m->net || after[t] != 0);
+        ct_table_batch_done(m->tables[t], H[kModelHdr + 2 * t], H[kModelHdr + 2 * t + 1], net || after[t] != 0);
     }
     if (status == CT_OK && H[kModelHdr + 2 * n + m->DWg] == CT_INFEASIBLE) {
         m->failed = true;

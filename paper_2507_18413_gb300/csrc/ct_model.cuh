@@ -49,7 +49,9 @@ struct ct_model {
     std::vector<int> tabVersion;
     std::vector<void*> allocs;
     int grid = 1;
-    bool net = false;  // the small-network kernel runs the fixpoints
+    bool net = false;  // the small-network kernel runs the fixpoints ...
+    int generalGrid = 1;    // ... but for the launches beyond it (kNetWork), which take so many CTAs
+    bool tuning = false;    // the grid of the small-network kernel is being tuned: no other launch
     bool broken = false;    // a device-side wait ran out: the model is unusable
     uint32_t armPolls = 0;  // test hook: the next launch's barrier waits run out after this many polls
     ct_batch* bsearch = nullptr;  // built by the first batched search, kept for the next ones
