@@ -65,8 +65,8 @@ typedef struct ct_options {
     int32_t host_fixpoint;    /* models: 1 = run the fixpoint queue on the host, one launch per table
                                  propagation (default: the whole fixpoint in one launch) */
     int32_t autotune;         /* 1 = pick the launch shape at creation by timing trial propagations:
-                                 for a table, batches of 16 or 8 row loads in flight (2 or 3 CTAs
-                                 per SM) and the CTA count (segments per CTA); for a model, the CTA
+                                 for a table, batches of 16 or 8 row loads in flight (1 or 2, or 3
+                                 CTAs per SM) and the CTA count (segments per CTA); for a model, the CTA
                                  count of the fixpoint launch (tables and segments per CTA). The
                                  trials run between a save and a restore, so the state is unchanged.
                                  Ignored when grid_blocks is set. */
@@ -93,9 +93,10 @@ typedef struct ct_options {
                                  chunks are live filters beside the update, each probed chunk
                                  recomputed from its stored value and the call's rows (Algorithm 2 at
                                  one chunk), and one grid barrier ends both; positive tables with
-                                 residues and a plan in shared memory, of more than 128 chunks (below,
-                                 one CTA propagates the table and its filter always follows the
-                                 update). Results are the same. */
+                                 residues and a plan in shared memory, but for those that one CTA
+                                 propagates (at most 128 chunks, 512 values and 16 variables of at
+                                 most 128 values), whose filter always follows the update. Results
+                                 are the same. */
 } ct_options;
 
 /* Static shape and live state of a table (ct_get_info). */
@@ -114,7 +115,9 @@ typedef struct ct_table_info {
     int32_t grid_blocks;   /* CTAs of the propagation launch */
     int32_t short_tuples;  /* retained tuples with at least one CT_STAR component */
     int64_t device_bytes;  /* device memory held by the table */
-    int32_t loads_in_flight; /* 16 (1 or 2 CTAs per SM) or 8 (3 CTAs per SM) row loads per lane */
+    int32_t loads_in_flight; /* row loads of a batch per lane: 16 (1 or 2 CTAs per SM, and tables that one
+                                CTA propagates) or 8 (3 CTAs per SM); at 1 CTA per SM, lists of more than
+                                32 rows that one warp walks go 32 at a time */
     int32_t autotuned;     /* 1 if the launch shape was chosen by trial propagations */
 } ct_table_info;
 
@@ -420,7 +423,7 @@ int ct_model_set_domains(ct_model* m, const uint32_t* words_host);
  * (the one-launch fixpoint fills all of them; the host queue only
  * propagations). Bytes are algorithmic, as for one table: updateTable
  * 4 * (non-zero words at entry) * (rows OR-ed + 2) per table propagation;
- * filterDomains 16 per residue hit, 512 per window probed and 16 per live
+ * filterDomains 4 per residue hit, 512 per window probed and 16 per live
  * chunk of every full scan. */
 typedef struct ct_model_stats {
     int64_t fixpoints;     /* launches of the fixpoint kernel */

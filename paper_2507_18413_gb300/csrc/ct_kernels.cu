@@ -836,7 +836,7 @@ int coresident() {
 }  // namespace
 
 // variant: bit 0 = local plan, bit 1 = wide (8 loads in flight, 3 CTAs per SM),
-// bit 2 (with bit 0 alone) = 16 loads at one CTA per SM: 255 registers, no spills
+// bit 2 (with bit 0 alone) = 16 loads at one CTA per SM: 231 registers, no spills
 int max_coresident_blocks(int variant) {
     int r = 0;
     switch (variant) {

@@ -13,8 +13,8 @@
 //   f3 = mean_c s * min_a p_c(a), f4 = mean_c max_a p_c(a),
 //   f5 = mean_c (-sum_a p_c(a) log2 p_c(a)) / log2(s),
 //   f6 = mean_c log2(1 + live_c) / 32, f7 = s / smax.
-// The counts are integers (one warp per (table, segment), lane per chunk);
-// the aggregation runs in double and is stored as float.
+// The counts are integers (a warp per (table, segment), lane per chunk, or on
+// small networks a CTA per variable and table); what is made of them is float.
 //
 // Network: h1 = relu(W1 x + b1), h2 = relu(W2 h1 + b2), out = W3 . h2 + b3,
 // float32, weights flat as W1[64][8], b1, W2[64][64], b2, W3[64], b3.
