@@ -257,15 +257,17 @@ int batch_propagate(ct_model* m) {
     }
     const int n = (int)m->tables.size();
     int nwork = 0;
-    int64_t units = 0;
+    int64_t cut = 0, units = 0;  // tables with rows to OR in the first round, and their segments
     for (int t = 0; t < n; ++t) {
         if ((st = ct_table_batch_prepare(m->tables[t], &m->h_calls[t])) != CT_OK) return st;
         if (!m->dirty[t]) continue;
         m->h_list[nwork++] = t;
+        if (m->dirty[t] != kDirtyCut) continue;
+        cut += 1;
         units += ct_table_dev(m->tables[t]).nseg;
     }
     if (nwork == 0) return CT_OK;
-    const bool net = m->net && (m->tuning || m->generalGrid < 1 || units * nwork <= kNetWork);
+    const bool net = m->net && (m->tuning || m->generalGrid < 1 || cut * units <= kNetWork);
     // device copies of the tables whose buffers moved (trail or level growth)
     for (int t = 0; t < n; ++t) {
         const int v = ct_table_version(m->tables[t]);
@@ -366,9 +368,9 @@ int popcount_var(const ct_model* m, int v) {
 
 void mark_var(ct_model* m, int v, int except, std::deque<int>* q) {
     for (int T : m->varTables[v]) {
-        if (T == except || m->dirty[T]) continue;
-        m->dirty[T] = 1;
-        if (q) q->push_back(T);
+        if (T == except) continue;
+        if (!m->dirty[T] && q) q->push_back(T);
+        m->dirty[T] = kDirtyCut;
     }
 }
 
@@ -573,7 +575,7 @@ int add_table_impl(ct_model* m, const int32_t* scope, int arity, const int32_t* 
     m->scopes.push_back(sc);
     m->d_tabOff.push_back(d_off);
     m->tabOff.push_back(offs);
-    m->dirty.push_back(1);
+    m->dirty.push_back(kDirtyNew);
     for (int v : sc) m->varTables[v].push_back(T);
     if (st == CT_INFEASIBLE) m->staticInfeasible = true;
     return st;

@@ -8,6 +8,8 @@
 
 struct ct_batch;  // the slots of a batched search (ct_search.cu)
 
+constexpr char kDirtyNew = 1, kDirtyCut = 2;
+
 struct ct_model {
     int nvars = 0;
     std::vector<int32_t> lo, size, nw, off;
@@ -19,7 +21,7 @@ struct ct_model {
     std::vector<int32_t*> d_tabOff;
     std::vector<std::vector<int32_t>> tabOff;
     std::vector<std::vector<int>> varTables;
-    std::vector<char> dirty;
+    std::vector<char> dirty;  // 0, or why the table is to propagate: new, or a variable of it was cut
     struct Level {
         std::vector<uint32_t> dom;
         std::vector<char> dirty;

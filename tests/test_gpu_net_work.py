@@ -43,6 +43,7 @@ def test_both_kernels_on_one_model(ntables, t, general):
     a, b = _models(nv, ntables, d, t, sol, 3, [{"profile": 1}, {"host_fixpoint": 1}])
     words = nv * 4
     assert C.ct_model_propagate(a) == C.ct_model_propagate(b) == C.CT_OK
+    assert C.ct_model_get_stats(a)[1]["phase_seconds"][1] == 0  # (no table was cut yet)
     ran, rounds = [], 0
     level = 0
     for k in range(12):
