@@ -136,20 +136,8 @@ __device__ __forceinline__ void bar_init(GridBarrier& b, unsigned* count, unsign
     b.target = threadIdx.x == 0 ? ld_relaxed(base) : 0u;
 }
 
-// The two halves of a barrier, for thread 0: the arrival (true: the last one)
-// and the bounded wait (false: it ran out, CT_ERR_TIMEOUT is set). A CTA with
-// nothing left to do after a barrier need not wait for it.
-__device__ __forceinline__ bool bar_arrive(GridBarrier& b) {
-    unsigned arrived;
-    b.target += gridDim.x;
-    // Release this CTA's writes (ordered before by the CTA barrier) and, for
-    // the last arrival, acquire everybody else's.
-    asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(b.count) : "memory");
-    if (arrived != b.target - 1u) return false;
-    *b.base = b.target;  // read by the next launch only
-    return true;
-}
-
+// Bounded wait of thread 0 for the count to reach its target (false: it ran out,
+// CT_ERR_TIMEOUT is set).
 __device__ __forceinline__ bool bar_wait(const GridBarrier& b) {
     unsigned it = 0;
     while ((int)(ld_acquire(b.count) - b.target) < 0) {
@@ -164,9 +152,35 @@ __device__ __forceinline__ bool bar_wait(const GridBarrier& b) {
 
 __device__ int bar_sync(GridBarrier& b, int* s_flag) {
     __syncthreads();
-    if (threadIdx.x == 0) *s_flag = bar_arrive(b) ? 2 : bar_wait(b) ? 1 : 0;
+    if (threadIdx.x == 0) {
+        unsigned arrived;
+        b.target += gridDim.x;
+        // Release this CTA's writes (ordered before by the CTA barrier) and, for
+        // the last arrival, acquire everybody else's.
+        asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(arrived) : "l"(b.count) : "memory");
+        if (arrived == b.target - 1u) {
+            *b.base = b.target;  // read by the next launch only
+            *s_flag = 2;
+        } else {
+            *s_flag = bar_wait(b) ? 1 : 0;
+        }
+    }
     __syncthreads();
     return *s_flag;
+}
+
+// A one-sided barrier at the end of a launch: every CTA but one releases its
+// writes and leaves (thread 0, after a CTA barrier), the one waits for them
+// (thread 0; bounded).
+__device__ __forceinline__ void bar_signal(const GridBarrier& b) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.count) : "memory");
+}
+
+__device__ __forceinline__ bool bar_collect(GridBarrier& b) {
+    b.target += gridDim.x - 1u;
+    if (!bar_wait(b)) return false;
+    *b.base = b.target;
+    return true;
 }
 
 struct Smem {
